@@ -127,7 +127,8 @@ struct ngs_ctx {
     cudaStream_t copy_stream = nullptr;
     cudaEvent_t ev_copied = nullptr;
 
-    // navigation scratch (occupied-any map, goals, frontier queues), grown on demand
+    // navigation scratch (occupied-any map, goals, free-cell bits, and for
+    // maps beyond the search on bits frontier queues), grown on demand
     unsigned char *nav_tmp = nullptr;
     size_t nav_tmp_bytes = 0;
 
@@ -1626,7 +1627,9 @@ NGS_API ngs_status ngs_nav_fields(ngs_ctx *c, const uint8_t *d_occ, int32_t nx, 
     cudaSetDevice(c->device);
     const size_t a_bytes = ((size_t)plane + 255) & ~(size_t)255;
     const size_t g_bytes = ((size_t)n_goals * sizeof(int2) + 255) & ~(size_t)255;
-    const size_t need = a_bytes + g_bytes + (size_t)n_goals * 2 * plane * sizeof(uint32_t);
+    const size_t f_bytes = ((size_t)nav_row_words(nx) * ny * sizeof(uint32_t) + 255) & ~(size_t)255;
+    const size_t need =
+        a_bytes + g_bytes + f_bytes + nav_queue_words(nx, ny, n_goals) * sizeof(uint32_t);
     cudaStream_t st = (cudaStream_t)stream;
     if (need > c->nav_tmp_bytes) {
         CK(cudaStreamSynchronize(st));
@@ -1643,6 +1646,8 @@ NGS_API ngs_status ngs_nav_fields(ngs_ctx *c, const uint8_t *d_occ, int32_t nx, 
     CK(cudaMemcpyAsync(dg, hg.data(), (size_t)n_goals * sizeof(int2), cudaMemcpyHostToDevice, st));
     const int e = launch_nav_fields(d_occ, nx, ny, k_lo, k_hi, inflate, dg, n_goals, c->nav_tmp,
                                     reinterpret_cast<uint32_t *>(c->nav_tmp + a_bytes + g_bytes),
+                                    reinterpret_cast<uint32_t *>(c->nav_tmp + a_bytes + g_bytes +
+                                                                 f_bytes),
                                     d_blocked, d_dist, c->num_sms, st);
     if (e != 0) {
         std::fprintf(stderr, "ngs: nav fields: %s\n", cudaGetErrorString((cudaError_t)e));

@@ -1,0 +1,80 @@
+"""Kernel variants at the sizes where they can go wrong, against the oracle or a
+plain reference of the same step."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def R():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_2603_15186_gb300 import Renderer
+    r = Renderer(cut_capacity=1 << 22, record_capacity=1 << 22, pair_capacity=1 << 24)
+    yield r
+    r.close()
+
+
+# one cell, one row, one column; rows of one word, of whole words and with a
+# remainder; fewer rows than the CTAs' halos and rows that do not divide evenly; one,
+# two and four words per thread at their largest; the first map beyond, by its words
+# and by its row length; one of corridors off one corridor (levels up to 900, wide
+# frontiers)
+NAV_MAPS = [(1, 1), (33, 1), (1, 70), (32, 9), (64, 40), (31, 33), (97, 65), (61, 129), (528, 276),
+            (511, 384), (511, 385), (511, 896), (511, 1920), (511, 1928), (5247, 64), (6000, 64),
+            (700, 900)]
+
+
+@pytest.mark.parametrize("nx,ny", NAV_MAPS)
+def test_nav_fields_and_paths_of_all_map_sizes(R, nx, ny):
+    import oracle as O
+    rng = np.random.default_rng(nx * 7919 + ny)
+    occ = (rng.random((2, ny, nx)) < 0.14).astype(np.uint8)
+    if (nx, ny) == (700, 900):
+        occ[:] = 0
+        occ[:, :, ::3] = 1
+        occ[:, ny // 2] = 0
+    goals = [(nx // 2, ny // 2), (nx - 1, ny - 1), (0, 0), (nx, 0)]
+    for x, y in goals[:3]:
+        occ[:, y, x] = 0
+    blocked, dist = R.nav_fields(torch.from_numpy(occ).cuda(), goals, 0, 1, 0)
+    b_ref = O.nav_blocked(occ, 0, 1, 0)
+    assert np.array_equal(blocked.cpu().numpy(), b_ref)
+    got = dist.cpu().numpy().view(np.uint32)
+    refs = [O.nav_field(b_ref, g) for g in goals]
+    for k in range(len(goals)):
+        assert np.array_equal(got[k], refs[k]), k
+    starts = [(int(rng.integers(nx)), int(rng.integers(ny)), int(rng.integers(4))) for _ in range(40)]
+    for max_len in (1, 32, 1500):
+        paths, lens = (t.cpu().numpy() for t in R.nav_paths(dist, starts, max_len))
+        for a, (i, j, g) in enumerate(starts):
+            ref = O.nav_path(refs[g], (i, j), max_len)
+            assert lens[a] == len(ref) and np.array_equal(paths[a, :lens[a]], ref), (a, max_len)
+            assert not paths[a, lens[a]:].any()
+
+
+def test_nav_paths_of_other_fields(R):
+    """A field that no breadth-first search gave is followed by the same rule: the
+    first neighbour one less than the count so far, else stay and count on."""
+    rng = np.random.default_rng(5)
+    ny, nx, max_len = 150, 170, 400
+    # plateaus and gaps: steps towards the left, some cells off by a few
+    dist = (np.arange(nx)[None, :] + rng.integers(0, 3, (ny, nx)) * (rng.random((ny, nx)) < 0.2)).astype(np.uint32)
+    dist[:, 60] += 2
+    starts = np.stack([rng.integers(0, nx, 60), rng.integers(0, ny, 60), np.zeros(60, int)], 1)
+    got = R.nav_paths(torch.from_numpy(dist.view(np.int32))[None].cuda(), starts, max_len)
+    paths, lens = (t.cpu().numpy() for t in got)
+    for a, (i, j, _) in enumerate(starts):
+        d, cells = int(dist[j, i]), []
+        while True:
+            cells.append((i, j))
+            if d == 0 or len(cells) == max_len:
+                break
+            for x, y in ((i + 1, j), (i - 1, j), (i, j + 1), (i, j - 1)):
+                if 0 <= x < nx and 0 <= y < ny and dist[y, x] == d - 1:
+                    i, j = x, y
+                    break
+            d -= 1
+        assert lens[a] == len(cells) and np.array_equal(paths[a, :len(cells)], cells), a
