@@ -13,11 +13,19 @@
 // Sigma_zz, (alpha, beta) = -(Sigma_xz, Sigma_yz) / Sigma_zz, C = (R S^-2 R^T)
 // restricted to xy, so no difference of large terms appears.
 //
-// One thread per node (interior nodes return at once): planes within the
-// slice's vertical support, cells of each slice's support box (the ellipse
-// where a >= 1/255, widened by a relative 1e-4 and 1e-6 m), each value folded
-// into the cell with atomicMax on its bits (non-negative floats order like
-// their bit patterns, so the result does not depend on the order).
+// One thread per node takes the planes within the slice's vertical support and the
+// box of cells of each slice's support (the ellipse where a >= 1/255, widened by a
+// relative 1e-4 and 1e-6 m). Boxes differ (a few cells to hundreds: log-normal
+// scales, interior nodes none), so a warp puts its leaves' boxes on a plane end to end
+// and its lanes take the cells one each; a value is folded into its cell with
+// atomicMax on its bits (non-negative floats order like their bit patterns, so the
+// result does not depend on the order). 4M leaves, 13 planes, 528 x 276 cells of 5 cm
+// (60 M cells in boxes): 1740 us with a loop per thread over its own boxes (6.6 of 32
+// lanes active) and a count per thread on one address, 366 us so; its atomics do not
+// bound it (a look at the cell before each, to leave out those that change nothing:
+// 538 us).
+#include <climits>
+
 #include "ngs_internal.cuh"
 
 namespace ngs {
@@ -43,79 +51,177 @@ __device__ __forceinline__ void load_sop<__nv_bfloat16>(const void *p, int64_t i
     v[2] = __uint_as_float(t.y << 16); v[3] = __uint_as_float(t.y & 0xffff0000u);
 }
 
+// One leaf's slice by one plane: what its cells' values need, and its support box.
+struct __align__(16) SliceItem {
+    float ez, cxx, cxy, cyy;
+    float o, mx, my, inv_w;
+    int32_t i0, j0, w;
+    uint32_t start;       // its first cell in the warp's list of cells
+};
+
+constexpr int kSliceThreads = 256;
+// a slice of more cells is spread over the warp by itself
+constexpr uint32_t kSliceBig = 1u << 16;
+
 template <typename A>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kSliceThreads)
 k_slice(SceneDev sc, SliceGrid g, uint32_t *__restrict__ value_bits,
         unsigned long long *work) {
-    const int64_t node = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (node >= sc.n) return;
-    if (__float_as_int(sc.box_hi[node].w) != 0) return;            // leaves only
-    const float4 p = sc.pos4[node];
-    if (__float_as_uint(p.w) & kNodeCullOpacity) return;           // 255 o < 1
-    float so[4];
-    load_sop<A>(sc.sop, node, so);
-    const float o = so[3];
-    const float K = 2.0f * logf(255.0f * o);                       // a >= 1/255 <=> q <= K
-    const float4 q4 = sc.quat[node];
-    const float qn = rsqrtf(q4.x * q4.x + q4.y * q4.y + q4.z * q4.z + q4.w * q4.w);
-    const float w = q4.x * qn, x = q4.y * qn, y = q4.z * qn, z = q4.w * qn;
-    const float R[9] = {1.f - 2.f * (y * y + z * z), 2.f * (x * y - w * z), 2.f * (x * z + w * y),
-                        2.f * (x * y + w * z), 1.f - 2.f * (x * x + z * z), 2.f * (y * z - w * x),
-                        2.f * (x * z - w * y), 2.f * (y * z + w * x), 1.f - 2.f * (x * x + y * y)};
-    float s2[3], is2[3];
+    __shared__ SliceItem s_item[kSliceThreads / 32][32];
+    __shared__ unsigned long long s_evals[kSliceThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t node = (int64_t)blockIdx.x * kSliceThreads + threadIdx.x;
+    int k0 = 0, k1 = -1;   // the planes that cut this thread's leaf
+    float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
+    float o = 0.f, K = 0.f, lambda = 0.f, alpha = 0.f, beta = 0.f;
+    float cxx = 0.f, cxy = 0.f, cyy = 0.f, ixx = 0.f, iyy = 0.f;
+    // leaves only, and only those that reach 255 o >= 1
+    if (node < sc.n && __float_as_int(sc.box_hi[node].w) == 0) p = sc.pos4[node];
+    else p.w = __uint_as_float(kNodeCullOpacity);
+    if (!(__float_as_uint(p.w) & kNodeCullOpacity)) {
+        float so[4];
+        load_sop<A>(sc.sop, node, so);
+        o = so[3];
+        K = 2.0f * logf(255.0f * o);                               // a >= 1/255 <=> q <= K
+        const float4 q4 = sc.quat[node];
+        const float qn = rsqrtf(q4.x * q4.x + q4.y * q4.y + q4.z * q4.z + q4.w * q4.w);
+        const float w = q4.x * qn, x = q4.y * qn, y = q4.z * qn, z = q4.w * qn;
+        const float R[9] = {1.f - 2.f * (y * y + z * z), 2.f * (x * y - w * z), 2.f * (x * z + w * y),
+                            2.f * (x * y + w * z), 1.f - 2.f * (x * x + z * z), 2.f * (y * z - w * x),
+                            2.f * (x * z - w * y), 2.f * (y * z + w * x), 1.f - 2.f * (x * x + y * y)};
+        float s2[3], is2[3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        s2[k] = expf(2.0f * so[k]);
-        is2[k] = expf(-2.0f * so[k]);
-    }
-    // Sigma's z row and Sigma^-1's xy block
-    float sxz = 0.f, syz = 0.f, szz = 0.f, cxx = 0.f, cxy = 0.f, cyy = 0.f;
+        for (int k = 0; k < 3; ++k) {
+            s2[k] = expf(2.0f * so[k]);
+            is2[k] = expf(-2.0f * so[k]);
+        }
+        // Sigma's z row and Sigma^-1's xy block
+        float sxz = 0.f, syz = 0.f, szz = 0.f;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        sxz += R[k] * s2[k] * R[6 + k];
-        syz += R[3 + k] * s2[k] * R[6 + k];
-        szz += R[6 + k] * s2[k] * R[6 + k];
-        cxx += R[k] * is2[k] * R[k];
-        cxy += R[k] * is2[k] * R[3 + k];
-        cyy += R[3 + k] * is2[k] * R[3 + k];
-    }
-    const float lambda = 1.0f / szz;
-    const float alpha = -sxz / szz, beta = -syz / szz;
-    const float det = cxx * cyy - cxy * cxy;
-    if (!(det > 0.0f) || !(K >= 0.0f)) return;
-    // planes within the vertical support lambda z'^2 <= K
-    const float rz = sqrtf(K / lambda) * 1.0001f + 1e-6f;
-    int k0 = (int)ceilf((p.z - rz - g.z0) / g.dz), k1 = (int)floorf((p.z + rz - g.z0) / g.dz);
-    k0 = max(k0, 0);
-    k1 = min(k1, g.nz - 1);
-    const float ixx = cyy / det, iyy = cxx / det;                  // C^-1 diagonal
-    const int64_t plane = (int64_t)g.nx * g.ny;
-    unsigned long long evals = 0;
-    for (int k = k0; k <= k1; ++k) {
-        const float zp = (g.z0 + (float)k * g.dz) - p.z;
-        const float ez = lambda * zp * zp;
-        const float rem = K - ez;
-        if (rem < 0.0f) continue;
-        const float hx = sqrtf(rem * ixx) * 1.0001f + 1e-6f, hy = sqrtf(rem * iyy) * 1.0001f + 1e-6f;
-        const float mx = p.x - zp * alpha, my = p.y - zp * beta;
-        const int i0 = max(0, (int)ceilf((mx - hx - g.x0) / g.cell - 0.5f));
-        const int i1 = min(g.nx - 1, (int)floorf((mx + hx - g.x0) / g.cell - 0.5f));
-        const int j0 = max(0, (int)ceilf((my - hy - g.y0) / g.cell - 0.5f));
-        const int j1 = min(g.ny - 1, (int)floorf((my + hy - g.y0) / g.cell - 0.5f));
-        uint32_t *vk = value_bits + (int64_t)k * plane;
-        for (int j = j0; j <= j1; ++j) {
-            const float dy = g.y0 + ((float)j + 0.5f) * g.cell - my;
-            for (int i = i0; i <= i1; ++i) {
-                const float dx = g.x0 + ((float)i + 0.5f) * g.cell - mx;
-                const float q = ez + cxx * dx * dx + 2.0f * cxy * dx * dy + cyy * dy * dy;
-                const float a = o * expf(-0.5f * q);
-                ++evals;
-                if (a >= (1.0f / 255.0f))
-                    atomicMax(&vk[(int64_t)j * g.nx + i], __float_as_uint(fminf(0.99f, a)));
-            }
+        for (int k = 0; k < 3; ++k) {
+            sxz += R[k] * s2[k] * R[6 + k];
+            syz += R[3 + k] * s2[k] * R[6 + k];
+            szz += R[6 + k] * s2[k] * R[6 + k];
+            cxx += R[k] * is2[k] * R[k];
+            cxy += R[k] * is2[k] * R[3 + k];
+            cyy += R[3 + k] * is2[k] * R[3 + k];
+        }
+        lambda = 1.0f / szz;
+        alpha = -sxz / szz;
+        beta = -syz / szz;
+        const float det = cxx * cyy - cxy * cxy;
+        if (det > 0.0f && K >= 0.0f) {
+            // planes within the vertical support lambda z'^2 <= K
+            const float rz = sqrtf(K / lambda) * 1.0001f + 1e-6f;
+            k0 = max((int)ceilf((p.z - rz - g.z0) / g.dz), 0);
+            k1 = min((int)floorf((p.z + rz - g.z0) / g.dz), g.nz - 1);
+            ixx = cyy / det;                                       // C^-1 diagonal
+            iyy = cxx / det;
         }
     }
-    if (work && evals) atomicAdd(work, evals);
+    const int64_t plane = (int64_t)g.nx * g.ny;
+    unsigned long long evals = 0;
+    const bool some = k0 <= k1;
+    const int k_lo = __reduce_min_sync(0xffffffffu, some ? k0 : INT_MAX);
+    const int k_hi = __reduce_max_sync(0xffffffffu, some ? k1 : INT_MIN);
+    // the value of cell (i, j) of item t, folded into the plane's cell
+    auto fold = [&](const SliceItem &t, uint32_t *vk, int i, int j) {
+        const float dy = g.y0 + ((float)j + 0.5f) * g.cell - t.my;
+        const float dx = g.x0 + ((float)i + 0.5f) * g.cell - t.mx;
+        // the terms in this order, the last one rounded before it is added
+        const float q = __fadd_rn(__fmaf_rn(2.0f * t.cxy * dx, dy, __fmaf_rn(t.cxx * dx, dx, t.ez)),
+                                  __fmul_rn(t.cyy * dy, dy));
+        const float a = t.o * expf(-0.5f * q);
+        if (a >= (1.0f / 255.0f))
+            atomicMax(vk + (uint32_t)j * (uint32_t)g.nx + (uint32_t)i,
+                      __float_as_uint(fminf(0.99f, a)));
+    };
+    SliceItem *items = s_item[warp];
+    for (int k = k_lo; k <= k_hi; ++k) {
+        uint32_t *vk = value_bits + (int64_t)k * plane;
+        SliceItem t;
+        uint32_t n = 0, h = 0;   // cells and rows of this thread's slice
+        if (k >= k0 && k <= k1) {
+            const float zp = (g.z0 + (float)k * g.dz) - p.z;
+            const float ez = lambda * zp * zp;
+            const float rem = K - ez;
+            if (rem >= 0.0f) {
+                const float hx = sqrtf(rem * ixx) * 1.0001f + 1e-6f, hy = sqrtf(rem * iyy) * 1.0001f + 1e-6f;
+                const float mx = p.x - zp * alpha, my = p.y - zp * beta;
+                const int i0 = max(0, (int)ceilf((mx - hx - g.x0) / g.cell - 0.5f));
+                const int i1 = min(g.nx - 1, (int)floorf((mx + hx - g.x0) / g.cell - 0.5f));
+                const int j0 = max(0, (int)ceilf((my - hy - g.y0) / g.cell - 0.5f));
+                const int j1 = min(g.ny - 1, (int)floorf((my + hy - g.y0) / g.cell - 0.5f));
+                if (i0 <= i1 && j0 <= j1) {
+                    t.ez = ez; t.cxx = cxx; t.cxy = cxy; t.cyy = cyy;
+                    t.o = o; t.mx = mx; t.my = my;
+                    t.i0 = i0; t.j0 = j0; t.w = i1 - i0 + 1;
+                    t.inv_w = 1.0f / (float)t.w;
+                    h = (uint32_t)(j1 - j0 + 1);
+                    n = (uint32_t)t.w * h;      // < 2^31, the grid's cells
+                    evals += n;
+                }
+            }
+        }
+        for (uint32_t big = __ballot_sync(0xffffffffu, n > kSliceBig); big; big &= big - 1) {
+            const int src = __ffs(big) - 1;
+            if (lane == src) items[0] = t;
+            const uint32_t rows = __shfl_sync(0xffffffffu, h, src);
+            __syncwarp();
+            const SliceItem u = items[0];
+            __syncwarp();
+            for (uint32_t j = 0; j < rows; ++j)
+                for (int i = lane; i < u.w; i += 32) fold(u, vk, u.i0 + i, u.j0 + (int)j);
+        }
+        if (n > kSliceBig) n = 0;
+        // the items that have cells, in lane order, and their cells end to end
+        const uint32_t has = __ballot_sync(0xffffffffu, n > 0);
+        if (has == 0) continue;
+        uint32_t incl = n;
+#pragma unroll
+        for (int s = 1; s < 32; s <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, incl, s);
+            if (lane >= s) incl += v;
+        }
+        const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+        if (n > 0) {
+            t.start = incl - n;
+            items[__popc(has & lanemask_lt())] = t;
+        }
+        __syncwarp();
+        // lane l also holds the start of item l
+        const uint32_t start = lane < __popc(has) ? items[lane].start : 0xffffffffu;
+        for (uint32_t c0 = 0; c0 < total; c0 += 32) {
+            // the item of cell c0 + lane: the last that starts at or before c0, plus
+            // the items that start between
+            const uint32_t at = __popc(__ballot_sync(0xffffffffu, start <= c0)) - 1;
+            const uint32_t off = start - c0;
+            const uint32_t marks =
+                __reduce_or_sync(0xffffffffu, start > c0 && off < 32u ? 1u << off : 0u);
+            const uint32_t c = c0 + lane;
+            if (c < total) {
+                const SliceItem u = items[at + __popc(marks & (lanemask_lt() | 1u << lane))];
+                // row and column in the box: exact, (r + 1/2) / w is at least
+                // 1 / (2 w) from an integer and r < 2^17
+                const uint32_t r = c - u.start;
+                const uint32_t jj = (uint32_t)(((float)r + 0.5f) * u.inv_w);
+                fold(u, vk, u.i0 + (int)(r - jj * (uint32_t)u.w), u.j0 + (int)jj);
+            }
+        }
+        __syncwarp();
+    }
+    // one count per CTA: a count per thread, all on one address, took most of the
+    // kernel's time
+    if (work) {
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) evals += __shfl_down_sync(0xffffffffu, evals, s);
+        if (lane == 0) s_evals[warp] = evals;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < kSliceThreads / 32; ++w) evals += s_evals[w];
+            if (evals) atomicAdd(work, evals);
+        }
+    }
 }
 
 __global__ void k_slice_mask(const uint32_t *__restrict__ value_bits, int64_t n, float threshold,
@@ -129,15 +235,15 @@ void launch_slice(const SceneDev &sc, const SliceGrid &g, float *value, uint8_t 
                   unsigned long long *work, int num_sms, cudaStream_t st) {
     const int64_t cells = (int64_t)g.nx * g.ny * g.nz;
     cudaMemsetAsync(value, 0, (size_t)cells * sizeof(float), st);
-    const int64_t blocks = (sc.n + 255) / 256;
+    const int64_t blocks = (sc.n + kSliceThreads - 1) / kSliceThreads;
     uint32_t *bits = reinterpret_cast<uint32_t *>(value);
     if (blocks > 0) {
         switch (sc.attr_dtype) {
-        case NGS_F16: k_slice<__half><<<(unsigned)blocks, 256, 0, st>>>(sc, g, bits, work); break;
+        case NGS_F16: k_slice<__half><<<(unsigned)blocks, kSliceThreads, 0, st>>>(sc, g, bits, work); break;
         case NGS_BF16:
-            k_slice<__nv_bfloat16><<<(unsigned)blocks, 256, 0, st>>>(sc, g, bits, work);
+            k_slice<__nv_bfloat16><<<(unsigned)blocks, kSliceThreads, 0, st>>>(sc, g, bits, work);
             break;
-        default: k_slice<float><<<(unsigned)blocks, 256, 0, st>>>(sc, g, bits, work); break;
+        default: k_slice<float><<<(unsigned)blocks, kSliceThreads, 0, st>>>(sc, g, bits, work); break;
         }
     }
     if (occ)

@@ -78,3 +78,26 @@ def test_nav_paths_of_other_fields(R):
                     break
             d -= 1
         assert lens[a] == len(cells) and np.array_equal(paths[a, :len(cells)], cells), a
+
+
+@pytest.mark.parametrize("cell,nx,ny,nz", [(0.05, 90, 85, 31), (0.004, 1000, 900, 3), (0.5, 9, 7, 2), (0.03, 1, 40, 40)])
+def test_slice_boxes_of_all_sizes(R, cell, nx, ny, nz):
+    """Boxes from none or one cell to more than a warp takes at once (leaves of up to
+    half a metre on 4 mm cells), and warps whose leaves lie on different planes."""
+    from types import SimpleNamespace
+    import oracle as O
+    from scenegen import make_uniform_box_scene
+    scene = make_uniform_box_scene(700, seed=9)
+    big = np.flatnonzero(scene.child_count == 0)[::50]
+    scene.log_scale[big] = np.log(np.float32(0.5)) - np.float32(0.3) * np.arange(3, dtype=np.float32)
+    R.load_scene(scene)
+    g = SimpleNamespace(x0=0.1, y0=0.05, cell=cell, nx=nx, ny=ny, z0=0.02, dz=0.09, nz=nz, threshold=0.3)
+    got, occ = (t.cpu().numpy() for t in R.slice_occupancy(g))
+    want, want_occ = O.slice_occupancy(scene, g)
+    # within 1e-3, but for cells at the 1/255 cut-off on one side only
+    exempt = (np.minimum(got, want) <= 1.0 / 255.0 + 1e-3) & (np.abs(got - want) > 1e-3)
+    assert exempt.mean() < 0.01
+    assert np.abs(got - want)[~exempt].max() <= 1e-3
+    near = np.abs(want - g.threshold) <= 1e-3
+    assert np.array_equal(occ[~near], want_occ[~near])
+    assert (want > 0).any()
