@@ -21,8 +21,12 @@ namespace {
 
 constexpr uint32_t kEpochStride = 32;   // epoch values reserved per sub-batch
 constexpr int kMaxCamsPerBatch = 1024;
-// ngs_select_cut takes the camera-blocked two-pass cut from this many cameras on
-constexpr int kCutBlockedMinCams = 4;
+// cuts of this many cameras or more (and no group of more than 32) are decided as
+// masks over the cameras, the others by the single-pass kernels. Measured on a 1M-leaf
+// floor, masks / single pass: 4 cameras 93 / 120 us (plain), 117 / 177 us (frustum), 116 /
+// 119 us (one group of 4); the masks' cost is that of 8 cameras for fewer, the single
+// pass takes 73, 87, 110 us for 1, 2, 3
+constexpr int kCutMasksMinCams = 4;
 constexpr int kMaxCamsPerCall = 1 << 16;
 constexpr int kTuneShapes = NGS_TUNE_SHAPES;
 // renders of one ngs_render_host call after a pair-buffer overflow
@@ -91,7 +95,8 @@ struct ngs_ctx {
     uint32_t *cut_off32 = nullptr;     // scratch for ngs_select_cut offsets
     CutCam *cut_cams = nullptr;        // ngs_select_cut_shared: cameras and groups
     int32_t *cut_groups = nullptr;
-    uint32_t *cut_counts = nullptr;    // many-camera ngs_select_cut: (camera, block) counts
+    CutChunk *cut_chunks = nullptr;    // cuts by masks: chunks of the cameras,
+    uint32_t *cut_counts = nullptr;    // (unit, block) counts
     uint32_t *cut_poff = nullptr;      // and their scanned offsets
 
     // occupancy-derived persistent grids
@@ -200,6 +205,7 @@ void free_work(ngs_ctx *c) {
     dfree(c->cut_off32);
     dfree(c->cut_cams);
     dfree(c->cut_groups);
+    dfree(c->cut_chunks);
     dfree(c->cut_counts);
     dfree(c->cut_poff);
     c->w = Work();
@@ -207,6 +213,7 @@ void free_work(ngs_ctx *c) {
     c->cut_off32 = nullptr;
     c->cut_cams = nullptr;
     c->cut_groups = nullptr;
+    c->cut_chunks = nullptr;
     c->cut_counts = nullptr;
     c->cut_poff = nullptr;
     c->work_ready = false;
@@ -332,6 +339,7 @@ ngs_status ensure_work(ngs_ctx *c) {
     A(dalloc(&c->cut_off32, kMaxCamsPerBatch + 1));
     A(dalloc(&c->cut_cams, kMaxCamsPerBatch));
     A(dalloc(&c->cut_groups, kMaxCamsPerBatch + 1));
+    A(dalloc(&c->cut_chunks, kMaxCamsPerBatch));
     A(dalloc(&c->cut_counts, (size_t)(nblk * kMaxCamsPerBatch)));
     A(dalloc(&c->cut_poff, (size_t)(nblk * kMaxCamsPerBatch)));
     A(dalloc(&w.work64, kWork64Words));
@@ -442,6 +450,80 @@ void fill_cut_cam(CutCam &d, const ngs_camera &k, float guard) {
     for (int i = 0; i < 3; ++i) d.pos[i] = k.pos[i];
     d.fx = k.fx;
     d.tau = k.tau;
+}
+
+// Units whose mask words fit in the record buffer at once (the words live there
+// between the passes of a cut: no render is in flight).
+int64_t cut_slice_units(const ngs_ctx *c) {
+    return c->w.rec_cap * (int64_t)sizeof(Rec32) /
+           (cut_words_per_unit(c->scene.n) * (int64_t)sizeof(uint32_t));
+}
+
+// Whether a cut goes by masks: enough cameras for a lane each, groups that fit a
+// mask, and room for at least one unit's words.
+bool cut_masks_ok(const ngs_ctx *c, int n_cams, const int32_t *group_begin, int n_units) {
+    if (n_cams < kCutMasksMinCams || cut_slice_units(c) < 1) return false;
+    if (group_begin)
+        for (int g = 0; g < n_units; ++g)
+            if (group_begin[g + 1] - group_begin[g] > 32) return false;
+    return true;
+}
+
+// The cuts of n_units cameras (group_begin null) or groups, enqueued on st: as
+// many units at a time as their mask words fit.
+ngs_status cut_by_masks(ngs_ctx *c, const std::vector<CutCam> &hc, const int32_t *group_begin,
+                        int n_units, bool frustum, int32_t *d_ids, int64_t *d_offsets, int64_t cap,
+                        cudaStream_t st) {
+    Work &w = c->w;
+    const SceneDev &sc = c->scene;
+    const int n_cams = (int)hc.size();
+    auto begin = [&](int u) { return group_begin ? group_begin[u] : u; };
+    int lanes = n_cams <= 8 ? 8 : n_cams <= 16 ? 16 : 32;
+    const int slice = (int)std::min<int64_t>(n_units, cut_slice_units(c));
+    std::vector<CutChunk> chunks;
+    std::vector<int> first_chunk;   // of each slice
+    for (int u0 = 0; u0 < n_units; u0 += slice) {
+        first_chunk.push_back((int)chunks.size());
+        const int u1 = std::min(n_units, u0 + slice);
+        for (int u = u0; u < u1;) {
+            CutChunk ch{begin(u), 0, u - u0, 0};
+            while (u < u1 && begin(u + 1) - ch.cam0 <= lanes) {
+                ch.n_cams = begin(u + 1) - ch.cam0;
+                ++ch.n_units;
+                ++u;
+            }
+            chunks.push_back(ch);
+        }
+    }
+    first_chunk.push_back((int)chunks.size());
+    CK(cudaMemcpyAsync(c->cut_cams, hc.data(), sizeof(CutCam) * n_cams, cudaMemcpyHostToDevice,
+                       st));
+    CK(cudaMemcpyAsync(c->cut_chunks, chunks.data(), sizeof(CutChunk) * chunks.size(),
+                       cudaMemcpyHostToDevice, st));
+    if (group_begin)
+        CK(cudaMemcpyAsync(c->cut_groups, group_begin, sizeof(int32_t) * (n_units + 1),
+                           cudaMemcpyHostToDevice, st));
+    const int64_t nblk = (sc.n + cut_partition_nodes() - 1) / cut_partition_nodes();
+    uint32_t *words = (uint32_t *)w.rec;
+    for (size_t k = 0; k + 1 < first_chunk.size(); ++k) {
+        const int u0 = (int)k * slice, nu = std::min(slice, n_units - u0);
+        ngs_status s = epoch_guard(c, st, kEpochStride);
+        if (s != NGS_OK) return s;
+        CK(cudaMemsetAsync(w.counters, 0, N_COUNTERS * sizeof(uint32_t), st));
+        k_bump_epoch<<<1, 1, 0, st>>>(w.epoch, kEpochStride);
+        launch_cut_masks(frustum, group_begin != nullptr, lanes, sc.box_lo, sc.box_hi, sc.n,
+                         c->cut_cams, c->cut_groups + u0, c->cut_chunks + first_chunk[k],
+                         first_chunk[k + 1] - first_chunk[k], words, c->cut_counts, w.err, st);
+        const int64_t np = nblk * nu, sparts = (np + scan_partition() - 1) / scan_partition();
+        launch_scan_u32(c->cut_counts, c->cut_poff, nullptr, np, c->cut_off32,
+                        w.counters + TK_SCAN, w.status, w.epoch, 0, w.err,
+                        (int)std::min<int64_t>(sparts, c->grid_scan), st);
+        launch_cut_write(words, c->cut_poff, c->cut_off32, sc.n, nu, k == 0,
+                         k + 2 == first_chunk.size(), cap, (uint32_t *)d_ids, d_offsets + u0,
+                         w.counters, w.err, st);
+    }
+    CK(cudaGetLastError());
+    return NGS_OK;
 }
 
 int bits_for(uint32_t n) {
@@ -1187,32 +1269,22 @@ NGS_API ngs_status ngs_select_cut(ngs_ctx *c, const ngs_camera *cams, int32_t n_
     ngs_status s = ensure_work(c);
     if (s != NGS_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
-    std::vector<DevCamera> hc(n_cams);
-    for (int i = 0; i < n_cams; ++i) fill_cam(hc[i], cams[i], c->tile_w, c->tile_h, nullptr);
     Work &w = c->w;
-    if ((s = epoch_guard(c, st, kEpochStride)) != NGS_OK) return s;
-    CK(cudaMemcpyAsync(w.cams, hc.data(), sizeof(DevCamera) * n_cams, cudaMemcpyHostToDevice, st));
-    CK(cudaMemsetAsync(w.counters, 0, N_COUNTERS * sizeof(uint32_t), st));
-    k_bump_epoch<<<1, 1, 0, st>>>(w.epoch, kEpochStride);
     const int64_t cap32 = std::min<int64_t>(cap, (1ll << 32) - 1);
-    if (n_cams >= kCutBlockedMinCams) {
-        // count per (camera, block), scan in camera-major order, write
-        const SceneDev &sc = c->scene;
-        const int64_t nblk = (sc.n + cut_partition_nodes() - 1) / cut_partition_nodes();
-        const int64_t np = nblk * n_cams;
-        launch_cut_blocked(false, sc.box_lo, sc.box_hi, sc.n, w.cams, nullptr, n_cams,
-                           c->cut_counts, nullptr, cap32, w.counters + TK_CUT, w.err, c->grid_cut,
-                           st);
-        const int64_t sparts = (np + scan_partition() - 1) / scan_partition();
-        launch_scan_u32(c->cut_counts, c->cut_poff, nullptr, np, c->cut_off32,
-                        w.counters + TK_SCAN, w.status, w.epoch, 0, w.err,
-                        (int)std::min<int64_t>(sparts, c->grid_scan), st);
-        launch_cut_cam_offsets(c->cut_poff, c->cut_off32, nblk, n_cams, cap32, d_offsets,
-                               w.counters, w.err, st);
-        launch_cut_blocked(true, sc.box_lo, sc.box_hi, sc.n, w.cams, nullptr, n_cams,
-                           c->cut_poff, (uint32_t *)d_ids, cap32, w.counters + TK_PRE, w.err,
-                           c->grid_cut, st);
+    if (cut_masks_ok(c, n_cams, nullptr, n_cams)) {
+        std::vector<CutCam> hc(n_cams);
+        for (int i = 0; i < n_cams; ++i) fill_cut_cam(hc[i], cams[i], 0.0f);
+        if ((s = cut_by_masks(c, hc, nullptr, n_cams, false, d_ids, d_offsets, cap32, st)) != NGS_OK)
+            return s;
     } else {
+        std::vector<DevCamera> hc(n_cams);
+        for (int i = 0; i < n_cams; ++i)
+            fill_cam(hc[i], cams[i], c->tile_w, c->tile_h, nullptr);
+        if ((s = epoch_guard(c, st, kEpochStride)) != NGS_OK) return s;
+        CK(cudaMemcpyAsync(w.cams, hc.data(), sizeof(DevCamera) * n_cams, cudaMemcpyHostToDevice,
+                           st));
+        CK(cudaMemsetAsync(w.counters, 0, N_COUNTERS * sizeof(uint32_t), st));
+        k_bump_epoch<<<1, 1, 0, st>>>(w.epoch, kEpochStride);
         launch_cut(c->scene, w.cams, n_cams, (uint32_t *)d_ids, cap32, c->cut_off32, w.counters,
                    w.counters + TK_CUT, w.status, w.epoch, 0, w.err, c->grid_cut, st);
         k_offsets_to_i64<<<(n_cams + 256) / 256, 256, 0, st>>>(c->cut_off32, d_offsets, n_cams);
@@ -1247,6 +1319,14 @@ NGS_API ngs_status ngs_select_cut_shared(ngs_ctx *c, const ngs_camera *cams, int
     std::vector<CutCam> hc(n_cams);
     for (int i = 0; i < n_cams; ++i) fill_cut_cam(hc[i], cams[i], guard_px);
     Work &w = c->w;
+    const int64_t cap32 = std::min<int64_t>(cap, (1ll << 32) - 1);
+    if (cut_masks_ok(c, n_cams, group_begin, n_groups)) {
+        s = cut_by_masks(c, hc, n_groups == n_cams ? nullptr : group_begin, n_groups,
+                         (flags & NGS_CUT_FRUSTUM) != 0, d_ids, d_offsets, cap32, st);
+        if (s != NGS_OK) return s;
+        CK(cudaStreamSynchronize(st));
+        return check_err(c);
+    }
     if ((s = epoch_guard(c, st, kEpochStride)) != NGS_OK) return s;
     CK(cudaMemcpyAsync(c->cut_cams, hc.data(), sizeof(CutCam) * n_cams, cudaMemcpyHostToDevice,
                        st));
@@ -1254,28 +1334,6 @@ NGS_API ngs_status ngs_select_cut_shared(ngs_ctx *c, const ngs_camera *cams, int
                        cudaMemcpyHostToDevice, st));
     CK(cudaMemsetAsync(w.counters, 0, N_COUNTERS * sizeof(uint32_t), st));
     k_bump_epoch<<<1, 1, 0, st>>>(w.epoch, kEpochStride);
-    const int64_t cap32 = std::min<int64_t>(cap, (1ll << 32) - 1);
-    if (n_groups == n_cams && n_cams >= kCutBlockedMinCams && (flags & NGS_CUT_FRUSTUM)) {
-        // one frustum-culled cut per camera: the camera-blocked two-pass form
-        const SceneDev &sc = c->scene;
-        const int64_t nblk = (sc.n + cut_partition_nodes() - 1) / cut_partition_nodes();
-        const int64_t np = nblk * n_cams;
-        launch_cut_blocked(false, sc.box_lo, sc.box_hi, sc.n, nullptr, c->cut_cams, n_cams,
-                           c->cut_counts, nullptr, cap32, w.counters + TK_CUT, w.err, c->grid_cut,
-                           st);
-        const int64_t sparts = (np + scan_partition() - 1) / scan_partition();
-        launch_scan_u32(c->cut_counts, c->cut_poff, nullptr, np, c->cut_off32,
-                        w.counters + TK_SCAN, w.status, w.epoch, 0, w.err,
-                        (int)std::min<int64_t>(sparts, c->grid_scan), st);
-        launch_cut_cam_offsets(c->cut_poff, c->cut_off32, nblk, n_cams, cap32, d_offsets,
-                               w.counters, w.err, st);
-        launch_cut_blocked(true, sc.box_lo, sc.box_hi, sc.n, nullptr, c->cut_cams, n_cams,
-                           c->cut_poff, (uint32_t *)d_ids, cap32, w.counters + TK_PRE, w.err,
-                           c->grid_cut, st);
-        CK(cudaGetLastError());
-        CK(cudaStreamSynchronize(st));
-        return check_err(c);
-    }
     launch_cut_shared((flags & NGS_CUT_FRUSTUM) != 0, c->scene.box_lo, c->scene.box_hi,
                       c->scene.n, c->cut_cams, c->cut_groups, n_groups, (uint32_t *)d_ids,
                       cap32, c->cut_off32, w.counters,

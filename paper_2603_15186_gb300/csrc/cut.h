@@ -32,25 +32,30 @@ void launch_cut_shared(bool frustum, const float4 *box_lo, const float4 *box_hi,
                        uint32_t *ticket, uint64_t *status, const uint32_t *epoch,
                        uint32_t epoch_off, int *err, int grid, cudaStream_t st);
 
-// Plain cut for many cameras (ngs_select_cut), in two passes over (block of
-// cut_partition_nodes() nodes, chunk of up to 8 cameras) partitions taken in
-// block-major order. The counting pass writes part_vals[c * nblk + b] = the
-// selected nodes of camera c in block b; a chained scan of those counts in
-// camera-major order gives each (camera, block) its output offset; the
-// writing pass reads those offsets from part_vals and writes the ids. Both
-// passes return at once if *err is set. With ccams (instead of cams, which is
-// then unused) each camera's cut is frustum-culled against its planes: the
-// shared cut of a group of one camera.
-void launch_cut_blocked(bool write, const float4 *box_lo, const float4 *box_hi, int64_t n_nodes,
-                        const DevCamera *cams, const CutCam *ccams, int n_cams,
-                        uint32_t *part_vals, uint32_t *ids, int64_t cap, uint32_t *ticket,
-                        const int *err, int grid, cudaStream_t st);
+// A chunk of a call's cameras, cams[cam0 .. cam0 + n_cams) (at most 32), and its
+// units (cameras or whole groups), unit0 counted within the slice.
+struct CutChunk {
+    int32_t cam0, n_cams, unit0, n_units;
+};
 
-// offsets[c] = part_off[c * nblk] for c < n_cams, offsets[n_cams] = *total
-// (int64); latches the capacity error when *total exceeds cap.
-void launch_cut_cam_offsets(const uint32_t *part_off, const uint32_t *total, int64_t nblk,
-                            int n_cams, int64_t cap, int64_t *offsets, uint32_t *counters,
-                            int *err, cudaStream_t st);
+// Cuts of many units, one slice of them at a time: launch_cut_masks decides, for
+// chunks of at most c <= 32 cameras, every (node, unit) into words[unit *
+// cut_words_per_unit() ...] and counts[unit * blocks + block] (blocks of
+// cut_partition_nodes() nodes); after an exclusive scan of the counts into part_off
+// (its sum in *total), launch_cut_write writes the units' offsets (offsets[0] ..
+// offsets[n_units], continuing from offsets[0] unless `first`) and ids; with `last`
+// also counters[CNT_CUT], and it latches the capacity error when the ids exceed cap.
+// group_begin (with groups): the slice's entries. Without groups a unit is a camera.
+// frustum: the cameras' planes cull.
+void launch_cut_masks(bool frustum, bool groups, int c, const float4 *box_lo,
+                      const float4 *box_hi, int64_t n_nodes, const CutCam *cams,
+                      const int32_t *group_begin, const CutChunk *chunks, int n_chunks,
+                      uint32_t *words, uint32_t *counts, const int *err, cudaStream_t st);
+void launch_cut_write(const uint32_t *words, const uint32_t *part_off, const uint32_t *total,
+                      int64_t n_nodes, int n_units, bool first, bool last, int64_t cap,
+                      uint32_t *ids, int64_t *offsets, uint32_t *counters, int *err,
+                      cudaStream_t st);
+int64_t cut_words_per_unit(int64_t n_nodes);
 
 }  // namespace ngs
 

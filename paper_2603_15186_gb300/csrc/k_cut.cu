@@ -216,215 +216,290 @@ k_cut_shared(const float4 *__restrict__ box_lo, const float4 *__restrict__ box_h
                    epoch_ptr, epoch_off, err);
 }
 
-// Many-camera plain cut. A partition is (node block b, chunk of kCutCams
-// cameras), taken in block-major order so that a block's boxes come from HBM
-// once and from L2 for its other chunks; every camera of the chunk is tested
-// on the node and parent boxes loaded once. Pass 1 stores each camera's count
-// for the block; pass 2 (after a scan of the counts in camera-major order)
-// recomputes the selection and writes the ids at the scanned offset plus the
-// prefix within the block. No partition waits on another.
-// With kFrustum (a frustum-culled cut per camera, i.e. shared cuts in groups of
-// one) a node is also dropped when its box lies outside one of the camera's
-// five planes: for a single camera that is its plain cut minus the culled
-// nodes (a culled parent culls the node).
-constexpr int kCutCams = 8;
-static_assert(kCutThreads / 32 == kCutCams, "one warp scans one camera's row counts");
+// Cuts of many cameras or groups ("units"), in three steps: k_cut_masks decides
+// every (node, unit) and keeps one bit each, 32 nodes to a word, and each unit's
+// count per node block; a scan of the counts in unit-major order gives the output
+// offsets (k_cut_unit_offsets: those of the units); k_cut_write turns the words into
+// ids, a pure stream.
+//
+// k_cut_masks: one CTA per (block of kCutPart nodes, chunk of up to C cameras). The
+// tests are taken with one lane per camera, 32 / C boxes at a time, so that a ballot
+// is the box's mask over the chunk's cameras: N (the camera keeps the box and it is
+// not fine enough) and, with kFrustum, V (the camera keeps it). Per word of 32 nodes
+//   - the distinct parents (siblings follow one another) are tested once each;
+//   - then the interior nodes that some camera of the chunk still wants refined;
+//   - a leaf has N = 0; its V is tested only for the cameras whose unit wants its
+//     parent refined, one lane per leaf, until a camera of the unit keeps it.
+// A unit's decision is bits: (leaf or no N_n) and (root or some N_p) and some V_n over
+// the unit's cameras. Without kGroups (units of one camera) that is the same formula
+// on whole masks, and a 32 x 32 bit transpose turns 32 nodes' masks into the cameras'
+// words. With kFrustum a word whose boxes' union every camera culls is left out (a box
+// outside a half-space has every box it contains outside too, also in float32: the
+// tests are monotone in the bounds).
+//
+// Bound by the issue of the tests (about 14 instructions for a granularity, 75 for
+// five planes). A test per (node, camera) on the node and on its parent, once to count
+// and once to write, took 683 + 1016 us for 64 plain cuts of 5.25 M nodes, and one
+// thread per node over its group's members 1557 us for 8 frustum-culled cuts of 8
+// cameras each; CUT_NOTE
+constexpr int kCutWords = kCutPart / 32;
 
-template <bool kWrite, bool kFrustum>
+template <bool kFrustum, bool kGroups, int C>
 __global__ void __launch_bounds__(kCutThreads)
-k_cut_blocked(const float4 *__restrict__ box_lo, const float4 *__restrict__ box_hi,
-              int64_t n_nodes, const DevCamera *__restrict__ cams,
-              const CutCam *__restrict__ ccams, int n_cams,
-              uint32_t *__restrict__ part_vals, uint32_t *__restrict__ ids, int64_t cap,
-              uint32_t *ticket, const int *err) {
-    __shared__ float s_cam[kCutCams][5];                   // pos xyz, fx, tau^2 (rounded)
-    __shared__ CutCam s_ccam[kFrustum ? kCutCams : 1];     // the cameras' planes
-    __shared__ uint32_t s_bal[kCutCams][kCutItems * 8];    // ballot per (camera, row, warp)
-    __shared__ uint32_t s_off[kCutCams][kCutItems * 8];    // its exclusive offset in the block
-    __shared__ uint32_t s_part;
+k_cut_masks(const float4 *__restrict__ box_lo, const float4 *__restrict__ box_hi,
+            int64_t n_nodes, const CutCam *__restrict__ cams,
+            const int32_t *__restrict__ group_begin, const CutChunk *__restrict__ chunks,
+            int n_chunks, uint32_t *__restrict__ words, uint32_t *__restrict__ counts,
+            const int *err) {
+    constexpr int G = 32 / C, kWarps = kCutThreads / 32;
+    static_assert(kCutWords % kWarps == 0 && kCutWords == 64, "two words per lane");
+    __shared__ float4 s_lo[kWarps][32], s_hi[kWarps][32];   // the boxes under test, per warp
+    __shared__ uint32_t s_word[C][kCutWords + 1];
+    __shared__ CutCam s_cam[kFrustum ? C : 1];
+    __shared__ uint32_t s_unit[kGroups ? C : 1];   // each unit's cameras of the chunk
     if (*err) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t nblk = (n_nodes + kCutPart - 1) / kCutPart;
-    const int nchunk = (n_cams + kCutCams - 1) / kCutCams;
-    const int64_t nparts = nblk * nchunk;
-    for (;;) {
-        if (tid == 0) s_part = atomicAdd(ticket, 1u);
-        __syncthreads();
-        const int64_t part = s_part;
-        if (part >= nparts) break;
-        const int64_t b = part / nchunk;
-        const int c0 = (int)(part - b * nchunk) * kCutCams;
-        const int nc = min(kCutCams, n_cams - c0);
-        if (tid < kCutCams * 5) {
-            const int j = tid / 5, f = tid - 5 * j;
-            float v = 0.0f;
-            if (j < nc) {
-                if (kFrustum) {
-                    const CutCam &k = ccams[c0 + j];
-                    v = f < 3 ? k.pos[f] : (f == 3 ? k.fx : __fmul_rn(k.tau, k.tau));
-                } else {
-                    const DevCamera &k = cams[c0 + j];
-                    v = f < 3 ? k.pos[f] : (f == 3 ? k.fx : __fmul_rn(k.tau, k.tau));
-                }
-            }
-            s_cam[j][f] = v;
-        }
-        if (kFrustum && tid < kCutCams * (int)(sizeof(CutCam) / 4)) {
-            const int j = tid / (int)(sizeof(CutCam) / 4), f = tid - j * (int)(sizeof(CutCam) / 4);
-            if (j < nc)
-                reinterpret_cast<float *>(&s_ccam[j])[f] =
-                    reinterpret_cast<const float *>(&ccams[c0 + j])[f];
+    const int64_t b = blockIdx.x / n_chunks;
+    const CutChunk ch = chunks[blockIdx.x - b * n_chunks];
+    const uint32_t live = ch.n_cams == 32 ? 0xffffffffu : (1u << ch.n_cams) - 1u;
+    // this lane's camera
+    const int cl = lane % C, grp = lane / C;
+    const CutCam cam = cams[ch.cam0 + min(cl, ch.n_cams - 1)];
+    const float tau2 = __fmul_rn(cam.tau, cam.tau);
+    if (kFrustum) {
+        if (tid < ch.n_cams) s_cam[tid] = cams[ch.cam0 + tid];
+        if (kGroups && tid < ch.n_units) {
+            const int g0 = group_begin[ch.unit0 + tid] - ch.cam0, g1 = group_begin[ch.unit0 + tid + 1] - ch.cam0;
+            s_unit[tid] = (g1 == 32 ? 0xffffffffu : (1u << g1) - 1u) & ~((1u << g0) - 1u);
         }
         __syncthreads();
-#pragma unroll 1
-        for (int k = 0; k < kCutItems; ++k) {
-            const int64_t node = b * kCutPart + k * kCutThreads + tid;
-            const bool valid = node < n_nodes;
-            float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo, plo = lo, phi = lo;
-            int parent = -1;
-            bool leaf = true;
-            if (valid) {
-                lo = box_lo[node];
-                hi = box_hi[node];
-                parent = __float_as_int(lo.w);
-                leaf = __float_as_int(hi.w) == 0;
-                if (parent >= 0) {
-                    plo = box_lo[parent];
-                    phi = box_hi[parent];
-                }
+    } else if (kGroups) {
+        if (tid < ch.n_units) {
+            const int g0 = group_begin[ch.unit0 + tid] - ch.cam0, g1 = group_begin[ch.unit0 + tid + 1] - ch.cam0;
+            s_unit[tid] = (g1 == 32 ? 0xffffffffu : (1u << g1) - 1u) & ~((1u << g0) - 1u);
+        }
+        __syncthreads();
+    }
+    // masks (N, V) of the staged boxes; a lane whose box is number `rank` gets them
+    auto test = [&](int n, int rank, uint32_t &N, uint32_t &V) {
+        __syncwarp();
+#pragma unroll 2
+        for (int t = 0; t < n; t += G) {
+            const int k = min(t + grp, n - 1);
+            const float4 lo = s_lo[warp][k], hi = s_hi[warp][k];
+            const bool keep = !kFrustum || !frustum_culled(cam, lo, hi);
+            const bool fine = fine_enough_pre(lo, hi, box_extent(lo, hi), cam.pos[0], cam.pos[1],
+                                              cam.pos[2], cam.fx, tau2);
+            const uint32_t nm = __ballot_sync(0xffffffffu, keep && !fine);
+            const uint32_t vm = kFrustum ? __ballot_sync(0xffffffffu, keep) : 0xffffffffu;
+            const int at = rank - t;
+            if (at >= 0 && at < G) {
+                N = nm >> (C * at % 32);
+                V = vm >> (C * at % 32);
             }
-            // kFrustum: the cameras whose view volume the union of the warp's
-            // node boxes can meet (a box outside a half-space has every box it
-            // contains outside too, also in float32: the tests are monotone in
-            // the bounds); the others cull all 32 nodes without a test per node
-            uint32_t live = (1u << nc) - 1u;
+        }
+        __syncwarp();
+    };
+    for (int j = warp; j < kCutWords; j += kWarps) {
+        const int64_t node = b * kCutPart + 32 * j + lane;
+        const bool valid = node < n_nodes;
+        float4 lo = make_float4(0.f, 0.f, 0.f, __int_as_float(-1)), hi = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (valid) {
+            lo = box_lo[node];
+            hi = box_hi[node];
+        }
+        const int parent = __float_as_int(lo.w);
+        const bool leaf = __float_as_int(hi.w) == 0;
+        bool look = __any_sync(0xffffffffu, valid);
+        if (kFrustum && look) {
+            const float inf = __int_as_float(0x7f800000);
+            float4 ulo = valid ? lo : make_float4(inf, inf, inf, 0.f);
+            float4 uhi = valid ? hi : make_float4(-inf, -inf, -inf, 0.f);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                ulo.x = fminf(ulo.x, __shfl_xor_sync(0xffffffffu, ulo.x, o));
+                ulo.y = fminf(ulo.y, __shfl_xor_sync(0xffffffffu, ulo.y, o));
+                ulo.z = fminf(ulo.z, __shfl_xor_sync(0xffffffffu, ulo.z, o));
+                uhi.x = fmaxf(uhi.x, __shfl_xor_sync(0xffffffffu, uhi.x, o));
+                uhi.y = fmaxf(uhi.y, __shfl_xor_sync(0xffffffffu, uhi.y, o));
+                uhi.z = fmaxf(uhi.z, __shfl_xor_sync(0xffffffffu, uhi.z, o));
+            }
+            look = __any_sync(0xffffffffu, cl < ch.n_cams && !frustum_culled(cam, ulo, uhi));
+        }
+        uint32_t sel = 0;     // bit u: unit u (camera, without kGroups) selects the node
+        if (look) {
+            // the parents
+            const int before = __shfl_up_sync(0xffffffffu, parent, 1);
+            const bool first = valid && parent >= 0 && (lane == 0 || parent != before);
+            const uint32_t firsts = __ballot_sync(0xffffffffu, first);
+            const int rank = __popc(firsts & (lanemask_lt() | 1u << lane)) - 1;
+            if (first) {
+                s_lo[warp][rank] = box_lo[parent];
+                s_hi[warp][rank] = box_hi[parent];
+            }
+            uint32_t Np = 0, Vp = 0;
+            test(__popc(firsts), valid && parent >= 0 ? rank : -1, Np, Vp);
+            if (valid && parent < 0) Np = 0xffffffffu;   // the root: as if a parent were refined
+            Np &= live;
+            // the cameras whose units want the parent refined
+            uint32_t want = Np;
+            if (kGroups) {
+                want = 0;
+                for (int u = 0; u < ch.n_units; ++u)
+                    if (Np & s_unit[u]) want |= s_unit[u];
+            }
+            // the interior nodes among them
+            uint32_t Nn = 0, Vn = kFrustum ? 0u : 0xffffffffu;
+            const bool inner = !leaf && want != 0;
+            const uint32_t inners = __ballot_sync(0xffffffffu, inner);
+            const int irank = __popc(inners & lanemask_lt());
+            if (inner) {
+                s_lo[warp][irank] = lo;
+                s_hi[warp][irank] = hi;
+            }
+            test(__popc(inners), inner ? irank : -1, Nn, Vn);
             if (kFrustum) {
-                const float inf = __int_as_float(0x7f800000);
-                float4 ulo = valid ? lo : make_float4(inf, inf, inf, 0.f);
-                float4 uhi = valid ? hi : make_float4(-inf, -inf, -inf, 0.f);
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    ulo.x = fminf(ulo.x, __shfl_xor_sync(0xffffffffu, ulo.x, o));
-                    ulo.y = fminf(ulo.y, __shfl_xor_sync(0xffffffffu, ulo.y, o));
-                    ulo.z = fminf(ulo.z, __shfl_xor_sync(0xffffffffu, ulo.z, o));
-                    uhi.x = fmaxf(uhi.x, __shfl_xor_sync(0xffffffffu, uhi.x, o));
-                    uhi.y = fmaxf(uhi.y, __shfl_xor_sync(0xffffffffu, uhi.y, o));
-                    uhi.z = fmaxf(uhi.z, __shfl_xor_sync(0xffffffffu, uhi.z, o));
-                }
-                uint32_t keep = 0;
-                if (ulo.x <= uhi.x) {   // some valid node
-#pragma unroll 1
-                    for (int j = 0; j < nc; ++j)
-                        if (!frustum_culled(s_ccam[j], ulo, uhi)) keep |= 1u << j;
-                }
-                live = keep;
-            }
-            const float ext_n = box_extent(lo, hi), ext_p = box_extent(plo, phi);
-            uint32_t m = 0;   // bit j: camera j selects the node
-#pragma unroll
-            for (int j = 0; j < kCutCams; ++j) {
-                if (valid && j < nc && ((live >> j) & 1u)) {
-                    const float px = s_cam[j][0], py = s_cam[j][1], pz = s_cam[j][2];
-                    const float fx = s_cam[j][3], tau2 = s_cam[j][4];
-                    // the rule of cut_selects, parent first (most nodes lie below the cut)
-                    if ((parent < 0 ||
-                         !fine_enough_pre(plo, phi, ext_p, px, py, pz, fx, tau2)) &&
-                        (leaf || fine_enough_pre(lo, hi, ext_n, px, py, pz, fx, tau2)))
-                        m |= 1u << j;
-                }
-            }
-            if (kFrustum) {
-                // not unrolled: the planes stay in shared memory instead of
-                // occupying registers for all cameras of the chunk at once
-                uint32_t rest = m;
-#pragma unroll 1
-                while (rest) {
-                    const int j = __ffs(rest) - 1;
-                    rest &= rest - 1;
-                    if (frustum_culled(s_ccam[j], lo, hi)) m &= ~(1u << j);
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < kCutCams; ++j) {
-                const uint32_t bal = __ballot_sync(0xffffffffu, (m >> j) & 1u);
-                if (lane == 0) s_bal[j][k * 8 + warp] = bal;
-            }
-        }
-        __syncthreads();
-        if (warp < nc) {
-            // warp j: exclusive scan of camera j's 64 (row, warp) counts in node order
-            const int j = warp;
-            const uint32_t v0 = __popc(s_bal[j][2 * lane]), v1 = __popc(s_bal[j][2 * lane + 1]);
-            uint32_t incl = v0 + v1;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += t;
-            }
-            const uint32_t excl = incl - (v0 + v1);
-            s_off[j][2 * lane] = excl;
-            s_off[j][2 * lane + 1] = excl + v0;
-            if (!kWrite && lane == 31) part_vals[(int64_t)(c0 + j) * nblk + b] = incl;
-        }
-        if (kWrite) {
-            __syncthreads();
-            for (int j = 0; j < nc; ++j) {
-                const uint64_t base = part_vals[(int64_t)(c0 + j) * nblk + b];
-#pragma unroll
-                for (int k = 0; k < kCutItems; ++k) {
-                    const uint32_t bal = s_bal[j][k * 8 + warp];
-                    if ((bal >> lane) & 1u) {
-                        const uint64_t pos =
-                            base + s_off[j][k * 8 + warp] + __popc(bal & lanemask_lt());
-                        if (pos < (uint64_t)cap)
-                            ids[pos] = (uint32_t)(b * kCutPart + k * kCutThreads + tid);
+                // the leaves: a lane each, camera by camera
+                uint32_t need = leaf ? want : 0u;
+                for (uint32_t c = __reduce_or_sync(0xffffffffu, need); c; c &= c - 1) {
+                    const int k = __ffs(c) - 1;
+                    if (need >> k & 1u) {
+                        if (!frustum_culled(s_cam[k], lo, hi)) {
+                            Vn |= 1u << k;
+                            if (kGroups)   // its unit's other cameras need not look
+                                for (int u = 0; u < ch.n_units; ++u)
+                                    if (s_unit[u] >> k & 1u) need &= ~s_unit[u];
+                        }
                     }
                 }
             }
+            if (kGroups) {
+                for (int u = 0; u < ch.n_units; ++u) {
+                    const uint32_t m = s_unit[u];
+                    if ((leaf || !(Nn & m)) && (Np & m) && (Vn & m)) sel |= 1u << u;
+                }
+            } else {
+                sel = (leaf ? 0xffffffffu : ~Nn) & Np & Vn;
+            }
+            if (!valid) sel = 0;
         }
-        __syncthreads();
+        // rows of nodes to rows of units
+        uint32_t x = sel, m = 0x0000ffffu;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const uint32_t y = __shfl_xor_sync(0xffffffffu, x, o);
+            x = lane & o ? (x & ~m) | (y & ~m) >> o : (x & m) | (y & m) << o;
+            m ^= m << (o >> 1);
+        }
+        if (lane < C) s_word[lane][j] = x;
+    }
+    __syncthreads();
+    for (int u = warp; u < ch.n_units; u += kWarps) {
+        const uint32_t x = s_word[u][2 * lane], y = s_word[u][2 * lane + 1];
+        const uint32_t n = __reduce_add_sync(0xffffffffu, (uint32_t)(__popc(x) + __popc(y)));
+        const int64_t at = (int64_t)(ch.unit0 + u) * nblk + b;
+        reinterpret_cast<uint2 *>(words)[at * (kCutWords / 2) + lane] = make_uint2(x, y);
+        if (lane == 0) counts[at] = n;
     }
 }
 
-__global__ void k_cut_cam_offsets(const uint32_t *__restrict__ part_off,
-                                  const uint32_t *__restrict__ total, int64_t nblk, int n_cams,
-                                  int64_t cap, int64_t *__restrict__ offsets,
-                                  uint32_t *__restrict__ counters, int *err) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i > n_cams) return;
-    const uint32_t t = *total;
-    offsets[i] = i < n_cams ? (int64_t)part_off[(int64_t)i * nblk] : (int64_t)t;
-    if (i == n_cams) {
-        counters[CNT_CUT] = t;
-        if ((int64_t)t > cap) latch_error(err, kErrCapacity);
+// The ids of one (unit, block) per warp, in unit-major order: two words per lane,
+// then 64 nodes at a time, every lane a node.
+__global__ void __launch_bounds__(256)
+k_cut_write(const uint32_t *__restrict__ words, const uint32_t *__restrict__ part_off,
+            const int64_t *__restrict__ offsets, int64_t nblk, int64_t n_parts,
+            uint32_t *__restrict__ ids, int64_t cap, const int *err) {
+    if (*err) return;
+    const int lane = threadIdx.x & 31;
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (w >= n_parts) return;
+    const uint2 two = reinterpret_cast<const uint2 *>(words)[w * (kCutWords / 2) + lane];
+    const uint32_t n0 = __popc(two.x), n = n0 + __popc(two.y);
+    uint32_t incl = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+    if (total == 0) return;
+    const int64_t base = offsets[0] + part_off[w];
+    const uint32_t excl = incl - n, lt = lanemask_lt();
+    // nothing past the caller's capacity (an earlier slice of a call that exceeds it)
+    const uint32_t room = (uint32_t)min(max(cap - base, (int64_t)0), (int64_t)total);
+    uint32_t *out = ids + base;
+    const uint32_t node0 = (uint32_t)(w % nblk) * kCutPart + lane;
+#pragma unroll 4
+    for (int j = 0; j < 32; ++j) {
+        const uint32_t x = __shfl_sync(0xffffffffu, two.x, j), y = __shfl_sync(0xffffffffu, two.y, j);
+        const uint32_t e = __shfl_sync(0xffffffffu, excl, j);
+        const uint32_t px = e + __popc(x & lt), py = e + __popc(x) + __popc(y & lt);
+        if ((x >> lane & 1u) && px < room) out[px] = node0 + 64 * j;
+        if ((y >> lane & 1u) && py < room) out[py] = node0 + 64 * j + 32;
     }
 }
 
-void launch_cut_blocked(bool write, const float4 *box_lo, const float4 *box_hi, int64_t n_nodes,
-                        const DevCamera *cams, const CutCam *ccams, int n_cams,
-                        uint32_t *part_vals, uint32_t *ids, int64_t cap, uint32_t *ticket,
-                        const int *err, int grid, cudaStream_t st) {
-    if (ccams) {
-        if (write)
-            k_cut_blocked<true, true><<<grid, kCutThreads, 0, st>>>(
-                box_lo, box_hi, n_nodes, cams, ccams, n_cams, part_vals, ids, cap, ticket, err);
-        else
-            k_cut_blocked<false, true><<<grid, kCutThreads, 0, st>>>(
-                box_lo, box_hi, n_nodes, cams, ccams, n_cams, part_vals, ids, cap, ticket, err);
-    } else if (write) {
-        k_cut_blocked<true, false><<<grid, kCutThreads, 0, st>>>(
-            box_lo, box_hi, n_nodes, cams, ccams, n_cams, part_vals, ids, cap, ticket, err);
-    } else {
-        k_cut_blocked<false, false><<<grid, kCutThreads, 0, st>>>(
-            box_lo, box_hi, n_nodes, cams, ccams, n_cams, part_vals, ids, cap, ticket, err);
+// offsets[i] of the units of one call's slice (int64, offsets[0] being where the
+// slice begins, 0 for the first one), and after the last slice the total.
+__global__ void k_cut_unit_offsets(const uint32_t *__restrict__ part_off,
+                                   const uint32_t *__restrict__ total, int64_t nblk, int n_units,
+                                   int first, int last, int64_t cap, int64_t *offsets,
+                                   uint32_t *__restrict__ counters, int *err) {
+    const int64_t base = first ? 0 : offsets[0];
+    __syncthreads();
+    for (int i = threadIdx.x; i <= n_units; i += blockDim.x) {
+        const int64_t v = base + (i < n_units ? part_off[(int64_t)i * nblk] : *total);
+        offsets[i] = v;
+        if (i == n_units && last) {
+            counters[CNT_CUT] = (uint32_t)v;
+            if (v > cap) latch_error(err, kErrCapacity);
+        }
     }
 }
 
-void launch_cut_cam_offsets(const uint32_t *part_off, const uint32_t *total, int64_t nblk,
-                            int n_cams, int64_t cap, int64_t *offsets, uint32_t *counters,
-                            int *err, cudaStream_t st) {
-    k_cut_cam_offsets<<<(n_cams + 256) / 256, 256, 0, st>>>(part_off, total, nblk, n_cams, cap,
-                                                            offsets, counters, err);
+int64_t cut_words_per_unit(int64_t n_nodes) {
+    return (n_nodes + kCutPart - 1) / kCutPart * kCutWords;
+}
+
+template <bool kFrustum, bool kGroups>
+static void launch_masks(int c, const float4 *box_lo, const float4 *box_hi, int64_t n_nodes,
+                         const CutCam *cams, const int32_t *group_begin, const CutChunk *chunks,
+                         int n_chunks, uint32_t *words, uint32_t *counts, const int *err,
+                         cudaStream_t st) {
+    const unsigned grid = (unsigned)((n_nodes + kCutPart - 1) / kCutPart * n_chunks);
+    if (c <= 8)
+        k_cut_masks<kFrustum, kGroups, 8><<<grid, kCutThreads, 0, st>>>(
+            box_lo, box_hi, n_nodes, cams, group_begin, chunks, n_chunks, words, counts, err);
+    else if (c <= 16)
+        k_cut_masks<kFrustum, kGroups, 16><<<grid, kCutThreads, 0, st>>>(
+            box_lo, box_hi, n_nodes, cams, group_begin, chunks, n_chunks, words, counts, err);
+    else
+        k_cut_masks<kFrustum, kGroups, 32><<<grid, kCutThreads, 0, st>>>(
+            box_lo, box_hi, n_nodes, cams, group_begin, chunks, n_chunks, words, counts, err);
+}
+
+void launch_cut_masks(bool frustum, bool groups, int c, const float4 *box_lo,
+                      const float4 *box_hi, int64_t n_nodes, const CutCam *cams,
+                      const int32_t *group_begin, const CutChunk *chunks, int n_chunks,
+                      uint32_t *words, uint32_t *counts, const int *err, cudaStream_t st) {
+    auto go = [&](auto f) {
+        f(c, box_lo, box_hi, n_nodes, cams, group_begin, chunks, n_chunks, words, counts, err, st);
+    };
+    if (frustum) groups ? go(launch_masks<true, true>) : go(launch_masks<true, false>);
+    else groups ? go(launch_masks<false, true>) : go(launch_masks<false, false>);
+}
+
+void launch_cut_write(const uint32_t *words, const uint32_t *part_off, const uint32_t *total,
+                      int64_t n_nodes, int n_units, bool first, bool last, int64_t cap,
+                      uint32_t *ids, int64_t *offsets, uint32_t *counters, int *err,
+                      cudaStream_t st) {
+    const int64_t nblk = (n_nodes + kCutPart - 1) / kCutPart, n_parts = nblk * n_units;
+    k_cut_unit_offsets<<<1, 256, 0, st>>>(part_off, total, nblk, n_units, first, last, cap,
+                                          offsets, counters, err);
+    // writes nothing once the capacity is exceeded (latched above)
+    k_cut_write<<<(unsigned)((n_parts + 7) / 8), 256, 0, st>>>(words, part_off, offsets, nblk,
+                                                               n_parts, ids, cap, err);
 }
 
 void launch_cut(const SceneDev &sc, const DevCamera *cams, int n_cams, uint32_t *ids, int64_t cap,

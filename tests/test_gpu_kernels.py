@@ -101,3 +101,40 @@ def test_slice_boxes_of_all_sizes(R, cell, nx, ny, nz):
     near = np.abs(want - g.threshold) <= 1e-3
     assert np.array_equal(occ[~near], want_occ[~near])
     assert (want > 0).any()
+
+
+@pytest.fixture(scope="module")
+def floor_views(small_floor):
+    from scenegen import walk_cameras
+    taus = np.random.default_rng(3).uniform(0.0, 40.0, 110)
+    return walk_cameras(small_floor, 110, seed=8, width=320, height=240, taus=taus)
+
+
+# record_capacity: 2^22 holds every mask word of a call, 2^10 those of five cameras of
+# this scene (calls cut in slices), 2^7 none (single-pass kernels)
+@pytest.mark.parametrize("records", [1 << 22, 1 << 10, 1 << 7])
+def test_cuts_by_masks_equal_single_pass_cuts(small_floor, floor_views, records):
+    from paper_2603_15186_gb300 import Renderer
+    R = Renderer(cut_capacity=1 << 22, record_capacity=records, pair_capacity=1 << 20)
+    R.load_scene(small_floor)
+    cams = floor_views
+
+    def lists(ids, off):
+        off = off.cpu().numpy()
+        return np.split(ids[:off[-1]].cpu().numpy(), off[1:-1])
+
+    plain = [lists(*R.select_cut([c]))[0] for c in cams[:70]]
+    for n in (4, 5, 8, 9, 16, 17, 32, 33, 70):
+        got = lists(*R.select_cut(cams[:n]))
+        assert len(got) == n and all(np.array_equal(a, b) for a, b in zip(got, plain)), n
+    rng = np.random.default_rng(2)
+    for frustum, guard in ((True, 0.0), (True, 24.0), (False, 0.0)):
+        for sizes in ([1] * 40, [4], [3, 5], [7, 9, 1], [32, 1, 31], list(rng.integers(1, 20, 7))):
+            n = int(sum(sizes))
+            gb = [0] + list(np.cumsum(sizes))
+            got = lists(*R.select_cut_shared(cams[:n], gb, frustum, guard))
+            # a group of 33 sends the whole call to the single-pass kernel
+            want = lists(*R.select_cut_shared(cams[:n + 33], gb + [n + 33], frustum, guard))[:-1]
+            assert all(np.array_equal(a, b) for a, b in zip(got, want)), (frustum, guard, sizes)
+            assert any(len(a) for a in got)
+    R.close()
