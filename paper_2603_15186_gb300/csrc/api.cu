@@ -304,6 +304,8 @@ ngs_status ensure_work(ngs_ctx *c) {
     sw = std::max<int64_t>(sw, (std::max(w.rec_cap, w.pair_cap) + sort_partition() - 1) /
                                    sort_partition() * 256);
     sw = std::max<int64_t>(sw, (w.rec_cap + scan_partition() - 1) / scan_partition());
+    w.status_limit = sw;
+    sw = std::max<int64_t>(sw, scan_status_words(w.rec_cap));
     w.status_words = sw;
     ngs_status st = NGS_OK;
     auto A = [&](ngs_status s) { if (st == NGS_OK) st = s; };
@@ -514,7 +516,7 @@ ngs_status cut_by_masks(ngs_ctx *c, const std::vector<CutCam> &hc, const int32_t
         launch_cut_masks(frustum, group_begin != nullptr, lanes, sc.box_lo, sc.box_hi, sc.n,
                          c->cut_cams, c->cut_groups + u0, c->cut_chunks + first_chunk[k],
                          first_chunk[k + 1] - first_chunk[k], words, c->cut_counts, w.err, st);
-        const int64_t np = nblk * nu, sparts = (np + scan_partition() - 1) / scan_partition();
+        const int64_t np = nblk * nu, sparts = scan_parts(np);
         launch_scan_u32(c->cut_counts, c->cut_poff, nullptr, np, c->cut_off32,
                         w.counters + TK_SCAN, w.status, w.epoch, 0, w.err,
                         (int)std::min<int64_t>(sparts, c->grid_scan), st);
@@ -658,11 +660,11 @@ void enqueue_batched(ngs_ctx *c, const SubBatch &sb, int sb_index, cudaStream_t 
 
 int kernels_of(const SubBatch &sb, bool batched, bool order) {
     // epoch bump, live partitions, fused cut + preprocess, partition scan and
-    // key gather (which also counts the depth histograms); depth sort (digit
-    // scan, 4 passes); pair offsets, duplication; tile sort (digit scan and
-    // passes, the last one writing the tile ranges) or, with a single tile,
-    // the ranges kernel; compositing; and in the batched path the stats copy
-    return 5 + 5 + 2 + (sb.tile_passes > 0 ? 1 + sb.tile_passes : 1) + 1 + (batched ? 1 : 0) +
+    // key gather (which also counts the depth histograms); depth sort (4
+    // passes); pair offsets, duplication; tile sort (the last pass writing the
+    // tile ranges) or, with a single tile, the ranges kernel; compositing; and
+    // in the batched path the stats copy
+    return 5 + 4 + 2 + std::max(sb.tile_passes, 1) + 1 + (batched ? 1 : 0) +
            (batched && order ? 1 : 0);
 }
 
@@ -764,8 +766,7 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
         da.hist_ready = true;       // counted by the key gather
         launch_sort(da, std::min(gsort_v, c->grid_sort32), st);
         eo += 4;
-        const int gscan = std::max<int64_t>(1, ((int64_t)n_vis + scan_partition() - 1) /
-                                                   scan_partition());
+        const int gscan = (int)std::max<int64_t>(1, scan_parts(n_vis));
         CK(cudaMemsetAsync(w.hist, 0, sizeof(uint32_t) * 256 * 3, st));
         launch_pair_offsets(w.rect, w.didx[0], w.counters + CNT_VIS, w.poff, w.counters,
                             w.pair_cap, w.counters + TK_SCAN, w.status, w.epoch, eo++, w.err,
@@ -1744,7 +1745,7 @@ NGS_API ngs_status ngs_sort_pairs(ngs_ctx *c, void *d_keys, uint32_t *d_vals, in
     ngs_status s = ensure_work(c);
     if (s != NGS_OK) return s;
     const int64_t parts = (n + sort_partition() - 1) / sort_partition();
-    if (parts * 256 > c->w.status_words) return NGS_ERR_CAPACITY;
+    if (parts * 256 > c->w.status_limit) return NGS_ERR_CAPACITY;
     if (n > c->sort_tmp_cap) {
         dfree(c->sort_tmp_keys);
         dfree(c->sort_tmp_vals);
@@ -1789,7 +1790,7 @@ NGS_API ngs_status ngs_scan_u32(ngs_ctx *c, const uint32_t *d_in, uint32_t *d_ou
     ngs_status s = ensure_work(c);
     if (s != NGS_OK) return s;
     const int64_t parts = (n + scan_partition() - 1) / scan_partition();
-    if (parts > c->w.status_words) return NGS_ERR_CAPACITY;
+    if (parts > c->w.status_limit) return NGS_ERR_CAPACITY;
     if ((s = epoch_guard(c, st, kEpochStride)) != NGS_OK) return s;
     CK(cudaMemsetAsync(c->w.counters, 0, N_COUNTERS * sizeof(uint32_t), st));
     k_bump_epoch<<<1, 1, 0, st>>>(c->w.epoch, kEpochStride);
@@ -1798,7 +1799,7 @@ NGS_API ngs_status ngs_scan_u32(ngs_ctx *c, const uint32_t *d_in, uint32_t *d_ou
         return NGS_OK;
     }
     launch_scan_u32(d_in, d_out, nullptr, n, d_total, c->w.counters + TK_SCAN, c->w.status,
-                    c->w.epoch, 0, c->w.err, (int)std::min<int64_t>(parts, c->grid_scan), st);
+                    c->w.epoch, 0, c->w.err, (int)std::min<int64_t>(scan_parts(n), c->grid_scan), st);
     CK(cudaGetLastError());
     return NGS_OK;
 }

@@ -14,6 +14,8 @@
 //   4. K6 finds each tile's [first, end) in the sorted pair array.
 // The radix passes on the depth digits thus run over Gaussians, not over
 // pairs, which is where the bytes are saved.
+#include <algorithm>
+
 #include "ngs_internal.cuh"
 
 namespace ngs {
@@ -21,8 +23,19 @@ namespace ngs {
 constexpr int kScanThreads = 256;
 constexpr int kScanItems = 8;
 constexpr int kScanPart = kScanThreads * kScanItems;
+// inputs of up to kScanFew elements (two partitions per SM at most) take partitions of
+// 2 elements per thread
+constexpr int kScanItemsFew = 2;
+constexpr int64_t kScanFew = 152 * 2048;
 
 int scan_partition() { return kScanPart; }
+int64_t scan_parts(int64_t n) {
+    const int64_t part = n <= kScanFew ? kScanThreads * kScanItemsFew : kScanPart;
+    return (n + part - 1) / part;
+}
+int64_t scan_status_words(int64_t n) {
+    return std::max(scan_parts(n), scan_parts(std::min(n, kScanFew)));
+}
 
 // K4 works on chunks of kDupChunk consecutive pairs
 constexpr int kDupThreads = 256;
@@ -35,13 +48,14 @@ __device__ __forceinline__ uint32_t rect_area(const uint2 r) {
     return (u.x1 - u.x0 + 1u) * (u.y1 - u.y0 + 1u);
 }
 
-// Block-wide exclusive scan of kScanItems values per thread (blocked layout:
-// thread t holds items t*kScanItems .. +kScanItems-1); returns the block total.
-__device__ __forceinline__ uint32_t block_scan(uint32_t v[kScanItems], uint32_t *s_warp) {
+// Block-wide exclusive scan of ITEMS values per thread (blocked layout:
+// thread t holds items t*ITEMS .. +ITEMS-1); returns the block total.
+template <int ITEMS>
+__device__ __forceinline__ uint32_t block_scan(uint32_t v[ITEMS], uint32_t *s_warp) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t sum = 0;
 #pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
+    for (int i = 0; i < ITEMS; ++i) {
         const uint32_t t = v[i];
         v[i] = sum;
         sum += t;
@@ -62,7 +76,7 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t v[kScanItems], uint32_t 
     }
     const uint32_t off = wbase + incl - sum;
 #pragma unroll
-    for (int i = 0; i < kScanItems; ++i) v[i] += off;
+    for (int i = 0; i < ITEMS; ++i) v[i] += off;
     return total;
 }
 
@@ -113,38 +127,44 @@ __device__ __forceinline__ void tile_digits_add(TileDigits &H, uint32_t k0, uint
     }
 }
 
-template <bool kGather>
-__global__ void __launch_bounds__(kScanThreads, 4)
-k_scan(const uint32_t *__restrict__ in, const uint2 *__restrict__ rect,
-       const uint32_t *__restrict__ idx, uint32_t *out, const uint32_t *n_dev, int64_t n_host,
-       uint32_t *total_out, int64_t total_cap, uint32_t *ticket, uint64_t *status,
-       const uint32_t *epoch_ptr, uint32_t epoch_off, int *err, uint32_t *chunk_first,
-       int64_t chunk_cap, uint2 *__restrict__ rect_out, const DevCamera *__restrict__ cams,
-       uint32_t *hist, int passes) {
-    __shared__ uint32_t s_warp[kScanThreads / 32];
-    __shared__ uint32_t s_val[kScanPart + kScanPart / 32];
-    __shared__ uint32_t s_part, s_prev;
-    __shared__ TileDigits s_td;
-    if (*err) return;
+// A chain of at most this many partitions (they all run at once) is looked back over
+// by a warp, 32 partitions per round trip; on longer chains, where a look-back ends
+// after a window or two, one thread took 8% less time than a warp.
+constexpr int kScanShortChain = 1024;
+// Rects of up to this many tile rows are counted by their own thread; a warp that has
+// a larger one deals all its rows to its lanes. 260k records of a 720p view on
+// 16-pixel tiles (25 tiles each, up to 45 rows): 73 us for the kernel with a loop per
+// thread and the chain walked by one thread, 61 us so, and 38 us with partitions of 512
+// records (kScanFew), as the nearest 2048 records alone hold a twentieth of the rows.
+constexpr uint32_t kScanFewRows = 4;
+
+struct ScanSmem {
+    uint32_t warp[kScanThreads / 32];
+    uint32_t val[kScanPart + kScanPart / 32];
+    uint32_t part, prev;
+    TileDigits td;
+};
+
+// The partitions of ITEMS elements per thread, taken from the ticket.
+template <bool kGather, int ITEMS>
+__device__ __forceinline__ void
+scan_partitions(ScanSmem &S, const uint32_t *__restrict__ in, const uint2 *__restrict__ rect,
+           const uint32_t *__restrict__ idx, uint32_t *out, int64_t n, uint32_t *total_out,
+           int64_t total_cap, uint32_t *ticket, uint64_t *status, uint32_t epoch, int *err,
+           uint32_t *chunk_first, int64_t chunk_cap, uint2 *__restrict__ rect_out,
+           const DevCamera *__restrict__ cams, const uint32_t *hist, int passes) {
+    constexpr int PART = kScanThreads * ITEMS;
     const int tid = threadIdx.x;
-    if (kGather && hist) {
-        for (int i = tid; i < (int)(sizeof(TileDigits) / 4); i += kScanThreads)
-            reinterpret_cast<uint32_t *>(&s_td)[i] = 0;
-        __syncthreads();
-    }
-    const int64_t n = n_dev ? (int64_t)*n_dev : n_host;
-    const int64_t nparts = (n + kScanPart - 1) / kScanPart;
-    const uint32_t epoch = *epoch_ptr + epoch_off;
-    if (nparts == 0 && blockIdx.x == 0 && tid == 0 && total_out) *total_out = 0;
+    const int64_t nparts = (n + PART - 1) / PART;
     for (;;) {
-        if (tid == 0) s_part = atomicAdd(ticket, 1u);
+        if (tid == 0) S.part = atomicAdd(ticket, 1u);
         __syncthreads();
-        const int64_t part = s_part;
+        const int64_t part = S.part;
         if (part >= nparts) break;
-        const int64_t pbase = part * kScanPart;
+        const int64_t pbase = part * PART;
         // striped: element pbase + i * threads + tid
 #pragma unroll
-        for (int i = 0; i < kScanItems; ++i) {
+        for (int i = 0; i < ITEMS; ++i) {
             const int k = i * kScanThreads + tid;
             const int64_t j = pbase + k;
             uint32_t v = 0;
@@ -157,56 +177,95 @@ k_scan(const uint32_t *__restrict__ in, const uint2 *__restrict__ rect,
                     v = in[j];
                 }
             }
-            s_val[scan_slot(k)] = v;
+            S.val[scan_slot(k)] = v;
         }
         __syncthreads();
-        // blocked: elements pbase + tid * kScanItems + i
-        uint32_t v[kScanItems], a[kScanItems];
+        // blocked: elements pbase + tid * ITEMS + i
+        uint32_t v[ITEMS], a[ITEMS];
 #pragma unroll
-        for (int i = 0; i < kScanItems; ++i) {
-            v[i] = s_val[scan_slot(tid * kScanItems + i)];
+        for (int i = 0; i < ITEMS; ++i) {
+            v[i] = S.val[scan_slot(tid * ITEMS + i)];
             a[i] = v[i];
         }
-        const uint32_t total = block_scan(v, s_warp);
-        if (tid == 0) {
+        const uint32_t total = block_scan<ITEMS>(v, S.warp);
+        if (tid < 32) {
             uint64_t *slot = status + part;
             uint32_t prev = 0;
-            if (part == 0) {
-                publish(slot, pack_status(kFlagPrefix, epoch, total));
-            } else {
-                publish(slot, pack_status(kFlagAgg, epoch, total));
-                look_back(status, part, 1, epoch, &prev, err);
-                publish(slot, pack_status(kFlagPrefix, epoch, prev + total));
+            if (tid == 0)
+                publish(slot, pack_status(part == 0 ? kFlagPrefix : kFlagAgg, epoch, total));
+            if (part > 0) {
+                if (nparts <= kScanShortChain) {
+                    look_back_warp(status, part, epoch, &prev, err);
+                    if (tid == 0) publish(slot, pack_status(kFlagPrefix, epoch, prev + total));
+                } else if (tid == 0) {
+                    look_back(status, part, 1, epoch, &prev, err);
+                    publish(slot, pack_status(kFlagPrefix, epoch, prev + total));
+                }
             }
-            s_prev = prev;
-            // a running total that crosses 2^32 wraps in the partition where it happens
-            if (total_cap >= 0 && prev + total < prev) latch_error(err, kErrCapacity);
-            if (part == nparts - 1) {
-                const uint64_t all = (uint64_t)prev + total;
-                if (total_out) *total_out = (uint32_t)all;
-                if (total_cap >= 0 && (int64_t)all > total_cap) latch_error(err, kErrCapacity);
+            if (tid == 0) {
+                S.prev = prev;
+                // a running total that crosses 2^32 wraps in the partition where it happens
+                if (total_cap >= 0 && prev + total < prev) latch_error(err, kErrCapacity);
+                if (part == nparts - 1) {
+                    const uint64_t all = (uint64_t)prev + total;
+                    if (total_out) *total_out = (uint32_t)all;
+                    if (total_cap >= 0 && (int64_t)all > total_cap) latch_error(err, kErrCapacity);
+                }
             }
         }
         if (kGather && hist && tid >= 32) {
             // while warp 0 looks back, the other warps count the tile digits
             // of the partition's Gaussians (each its tile keys, rectangle row
             // by row), reading back the depth-ordered rects just written
+            const int lane = tid & 31;
 #pragma unroll 1
-            for (int k = tid - 32; k < kScanPart && pbase + k < n; k += kScanThreads - 32) {
-                const RectU u = unpack_rect(rect_out[pbase + k]);
-                const uint32_t tb = cams[u.cam].tile_base;
-                const uint32_t tsx = (uint32_t)cams[u.cam].tiles_x;
-                for (uint32_t ty = u.y0; ty <= u.y1; ++ty)
-                    tile_digits_add(s_td, tb + ty * tsx + u.x0, u.x1 - u.x0 + 1u, passes);
+            for (int k0 = tid - lane - 32; k0 < PART && pbase + k0 < n;
+                 k0 += kScanThreads - 32) {
+                const int k = k0 + lane;
+                uint32_t key = 0, tsx = 0, w = 0, h = 0;   // first tile key, row stride, size
+                if (pbase + k < n) {
+                    const RectU u = unpack_rect(rect_out[pbase + k]);
+                    tsx = (uint32_t)cams[u.cam].tiles_x;
+                    key = cams[u.cam].tile_base + u.y0 * tsx + u.x0;
+                    w = u.x1 - u.x0 + 1u;
+                    h = u.y1 - u.y0 + 1u;
+                }
+                if (__reduce_max_sync(0xffffffffu, h) <= kScanFewRows) {
+                    for (uint32_t y = 0; y < h; ++y) tile_digits_add(S.td, key + y * tsx, w, passes);
+                    continue;
+                }
+                // rects of many rows (a view close to its Gaussians): the rows of the
+                // 32 rects end to end, one per lane
+                uint32_t incl = h;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += t;
+                }
+                const uint32_t rows = __shfl_sync(0xffffffffu, incl, 31);
+                // lanes past the last rect (h = 0) start at `rows`: never reached
+                const uint32_t start = incl - h;
+                for (uint32_t c0 = 0; c0 < rows; c0 += 32) {
+                    const uint32_t before = __popc(__ballot_sync(0xffffffffu, start <= c0)) - 1u;
+                    const uint32_t off = start - c0;
+                    const uint32_t marks =
+                        __reduce_or_sync(0xffffffffu, start > c0 && off < 32u ? 1u << off : 0u);
+                    const int src = (int)(before + __popc(marks & (lanemask_lt() | 1u << lane)));
+                    const uint32_t sk = __shfl_sync(0xffffffffu, key, src),
+                                   st = __shfl_sync(0xffffffffu, tsx, src),
+                                   sw = __shfl_sync(0xffffffffu, w, src),
+                                   ss = __shfl_sync(0xffffffffu, start, src);
+                    if (c0 + lane < rows) tile_digits_add(S.td, sk + (c0 + lane - ss) * st, sw, passes);
+                }
             }
         }
         __syncthreads();
-        const uint32_t prev = s_prev;
-        const int64_t base = pbase + (int64_t)tid * kScanItems;
+        const uint32_t prev = S.prev;
+        const int64_t base = pbase + (int64_t)tid * ITEMS;
 #pragma unroll
-        for (int i = 0; i < kScanItems; ++i) {
+        for (int i = 0; i < ITEMS; ++i) {
             const uint32_t lo = prev + v[i];
-            s_val[scan_slot(tid * kScanItems + i)] = lo;
+            S.val[scan_slot(tid * ITEMS + i)] = lo;
             const int64_t j = base + i;
             if (kGather && a[i] && j < n) {
                 const uint64_t hi = (uint64_t)lo + a[i];
@@ -217,33 +276,63 @@ k_scan(const uint32_t *__restrict__ in, const uint2 *__restrict__ rect,
         }
         __syncthreads();
 #pragma unroll
-        for (int i = 0; i < kScanItems; ++i) {
+        for (int i = 0; i < ITEMS; ++i) {
             const int k = i * kScanThreads + tid;
-            if (pbase + k < n) out[pbase + k] = s_val[scan_slot(k)];
+            if (pbase + k < n) out[pbase + k] = S.val[scan_slot(k)];
         }
         __syncthreads();
     }
+}
+
+template <bool kGather>
+__global__ void __launch_bounds__(kScanThreads, 5)
+k_scan(const uint32_t *__restrict__ in, const uint2 *__restrict__ rect,
+       const uint32_t *__restrict__ idx, uint32_t *out, const uint32_t *n_dev, int64_t n_host,
+       uint32_t *total_out, int64_t total_cap, uint32_t *ticket, uint64_t *status,
+       const uint32_t *epoch_ptr, uint32_t epoch_off, int *err, uint32_t *chunk_first,
+       int64_t chunk_cap, uint2 *__restrict__ rect_out, const DevCamera *__restrict__ cams,
+       uint32_t *hist, int passes, uint32_t *done) {
+    __shared__ ScanSmem S;
+    if (*err) return;
+    const int tid = threadIdx.x;
+    if (kGather && hist) {
+        for (int i = tid; i < (int)(sizeof(TileDigits) / 4); i += kScanThreads)
+            reinterpret_cast<uint32_t *>(&S.td)[i] = 0;
+        __syncthreads();
+    }
+    const int64_t n = n_dev ? (int64_t)*n_dev : n_host;
+    const uint32_t epoch = *epoch_ptr + epoch_off;
+    if (n == 0 && blockIdx.x == 0 && tid == 0 && total_out) *total_out = 0;
+    if (n <= kScanFew)
+        scan_partitions<kGather, kScanItemsFew>(S, in, rect, idx, out, n, total_out, total_cap,
+                                                ticket, status, epoch, err, chunk_first,
+                                                chunk_cap, rect_out, cams, hist, passes);
+    else
+        scan_partitions<kGather, kScanItems>(S, in, rect, idx, out, n, total_out, total_cap, ticket,
+                                             status, epoch, err, chunk_first, chunk_cap, rect_out,
+                                             cams, hist, passes);
     if (kGather && hist) {
         // the CTA's digit counts into hist: pass 0 from the prefix sum of its
         // difference array (one digit per thread), passes 1, 2 directly
         static_assert(kScanThreads == 256, "one thread per digit");
         const int lane = tid & 31, warp = tid >> 5;
         __syncthreads();
-        uint32_t x = s_td.d0[tid];
+        uint32_t x = S.td.d0[tid];
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const uint32_t t = __shfl_up_sync(0xffffffffu, x, o);
             if (lane >= o) x += t;
         }
-        if (lane == 31) s_warp[warp] = x;
+        if (lane == 31) S.warp[warp] = x;
         __syncthreads();
-        for (int w = 0; w < warp; ++w) x += s_warp[w];
-        const uint32_t c0 = x + s_td.full;
+        for (int w = 0; w < warp; ++w) x += S.warp[w];
+        const uint32_t c0 = x + S.td.full;
         if (c0) atomicAdd(&hist[tid], c0);
         for (int q = 1; q < passes; ++q) {
-            const uint32_t v = s_td.hh[q - 1][tid];
+            const uint32_t v = S.td.hh[q - 1][tid];
             if (v) atomicAdd(&hist[q * 256 + tid], v);
         }
+        digit_scan_by_last(hist, passes, done, &S.part, S.warp);
     }
 }
 
@@ -252,7 +341,8 @@ void launch_scan_u32(const uint32_t *in, uint32_t *out, const uint32_t *n_dev, i
                      uint32_t epoch_off, int *err, int grid, cudaStream_t st) {
     k_scan<false><<<grid, kScanThreads, 0, st>>>(in, nullptr, nullptr, out, n_dev, n_host, total,
                                                  -1, ticket, status, epoch, epoch_off, err,
-                                                 nullptr, 0, nullptr, nullptr, nullptr, 0);
+                                                 nullptr, 0, nullptr, nullptr, nullptr, 0,
+                                                 nullptr);
 }
 
 void launch_pair_offsets(const uint2 *rect, const uint32_t *sorted_idx, const uint32_t *n_vis,
@@ -264,7 +354,8 @@ void launch_pair_offsets(const uint2 *rect, const uint32_t *sorted_idx, const ui
                                                 counters + CNT_PAIRS, pair_cap, ticket, status,
                                                 epoch, epoch_off, err, chunk_first,
                                                 dup_chunks(pair_cap), rect_sorted, cams,
-                                                passes > 0 ? hist : nullptr, passes);
+                                                passes > 0 ? hist : nullptr, passes,
+                                                counters + CNT_DONE + 2);
 }
 
 // K4: the pair array is cut into chunks of kDupChunk pairs, so every CTA

@@ -938,16 +938,17 @@ k_part_scan(const uint32_t *__restrict__ vis_count, int n_cams, int64_t nblk,
 // of its visible Gaussians (skipping holes) and writes their record indices at
 // the partition's dense position. On the
 // way it counts the digit histograms of the four 8-bit passes of the depth
-// sort into hist[4][256] (zeroed beforehand): positive float depths share
+// sort into hist[4][256] (zeroed beforehand; the last CTA scans them): positive float depths share
 // their high digits, so a warp whose keys agree on a digit adds its count once
 // instead of contending on one shared-memory counter.
 __global__ void __launch_bounds__(256)
 k_part_gather(const uint32_t *__restrict__ part_list, int n_cams, int64_t nblk,
               const uint2 *__restrict__ part_info, const uint32_t *__restrict__ part_pos,
               const uint32_t *__restrict__ dkey_sparse, uint32_t *__restrict__ dkey,
-              uint32_t *__restrict__ didx, const uint32_t *counters, int64_t cap,
+              uint32_t *__restrict__ didx, uint32_t *counters, int64_t cap,
               uint32_t *hist, const int *err) {
     __shared__ uint32_t s_h[4][256];
+    __shared__ uint32_t s_last, s_warp[8];
     if (*err) return;
     const int tid = threadIdx.x;
     for (int i = tid; i < 4 * 256; i += blockDim.x) (&s_h[0][0])[i] = 0;
@@ -1011,6 +1012,7 @@ k_part_gather(const uint32_t *__restrict__ part_list, int n_cams, int64_t nblk,
         const uint32_t v = (&s_h[0][0])[i];
         if (v) atomicAdd(&hist[i], v);
     }
+    digit_scan_by_last(hist, 4, counters + CNT_DONE + 1, &s_last, s_warp);
 }
 
 template <bool kBlend>

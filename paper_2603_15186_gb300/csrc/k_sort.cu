@@ -21,6 +21,8 @@
 // Partitions are 8192 keys (32-bit) or 4096 (64-bit) over 512 threads: long
 // runs per digit keep the scattered writes close to whole sectors, and values
 // are read only once the keys are ranked, which keeps two CTAs resident.
+#include <algorithm>
+
 #include "ngs_internal.cuh"
 
 namespace ngs {
@@ -40,23 +42,38 @@ __device__ __forceinline__ uint32_t digit_of(K key, int shift, uint32_t mask) {
     return (uint32_t)(key >> shift) & mask;
 }
 
+// kUp keys per thread are requested at once, eight CTAs per SM: 12.3M 32-bit keys in
+// 28 us (84 us with one key at a time and two CTAs per SM, a chain of memory round
+// trips). The CTA that is done last scans the digits.
+constexpr int kUp = 8;
+
 template <typename K>
 __global__ void __launch_bounds__(kSortThreads)
 k_upsweep(const K *__restrict__ keys, const uint32_t *n_dev, int64_t n_host, int begin_bit,
-          int end_bit, uint32_t *__restrict__ hist, const int *err) {
+          int end_bit, uint32_t *hist, uint32_t *done, const int *err) {
     __shared__ uint32_t s_h[kMaxPasses][kRadix];
+    __shared__ uint32_t s_last, s_warp[kSortWarps];
     if (*err) return;
     const int passes = (end_bit - begin_bit + 7) / 8;
     for (int i = threadIdx.x; i < passes * kRadix; i += kSortThreads) (&s_h[0][0])[i] = 0;
     __syncthreads();
     const int64_t n = n_dev ? (int64_t)*n_dev : n_host;
-    for (int64_t i = (int64_t)blockIdx.x * kSortThreads + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * kSortThreads) {
-        const K k = keys[i];
-        for (int p = 0; p < passes; ++p) {
-            const int sh = begin_bit + 8 * p;
-            const int bits = min(8, end_bit - sh);
-            atomicAdd(&s_h[p][digit_of(k, sh, (1u << bits) - 1u)], 1u);
+    for (int64_t i0 = (int64_t)blockIdx.x * kSortThreads * kUp + threadIdx.x; i0 < n;
+         i0 += (int64_t)gridDim.x * kSortThreads * kUp) {
+        K k[kUp];
+#pragma unroll
+        for (int u = 0; u < kUp; ++u) {
+            const int64_t i = i0 + u * kSortThreads;
+            k[u] = i < n ? keys[i] : (K)0;
+        }
+#pragma unroll
+        for (int u = 0; u < kUp; ++u) {
+            if (i0 + u * kSortThreads >= n) break;
+            for (int p = 0; p < passes; ++p) {
+                const int sh = begin_bit + 8 * p;
+                const int bits = min(8, end_bit - sh);
+                atomicAdd(&s_h[p][digit_of(k[u], sh, (1u << bits) - 1u)], 1u);
+            }
         }
     }
     __syncthreads();
@@ -64,26 +81,7 @@ k_upsweep(const K *__restrict__ keys, const uint32_t *n_dev, int64_t n_host, int
         const uint32_t v = (&s_h[0][0])[i];
         if (v) atomicAdd(&hist[i], v);
     }
-}
-
-// hist[p][d] -> exclusive prefix over d (one block per pass)
-__global__ void k_digit_scan(uint32_t *hist, const int *err) {
-    __shared__ uint32_t s_w[kSortWarps];
-    if (*err) return;
-    uint32_t *h = hist + blockIdx.x * kRadix;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t v = h[tid];
-    uint32_t incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-    }
-    if (lane == 31) s_w[warp] = incl;
-    __syncthreads();
-    uint32_t wbase = 0;
-    for (int w = 0; w < warp; ++w) wbase += s_w[w];
-    h[tid] = wbase + incl - v;
+    digit_scan_by_last(hist, passes, done, &s_last, s_warp);
 }
 
 // Partition shape per key width: 512 threads; 16 (32-bit keys) or 8 (64-bit
@@ -295,10 +293,12 @@ static void launch_sort_t(const SortArgs &a, int grid, cudaStream_t st) {
     const size_t smem = sizeof(SortSmem<K>);
     if (!a.hist_ready) {
         cudaMemsetAsync(a.hist, 0, sizeof(uint32_t) * kRadix * passes, st);
-        k_upsweep<K><<<grid, kSortThreads, 0, st>>>((const K *)a.keys[0], a.n_dev, a.n_host,
-                                                    a.begin_bit, a.end_bit, a.hist, a.err);
+        const int ugrid = (int)std::max<int64_t>(
+            1, std::min<int64_t>((a.n_max + kSortThreads * kUp - 1) / (kSortThreads * kUp), 8 * 152));
+        k_upsweep<K><<<ugrid, kSortThreads, 0, st>>>((const K *)a.keys[0], a.n_dev, a.n_host,
+                                                     a.begin_bit, a.end_bit, a.hist,
+                                                     a.tickets + kMaxPasses, a.err);
     }
-    k_digit_scan<<<passes, kRadix, 0, st>>>(a.hist, a.err);
     if (a.hook) a.hook(a.hook_user, 0);
     for (int p = 0; p < passes; ++p) {
         const int src = p & 1, dst = src ^ 1;

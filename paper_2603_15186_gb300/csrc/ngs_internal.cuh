@@ -272,6 +272,69 @@ __device__ __forceinline__ bool look_back(const uint64_t *status, int64_t part, 
     return true;
 }
 
+// Exclusive prefix over the 256 digits of each of `passes` histograms, by the CTA (of
+// at least 256 threads) that added its counts last; every CTA of the launch calls it
+// after its own. done: one word, zero before the launch. s_last, s_warp: shared, 1 and 8
+// words.
+__device__ __forceinline__ void digit_scan_by_last(uint32_t *hist, int passes, uint32_t *done,
+                                                   uint32_t *s_last, uint32_t *s_warp) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) *s_last = atomicAdd(done, 1u) + 1u == gridDim.x;
+    __syncthreads();
+    if (!*s_last) return;
+    __threadfence();
+    for (int p = 0; p < passes; ++p) {
+        uint32_t v = 0, incl = 0;
+        if (tid < 256) {
+            incl = v = __ldcg(hist + p * 256 + tid);
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
+            }
+            if (lane == 31) s_warp[tid >> 5] = incl;
+        }
+        __syncthreads();
+        if (tid < 256) {
+            for (int w = 0; w < tid >> 5; ++w) incl += s_warp[w];
+            hist[p * 256 + tid] = incl - v;
+        }
+        __syncthreads();
+    }
+}
+
+// look_back by a whole warp (all lanes call it with the same arguments and get the
+// same result), 32 predecessors per round trip: for a short chain whose partitions
+// all run at once, where a look-back walks most of the chain.
+__device__ __forceinline__ bool look_back_warp(const uint64_t *status, int64_t part,
+                                               uint32_t epoch, uint32_t *excl, int *err) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t ep = epoch & kEpochMask;
+    uint32_t acc = 0, spins = 0;
+    for (int64_t j = part - 1; j >= 0;) {
+        // what lies before the first partition is an inclusive prefix of 0
+        const uint64_t w = j - lane >= 0 ? peek(status + (j - lane)) : pack_status(kFlagPrefix, ep, 0u);
+        const uint64_t flag = w & (3ull << 62);
+        const bool known = ((uint32_t)(w >> 32) & kEpochMask) == ep && flag != 0;
+        const uint32_t unknown = __ballot_sync(0xffffffffu, !known);
+        const uint32_t prefix = __ballot_sync(0xffffffffu, known && flag == kFlagPrefix);
+        const int n_known = unknown ? __ffs(unknown) - 1 : 32;
+        const int to = prefix ? __ffs(prefix) : 33;    // lanes up to the first prefix
+        acc += __reduce_add_sync(0xffffffffu, lane < min(n_known, to) ? (uint32_t)w : 0u);
+        if (to <= n_known) break;
+        j -= n_known;
+        if (unknown && ++spins > kSpinLimit) {
+            if (lane == 0) latch_error(err, kErrTimeout);
+            *excl = acc;
+            return false;
+        }
+    }
+    *excl = acc;
+    return true;
+}
+
 // ---------------------------------------------------------------------------
 // work-buffer bundle for one render sub-batch
 // ---------------------------------------------------------------------------
@@ -282,6 +345,7 @@ struct Work {
     uint32_t *epoch = nullptr;        // device epoch base, bumped per sub-batch
     uint64_t *status = nullptr;       // chained-scan words
     int64_t status_words = 0;
+    int64_t status_limit = 0;         // bounds the standalone sort and scan (<= status_words)
     int *err = nullptr;               // latched device error
     uint32_t *cut_ids = nullptr;      int64_t cut_cap = 0;
     uint32_t *cut_off = nullptr;      // [cams + 1]
@@ -320,7 +384,9 @@ constexpr int kWork64Words = 2 + 2 * kTailSlots;
 // ticket slots in Work::counters
 enum : int {
     CNT_CUT = 0, CNT_VIS = 1, CNT_PAIRS = 2, TK_CUT = 3, TK_PRE = 4, TK_SCAN = 5, TK_DUP = 6,
-    TK_SORT0 = 8,             // 8 .. 8 + 16: one ticket per sort pass
+    TK_SORT0 = 8,             // 8 .. 15: one ticket per sort pass (depth 4, tiles 3)
+    CNT_DONE = 16,            // CTAs done counting digits: a standalone sort's upsweep (at
+                              // its tickets + 8), the key gather, the offset scan
     CNT_ALLOC = 24,           // 24, 25: 64-bit record allocation counter
     CNT_LIVE = 26,            // live cut+preprocess partitions
     CNT_GROUPS = 27,          // groups of live partitions (same node block)
@@ -356,7 +422,8 @@ void launch_cutpre(const SceneDev &sc, const DevCamera *cams, int n_cams, void *
 int cutpre_partition_nodes();
 void cutpre_init_attributes();
 // dense depth keys (camera-major, node order) and their record indices for the
-// sort, and the depth sort's digit histograms in hist[4][256]; counters[CNT_VIS]
+// sort, and the exclusive prefixes of the depth sort's digit histograms in hist[4][256];
+// counters[CNT_VIS], [CNT_DONE + 1]
 void launch_gather_keys(const uint32_t *vis_count, int n_cams, const SceneDev &sc,
                         const uint2 *part_info, uint32_t *part_pos, const uint32_t *part_list,
                         const uint32_t *dkey_sparse, uint32_t *dkey, uint32_t *didx,
@@ -375,7 +442,7 @@ struct SortArgs {
     int key_bytes;
     int begin_bit, end_bit;
     bool vals_identity;       // first pass takes value = input index
-    bool hist_ready;          // hist already holds the digit counts (no upsweep)
+    bool hist_ready;          // hist already holds the digit counts' exclusive prefixes
     uint32_t *hist;           // [passes][256]
     // last pass: skip_last_keys writes the values only (the sorted keys are
     // not needed afterwards); a non-null ranges (32-bit tile keys only) also
@@ -383,7 +450,7 @@ struct SortArgs {
     // ~first, so zeroed entries mean "no pairs"), and implies skip_last_keys
     bool skip_last_keys;
     uint2 *ranges;
-    uint32_t *tickets;        // one per pass
+    uint32_t *tickets;        // one per pass; without hist_ready also tickets[8]
     uint64_t *status;
     const uint32_t *epoch;
     uint32_t epoch_off;
@@ -403,13 +470,16 @@ void launch_sort(const SortArgs &a, int grid, cudaStream_t st);
 void launch_scan_u32(const uint32_t *in, uint32_t *out, const uint32_t *n_dev, int64_t n_host,
                      uint32_t *total, uint32_t *ticket, uint64_t *status, const uint32_t *epoch,
                      uint32_t epoch_off, int *err, int grid, cudaStream_t st);
-int scan_partition();
+int scan_partition();                   // largest partition
+int64_t scan_parts(int64_t n);          // partitions of a scan of n elements
+int64_t scan_status_words(int64_t n);   // look-back words of scans of up to n elements
 
 // binning: tiles-touched scan over depth order (also the first record of every
 // pair chunk, chunk_first[dup_chunks(pair_cap)], and the rects in depth order
-// in rect_sorted); with hist, it also adds the digit counts
-// of the pairs' tile keys (camera tile base + row * tiles_x + column) for
-// `passes` 8-bit radix passes to hist[passes][256] (zeroed by the caller)
+// in rect_sorted); with passes, it also counts the digits of the pairs' tile
+// keys (camera tile base + row * tiles_x + column) for that many 8-bit radix
+// passes and leaves their exclusive prefixes in hist[passes][256] (zeroed by the
+// caller); counters[CNT_PAIRS], [CNT_DONE + 2]
 void launch_pair_offsets(const uint2 *rect, const uint32_t *sorted_idx, const uint32_t *n_vis,
                          uint32_t *poff, uint32_t *counters, int64_t pair_cap, uint32_t *ticket,
                          uint64_t *status, const uint32_t *epoch, uint32_t epoch_off, int *err,

@@ -46,7 +46,8 @@ constexpr size_t kOffVals = align256(kOffKeys + 8 * kStaticMaxPairs);   // alter
 constexpr size_t kOffStatus = align256(kOffVals + 4 * kStaticMaxPairs); // look-back words
 constexpr size_t kOffHist = align256(kOffStatus + 8 * 256 * kStaticParts);
 constexpr size_t kOffTickets = align256(kOffHist + 4 * 8 * 256);
-constexpr size_t kOffEpoch = align256(kOffTickets + 4 * 8);
+constexpr size_t kTickets = 9;   // one per pass, and the histogram's
+constexpr size_t kOffEpoch = align256(kOffTickets + 4 * kTickets);
 constexpr size_t kOffErr = align256(kOffEpoch + 4);       // error of the running call
 constexpr size_t kOffLatched = kOffErr + 4;                 // first error since the last query
 constexpr size_t kScratchBytes = align256(kOffLatched + 4);
@@ -133,7 +134,7 @@ extern "C" NGS_API ngs_status ngs_sort_pairs_static(void *d_keys, uint32_t *d_va
                 return NGS_ERR_CUDA;
         }
     }
-    if (cudaMemsetAsync(tickets, 0, 4 * 8, st) != cudaSuccess) return NGS_ERR_CUDA;
+    if (cudaMemsetAsync(tickets, 0, 4 * kTickets, st) != cudaSuccess) return NGS_ERR_CUDA;
     k_static_begin<<<1, 1, 0, st>>>(epoch, 32u, err, (int *)(base + kOffLatched));
     SortArgs a{};
     a.keys[0] = d_keys; a.keys[1] = base + kOffKeys;

@@ -138,3 +138,54 @@ def test_cuts_by_masks_equal_single_pass_cuts(small_floor, floor_views, records)
             assert all(np.array_equal(a, b) for a, b in zip(got, want)), (frustum, guard, sizes)
             assert any(len(a) for a in got)
     R.close()
+
+
+# one key into a second partition (4096 or 8192 keys), the keys that the histogram's
+# CTAs take at once (2048) and one more, several rounds of all its CTAs
+@pytest.mark.parametrize("key_bytes,n", [(4, 2048), (4, 2049), (4, 8193), (4, 311_297), (4, 6_000_001),
+                                         (8, 2049), (8, 4097), (8, 700_001)])
+def test_sort_histogram_sizes(R, key_bytes, n):
+    g = torch.Generator(device="cuda").manual_seed(n)
+    # few distinct high digits, as depths have
+    keys = torch.randint(0, 1 << 27, (n,), generator=g, device="cuda", dtype=torch.int64)
+    if key_bytes == 8:
+        keys |= torch.randint(0, 3, (n,), generator=g, device="cuda", dtype=torch.int64) << 40
+    else:
+        keys = keys.to(torch.int32)
+    vals = torch.arange(n, device="cuda", dtype=torch.int32)
+    want, order = torch.sort(keys, stable=True)
+    R.sort_pairs(keys, vals)
+    torch.cuda.synchronize()
+    assert torch.equal(keys, want) and torch.equal(vals, order.to(torch.int32))
+
+
+# partitions of 512 elements up to 152 * 2048, of 2048 beyond
+@pytest.mark.parametrize("n", [511, 512, 513, 16_385, 311_296, 311_297, 4_000_001])
+def test_scan_partition_sizes(R, n):
+    x = torch.randint(0, 1000, (n,), device="cuda", dtype=torch.int32)
+    out, total = R.scan_u32(x)
+    torch.cuda.synchronize()
+    want = torch.cumsum(x.to(torch.int64), 0)
+    assert int(total) == int(want[-1]) & 0xffffffff or int(total) == int(want[-1])
+    assert torch.equal(out.to(torch.int64) & 0xffffffff, (want - x) & 0xffffffff)
+
+
+@pytest.mark.parametrize("dtype,tile", [("f32", 16), ("f16", 8)])
+def test_tall_rects_next_to_small_ones(R, dtype, tile):
+    """A view from among large Gaussians: rects of one to all of the tile rows in one
+    warp, several hundred thousand pairs; pixels as on tiles of one row of rects."""
+    from scenegen import look_camera, make_uniform_box_scene, quantize_attributes
+    scene = make_uniform_box_scene(3000, seed=4)
+    leaves = np.flatnonzero(scene.child_count == 0)
+    scene.log_scale[leaves[::9]] += np.float32(2.0)
+    cam = look_camera((2.0, 2.0, 1.2), 0.4, 640, 480, tau=0.0)
+    stored = None if dtype == "f32" else quantize_attributes(scene, dtype)[0]
+    R.load_scene(scene, attr_dtype=dtype, stored=stored)
+    images = []
+    for t in (tile, 32):
+        R.set_tile(t, t)
+        images.append(R.render([cam])[0].clone())
+        ranges, pairs = R.tile_ranges(0, -(-640 // t) * -(-480 // t), 1 << 23)
+        assert pairs == R.stats()["pair_total"] == int((ranges[:, 1] - ranges[:, 0]).sum())
+    R.set_tile(16, 16)
+    assert pairs > 20_000 and torch.equal(images[0], images[1])
