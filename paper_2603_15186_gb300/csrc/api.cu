@@ -140,7 +140,8 @@ struct ngs_ctx {
     // standalone sort/scan scratch
     void *sort_tmp_keys = nullptr;
     uint32_t *sort_tmp_vals = nullptr;
-    int64_t sort_tmp_cap = 0;
+    size_t sort_tmp_key_bytes = 0;     // keys of both widths share the buffer
+    int64_t sort_tmp_cap = 0;          // values
 };
 
 namespace {
@@ -1746,15 +1747,17 @@ NGS_API ngs_status ngs_sort_pairs(ngs_ctx *c, void *d_keys, uint32_t *d_vals, in
     if (s != NGS_OK) return s;
     const int64_t parts = (n + sort_partition() - 1) / sort_partition();
     if (parts * 256 > c->w.status_limit) return NGS_ERR_CAPACITY;
-    if (n > c->sort_tmp_cap) {
+    if (n > c->sort_tmp_cap || (size_t)n * key_bytes > c->sort_tmp_key_bytes) {
         dfree(c->sort_tmp_keys);
         dfree(c->sort_tmp_vals);
         c->sort_tmp_keys = nullptr;
         c->sort_tmp_vals = nullptr;
+        c->sort_tmp_key_bytes = 0;
         c->sort_tmp_cap = 0;
         if (dalloc((unsigned char **)&c->sort_tmp_keys, (size_t)n * key_bytes) != NGS_OK ||
             dalloc(&c->sort_tmp_vals, (size_t)n) != NGS_OK)
             return NGS_ERR_OUT_OF_MEMORY;
+        c->sort_tmp_key_bytes = (size_t)n * key_bytes;
         c->sort_tmp_cap = n;
     }
     const int passes = sort_passes(begin_bit, end_bit);

@@ -189,3 +189,19 @@ def test_tall_rects_next_to_small_ones(R, dtype, tile):
         assert pairs == R.stats()["pair_total"] == int((ranges[:, 1] - ranges[:, 0]).sum())
     R.set_tile(16, 16)
     assert pairs > 20_000 and torch.equal(images[0], images[1])
+
+
+def test_sort_key_widths_share_the_scratch():
+    """64-bit keys after as many 32-bit keys (and the other way round): the context's
+    scratch is large enough for either."""
+    from paper_2603_15186_gb300 import Renderer
+    r = Renderer(cut_capacity=1 << 20, record_capacity=1 << 22, pair_capacity=1 << 22)
+    n = 3_000_000
+    for dtype in (torch.int32, torch.int64, torch.int32):
+        keys = torch.randint(0, 1 << 30, (n,), device="cuda", dtype=dtype)
+        vals = torch.arange(n, device="cuda", dtype=torch.int32)
+        want, order = torch.sort(keys, stable=True)
+        r.sort_pairs(keys, vals)
+        torch.cuda.synchronize()
+        assert torch.equal(keys, want) and torch.equal(vals, order.to(torch.int32))
+    r.close()
