@@ -175,6 +175,28 @@ void dfree(void *p) {
 
 __global__ void k_bump_epoch(uint32_t *epoch, uint32_t inc) { *epoch += inc; }
 
+// Start of a sub-batch: everything its kernels count up from zero, and the epoch.
+// One launch in the place of five clears and the epoch's: on a small view each of
+// them took as long as this kernel (2 us with the gap before it).
+__global__ void k_begin(uint32_t *epoch, uint32_t inc, uint32_t *counters, uint32_t *hist,
+                        uint32_t *vis_count, int n_cams, uint2 *ranges, uint32_t n_tiles,
+                        unsigned long long *work64, int n_work64) {
+    const uint32_t i0 = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+    if (i0 == 0) *epoch += inc;
+    for (uint32_t i = i0; i < N_COUNTERS; i += step) counters[i] = 0;
+    for (uint32_t i = i0; i < kHistWords; i += step) hist[i] = 0;
+    for (uint32_t i = i0; i < (uint32_t)n_cams; i += step) vis_count[i] = 0;
+    for (uint32_t i = i0; i < n_tiles; i += step) ranges[i] = make_uint2(0u, 0u);
+    for (uint32_t i = i0; i < (uint32_t)n_work64; i += step) work64[i] = 0;
+}
+
+// n_work64: the words of work64 to clear (the first sub-batch of a render: all)
+void launch_begin(const Work &w, int n_cams, uint32_t n_tiles, int n_work64, cudaStream_t st) {
+    const uint32_t grid = std::min<uint32_t>((std::max<uint32_t>(n_tiles, kHistWords) + 255) / 256, 1024);
+    k_begin<<<grid, 256, 0, st>>>(w.epoch, kEpochStride, w.counters, w.hist, w.vis_count, n_cams,
+                                  w.ranges, n_tiles, w.work64, n_work64);
+}
+
 __global__ void k_offsets_to_i64(const uint32_t *in, int64_t *out, int n) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i <= n) out[i] = in[i];
@@ -187,11 +209,8 @@ __global__ void k_wait_probe(const uint64_t *status, const uint32_t *epoch_ptr, 
     look_back(status, 1, 1, *epoch_ptr + kEpochStride - 1, &prev, err);
 }
 
-// per sub-batch: cut, visible and pair totals, and the cut + preprocess
-// candidates (slots allocated, the low word of the 64-bit counter)
 __global__ void k_copy_stats(const uint32_t *counters, uint32_t *stats) {
-    if (threadIdx.x < 3) stats[threadIdx.x] = counters[threadIdx.x];
-    if (threadIdx.x == 3) stats[3] = counters[CNT_ALLOC];
+    keep_stats(counters, stats);
 }
 
 void free_work(ngs_ctx *c) {
@@ -335,7 +354,7 @@ ngs_status ensure_work(ngs_ctx *c) {
         A(dalloc(&w.pval[i], (size_t)w.pair_cap));
     }
     A(dalloc(&w.ranges, (size_t)w.ranges_cap));
-    A(dalloc(&w.hist, 8 * 256));
+    A(dalloc(&w.hist, kHistWords));
     A(dalloc(&w.cams, (size_t)w.cams_cap));
     c->stats_cap = 4096;
     A(dalloc(&c->stats_dev, (size_t)c->stats_cap * 4));
@@ -581,9 +600,7 @@ void enqueue_batched(ngs_ctx *c, const SubBatch &sb, int sb_index, cudaStream_t 
     const int nc = sb.c1 - sb.c0;
     const DevCamera *cams = w.cams + sb.c0;
     mark(c, sb_index, MK_START, st);
-    cudaMemsetAsync(w.counters, 0, N_COUNTERS * sizeof(uint32_t), st);
-    cudaMemsetAsync(w.ranges, 0, (size_t)sb.n_tiles * sizeof(uint2), st);
-    k_bump_epoch<<<1, 1, 0, st>>>(w.epoch, kEpochStride);
+    launch_begin(w, nc, sb.n_tiles, sb_index == 0 ? kWork64Words : 0, st);
     uint32_t eo = 0;
     launch_cutpre(c->scene, cams, nc, w.rec, w.rec_cap, w.dkey[1], w.rect,
                   c->node_ids ? w.node_id : nullptr, w.vis_count,
@@ -609,10 +626,10 @@ void enqueue_batched(ngs_ctx *c, const SubBatch &sb, int sb_index, cudaStream_t 
     eo += 4;
     const int dsel = 4 & 1;  // four passes: the result is back in buffer 0
     // the tile sort's digit histograms are counted by the offset scan
-    cudaMemsetAsync(w.hist, 0, sizeof(uint32_t) * 256 * 3, st);
+    uint32_t *thist = w.hist + kTileHist;
     launch_pair_offsets(w.rect, w.didx[dsel], w.counters + CNT_VIS, w.poff, w.counters,
                         w.pair_cap, w.counters + TK_SCAN, w.status, w.epoch, eo++, w.err,
-                        w.chunk_first, w.rect_sorted, cams, w.hist, sb.tile_passes,
+                        w.chunk_first, w.rect_sorted, cams, thist, sb.tile_passes,
                         c->grid_scan, st);
     mark(c, sb_index, MK_POFF, st);
     launch_duplicate(w.rect_sorted, w.didx[dsel], w.poff, w.chunk_first, w.counters + CNT_VIS,
@@ -629,7 +646,7 @@ void enqueue_batched(ngs_ctx *c, const SubBatch &sb, int sb_index, cudaStream_t 
         pa.key_bytes = 4; pa.begin_bit = 0; pa.end_bit = 8 * sb.tile_passes;
         pa.vals_identity = false;
         pa.hist_ready = true;   // counted by the offset scan
-        pa.hist = w.hist; pa.tickets = w.counters + TK_SORT0 + 4; pa.status = w.status;
+        pa.hist = thist; pa.tickets = w.counters + TK_SORT0 + 4; pa.status = w.status;
         pa.epoch = w.epoch; pa.epoch_off = eo; pa.err = w.err;
         pa.hook = c->timing ? sort_hook : nullptr; pa.hook_user = &th;
         pa.ranges = w.ranges;   // the last pass records the tile ranges
@@ -647,7 +664,10 @@ void enqueue_batched(ngs_ctx *c, const SubBatch &sb, int sb_index, cudaStream_t 
     const int cgrid = (int)std::min<int64_t>(
         items, (int64_t)c->num_sms *
                    std::max(1, composite_blocks_per_sm(c->scene.attr_dtype, cw, ch, c->batch)));
-    if (c->composite_order) launch_tile_order(w.ranges, sb.n_tiles, w.order, w.err, st);
+    // what the sub-batch counted (final by now) is kept by the same launch
+    uint32_t *kept = sb_index < c->stats_cap / 4 ? c->stats_dev + 4 * sb_index : nullptr;
+    if (c->composite_order)
+        launch_tile_order(w.ranges, sb.n_tiles, w.order, w.err, w.counters, kept, st);
     launch_composite(c->scene.attr_dtype, c->tile_w, c->tile_h, cw, ch, c->batch, true, cams, nc,
                      sb.n_tiles, w.ranges, w.pval[psel], w.rec, w.counters + TK_COMPOSITE,
                      std::max(cgrid, 1), w.err, w.work64,
@@ -655,18 +675,17 @@ void enqueue_batched(ngs_ctx *c, const SubBatch &sb, int sb_index, cudaStream_t 
                      sb_index < kTailSlots ? w.work64 + 2 + 2 * sb_index : nullptr, st);
     mark(c, sb_index, MK_COMPOSITE, st);
     record_event(c->ev_sb[sb_index], st);
-    if (sb_index < c->stats_cap / 4)
-        k_copy_stats<<<1, 32, 0, st>>>(w.counters, c->stats_dev + 4 * sb_index);
+    if (kept && !c->composite_order) k_copy_stats<<<1, 32, 0, st>>>(w.counters, kept);
 }
 
 int kernels_of(const SubBatch &sb, bool batched, bool order) {
-    // epoch bump, live partitions, fused cut + preprocess, partition scan and
-    // key gather (which also counts the depth histograms); depth sort (4
-    // passes); pair offsets, duplication; tile sort (the last pass writing the
-    // tile ranges) or, with a single tile, the ranges kernel; compositing; and
-    // in the batched path the stats copy
-    return 5 + 4 + 2 + std::max(sb.tile_passes, 1) + 1 + (batched ? 1 : 0) +
-           (batched && order ? 1 : 0);
+    // start, live partitions, fused cut + preprocess, partition scan and key
+    // gather (which also counts the depth histograms); depth sort (4 passes);
+    // pair offsets, duplication; tile sort (the last pass writing the tile
+    // ranges) or, with a single tile, the ranges kernel; compositing; and in the
+    // batched path the tile order, or else the stats copy
+    (void)order;
+    return 5 + 4 + 2 + std::max(sb.tile_passes, 1) + 1 + (batched ? 1 : 0);
 }
 
 ngs_status read_u32(const uint32_t *d, uint32_t *h, cudaStream_t st) {
@@ -715,7 +734,6 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
     int64_t cut_tot = 0, vis_tot = 0, pair_tot = 0;
     ngs_status es0 = ensure_events(c, n_cams);
     if (es0 != NGS_OK) return es0;
-    CK(cudaMemsetAsync(w.work64, 0, kWork64Words * sizeof(unsigned long long), st));
     c->kernels_per_render = 0;
     for (int ci = 0; ci < n_cams; ++ci) {
         SubBatch sb{ci, ci + 1, 0, 0};
@@ -728,9 +746,7 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
         ngs_status es = epoch_guard(c, st, kEpochStride);
         if (es != NGS_OK) return es;
         mark(c, ci, MK_START, st);
-        CK(cudaMemsetAsync(w.counters, 0, N_COUNTERS * sizeof(uint32_t), st));
-        CK(cudaMemsetAsync(w.ranges, 0, (size_t)sb.n_tiles * sizeof(uint2), st));
-        k_bump_epoch<<<1, 1, 0, st>>>(w.epoch, kEpochStride);
+        launch_begin(w, 1, sb.n_tiles, ci == 0 ? kWork64Words : 0, st);
         uint32_t eo = 0;
         const int64_t nblk = (c->scene.n + cutpre_partition_nodes() - 1) / cutpre_partition_nodes();
         launch_cutpre(c->scene, cams, 1, w.rec, w.rec_cap, w.dkey[1], w.rect,
@@ -768,10 +784,10 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
         launch_sort(da, std::min(gsort_v, c->grid_sort32), st);
         eo += 4;
         const int gscan = (int)std::max<int64_t>(1, scan_parts(n_vis));
-        CK(cudaMemsetAsync(w.hist, 0, sizeof(uint32_t) * 256 * 3, st));
+        uint32_t *thist = w.hist + kTileHist;
         launch_pair_offsets(w.rect, w.didx[0], w.counters + CNT_VIS, w.poff, w.counters,
                             w.pair_cap, w.counters + TK_SCAN, w.status, w.epoch, eo++, w.err,
-                            w.chunk_first, w.rect_sorted, cams, w.hist, sb.tile_passes, gscan,
+                            w.chunk_first, w.rect_sorted, cams, thist, sb.tile_passes, gscan,
                             st);
         mark(c, ci, MK_POFF, st);
         if ((s = read_u32(w.counters + CNT_PAIRS, &n_pairs, st)) != NGS_OK) return s;
@@ -795,7 +811,7 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
             pa.key_bytes = 4; pa.begin_bit = 0; pa.end_bit = 8 * sb.tile_passes;
             pa.vals_identity = false;
             pa.hist_ready = true;   // counted by the offset scan
-            pa.hist = w.hist; pa.tickets = w.counters + TK_SORT0 + 4; pa.status = w.status;
+            pa.hist = thist; pa.tickets = w.counters + TK_SORT0 + 4; pa.status = w.status;
             pa.epoch = w.epoch; pa.epoch_off = eo; pa.err = w.err;
             pa.hook = c->timing ? sort_hook : nullptr; pa.hook_user = &th;
             pa.ranges = w.ranges;   // the last pass records the tile ranges
@@ -863,7 +879,6 @@ ngs_status render_batched(ngs_ctx *c, int n_cams, cudaStream_t st) {
             drop_graph(c);
             if (!c->cap_stream) CK(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
             CK(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
-            cudaMemsetAsync(w.work64, 0, kWork64Words * sizeof(unsigned long long), c->cap_stream);
             for (size_t i = 0; i < sbs.size(); ++i) enqueue_batched(c, sbs[i], (int)i, c->cap_stream);
             cudaGraph_t g = nullptr;
             cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
@@ -884,7 +899,6 @@ ngs_status render_batched(ngs_ctx *c, int n_cams, cudaStream_t st) {
         }
         CK(cudaGraphLaunch(c->gexec, st));
     } else {
-        CK(cudaMemsetAsync(w.work64, 0, kWork64Words * sizeof(unsigned long long), st));
         for (size_t i = 0; i < sbs.size(); ++i) enqueue_batched(c, sbs[i], (int)i, st);
         c->stats.graph_replayed = 0;
     }

@@ -466,8 +466,9 @@ __device__ __forceinline__ uint32_t length_class(uint2 rg) {
 
 __global__ void __launch_bounds__(1024)
 k_tile_order(const uint2 *__restrict__ ranges, uint32_t n_tiles, uint32_t *__restrict__ order,
-             const int *err) {
+             const int *err, const uint32_t *counters, uint32_t *stats) {
     __shared__ uint32_t s_hist[64], s_cur[64];
+    if (stats) keep_stats(counters, stats);   // also of a sub-batch that overflowed
     if (*err) return;
     if (threadIdx.x < 64) s_hist[threadIdx.x] = 0;
     __syncthreads();
@@ -487,8 +488,8 @@ k_tile_order(const uint2 *__restrict__ ranges, uint32_t n_tiles, uint32_t *__res
 }
 
 void launch_tile_order(const uint2 *ranges, uint32_t n_tiles, uint32_t *order, const int *err,
-                       cudaStream_t st) {
-    k_tile_order<<<1, 1024, 0, st>>>(ranges, n_tiles, order, err);
+                       const uint32_t *counters, uint32_t *stats, cudaStream_t st) {
+    k_tile_order<<<1, 1024, 0, st>>>(ranges, n_tiles, order, err, counters, stats);
 }
 
 template <typename R, int TW, int TH, int BATCH>

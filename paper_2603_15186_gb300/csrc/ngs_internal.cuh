@@ -369,7 +369,8 @@ struct Work {
     uint32_t *pval[2] = {nullptr, nullptr};
     int64_t pair_cap = 0;
     uint2 *ranges = nullptr;          int64_t ranges_cap = 0;
-    uint32_t *hist = nullptr;         // [passes][256] radix histograms
+    uint32_t *hist = nullptr;         // kHistWords: [4][256] of the depth sort, at kTileHist
+                                      // [3][256] of the tile sort; standalone sorts: [8][256]
     DevCamera *cams = nullptr;        int64_t cams_cap = 0;
     // compositing work counters: [0] records staged, [1] pixel-Gaussian
     // evaluations, then per sub-batch (up to kTailSlots) the tail words of its
@@ -380,6 +381,8 @@ struct Work {
 
 constexpr int kTailSlots = 64;
 constexpr int kWork64Words = 2 + 2 * kTailSlots;
+
+constexpr uint32_t kHistWords = 8 * 256, kTileHist = 4 * 256;
 
 // ticket slots in Work::counters
 enum : int {
@@ -392,6 +395,14 @@ enum : int {
     CNT_GROUPS = 27,          // groups of live partitions (same node block)
     TK_COMPOSITE = 28, N_COUNTERS = 32
 };
+
+// per sub-batch: cut, visible and pair totals, and the cut + preprocess
+// candidates (slots allocated, the low word of the 64-bit counter); by the first
+// four threads of a CTA
+__device__ __forceinline__ void keep_stats(const uint32_t *counters, uint32_t *stats) {
+    if (threadIdx.x < 3) stats[threadIdx.x] = counters[threadIdx.x];
+    if (threadIdx.x == 3) stats[3] = counters[CNT_ALLOC];
+}
 
 // ---------------------------------------------------------------------------
 // kernel launchers (one translation unit each)
@@ -519,9 +530,9 @@ void launch_composite(int attr_dtype, int tile_w, int tile_h, int cta_w, int cta
                       uint32_t *ticket, int grid, const int *err, unsigned long long *work64,
                       const uint32_t *order, unsigned long long *tail, cudaStream_t st);
 // the tiles [0, n_tiles) of a sub-batch, longest list first (classes of half
-// an octave), into order[n_tiles]
+// an octave), into order[n_tiles]; with stats, also keep_stats
 void launch_tile_order(const uint2 *ranges, uint32_t n_tiles, uint32_t *order, const int *err,
-                       cudaStream_t st);
+                       const uint32_t *counters, uint32_t *stats, cudaStream_t st);
 int composite_blocks_per_sm(int attr_dtype, int tile_w, int tile_h, int batch);
 void composite_init_attributes();
 
