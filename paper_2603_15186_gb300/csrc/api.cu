@@ -474,11 +474,12 @@ void fill_cut_cam(CutCam &d, const ngs_camera &k, float guard) {
     d.tau = k.tau;
 }
 
-// Units whose mask words fit in the record buffer at once (the words live there
-// between the passes of a cut: no render is in flight).
+// Units whose words and nodes' masks fit in the record buffer at once (they live there
+// between the passes of a cut: no render is in flight), each with a chunk of its own.
 int64_t cut_slice_units(const ngs_ctx *c) {
     return c->w.rec_cap * (int64_t)sizeof(Rec32) /
-           (cut_words_per_unit(c->scene.n) * (int64_t)sizeof(uint32_t));
+           (cut_words_per_unit(c->scene.n) * (int64_t)sizeof(uint32_t) +
+            c->scene.n * (int64_t)sizeof(uint2));
 }
 
 // Whether a cut goes by masks: enough cameras for a lane each, groups that fit a
@@ -526,7 +527,8 @@ ngs_status cut_by_masks(ngs_ctx *c, const std::vector<CutCam> &hc, const int32_t
         CK(cudaMemcpyAsync(c->cut_groups, group_begin, sizeof(int32_t) * (n_units + 1),
                            cudaMemcpyHostToDevice, st));
     const int64_t nblk = (sc.n + cut_partition_nodes() - 1) / cut_partition_nodes();
-    uint32_t *words = (uint32_t *)w.rec;
+    uint2 *masks = (uint2 *)w.rec;
+    uint32_t *words = (uint32_t *)(masks + (int64_t)slice * sc.n);
     for (size_t k = 0; k + 1 < first_chunk.size(); ++k) {
         const int u0 = (int)k * slice, nu = std::min(slice, n_units - u0);
         ngs_status s = epoch_guard(c, st, kEpochStride);
@@ -535,7 +537,7 @@ ngs_status cut_by_masks(ngs_ctx *c, const std::vector<CutCam> &hc, const int32_t
         k_bump_epoch<<<1, 1, 0, st>>>(w.epoch, kEpochStride);
         launch_cut_masks(frustum, group_begin != nullptr, lanes, sc.box_lo, sc.box_hi, sc.n,
                          c->cut_cams, c->cut_groups + u0, c->cut_chunks + first_chunk[k],
-                         first_chunk[k + 1] - first_chunk[k], words, c->cut_counts, w.err, st);
+                         first_chunk[k + 1] - first_chunk[k], masks, words, c->cut_counts, w.err, st);
         const int64_t np = nblk * nu, sparts = scan_parts(np);
         launch_scan_u32(c->cut_counts, c->cut_poff, nullptr, np, c->cut_off32,
                         w.counters + TK_SCAN, w.status, w.epoch, 0, w.err,

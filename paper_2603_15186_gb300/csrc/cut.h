@@ -41,7 +41,7 @@ struct CutChunk {
 // Cuts of many units, one slice of them at a time: launch_cut_masks decides, for
 // chunks of at most c <= 32 cameras, every (node, unit) into words[unit *
 // cut_words_per_unit() ...] and counts[unit * blocks + block] (blocks of
-// cut_partition_nodes() nodes); after an exclusive scan of the counts into part_off
+// cut_partition_nodes() nodes), with masks[n_chunks][n_nodes] as scratch; after an exclusive scan of the counts into part_off
 // (its sum in *total), launch_cut_write writes the units' offsets (offsets[0] ..
 // offsets[n_units], continuing from offsets[0] unless `first`) and ids; with `last`
 // also counters[CNT_CUT], and it latches the capacity error when the ids exceed cap.
@@ -50,7 +50,8 @@ struct CutChunk {
 void launch_cut_masks(bool frustum, bool groups, int c, const float4 *box_lo,
                       const float4 *box_hi, int64_t n_nodes, const CutCam *cams,
                       const int32_t *group_begin, const CutChunk *chunks, int n_chunks,
-                      uint32_t *words, uint32_t *counts, const int *err, cudaStream_t st);
+                      uint2 *masks, uint32_t *words, uint32_t *counts, const int *err,
+                      cudaStream_t st);
 void launch_cut_write(const uint32_t *words, const uint32_t *part_off, const uint32_t *total,
                       int64_t n_nodes, int n_units, bool first, bool last, int64_t cap,
                       uint32_t *ids, int64_t *offsets, uint32_t *counters, int *err,

@@ -216,106 +216,68 @@ k_cut_shared(const float4 *__restrict__ box_lo, const float4 *__restrict__ box_h
                    epoch_ptr, epoch_off, err);
 }
 
-// Cuts of many cameras or groups ("units"), in three steps: k_cut_masks decides
-// every (node, unit) and keeps one bit each, 32 nodes to a word, and each unit's
-// count per node block; a scan of the counts in unit-major order gives the output
-// offsets (k_cut_unit_offsets: those of the units); k_cut_write turns the words into
-// ids, a pure stream.
+// Cuts of many cameras or groups ("units"), in four steps: k_cut_nodes tests every
+// interior node for every camera; k_cut_masks decides every (node, unit) from that and
+// keeps one bit each, 32 nodes to a word, and each unit's count per node block; a scan
+// of the counts in unit-major order gives the output offsets (k_cut_unit_offsets: those
+// of the units); k_cut_write turns the words into ids, a pure stream.
 //
-// k_cut_masks: one CTA per (block of kCutPart nodes, chunk of up to C cameras). The
-// tests are taken with one lane per camera, 32 / C boxes at a time, so that a ballot
-// is the box's mask over the chunk's cameras: N (the camera keeps the box and it is
-// not fine enough) and, with kFrustum, V (the camera keeps it). Per word of 32 nodes
-//   - the distinct parents (siblings follow one another) are tested once each;
-//   - then the interior nodes that some camera of the chunk still wants refined;
-//   - a leaf has N = 0; its V is tested only for the cameras whose unit wants its
-//     parent refined, one lane per leaf, until a camera of the unit keeps it.
-// A unit's decision is bits: (leaf or no N_n) and (root or some N_p) and some V_n over
-// the unit's cameras. Without kGroups (units of one camera) that is the same formula
-// on whole masks, and a 32 x 32 bit transpose turns 32 nodes' masks into the cameras'
-// words. With kFrustum a word whose boxes' union every camera culls is left out (a box
-// outside a half-space has every box it contains outside too, also in float32: the
-// tests are monotone in the bounds).
+// Both of the first run one CTA per (block of kCutPart nodes, chunk of up to C cameras)
+// and use bit masks over the chunk's cameras: N (the camera keeps the node's box and it
+// is not fine enough) and, with kFrustum, V (the camera keeps it).
+//   k_cut_nodes: one lane per camera, 32 / C boxes at a time, so that a ballot is a box's
+//     mask. With kFrustum 32 nodes whose boxes' union every camera culls go without
+//     tests (a box outside a half-space has every box it contains outside too, also in
+//     float32: the tests are monotone in the bounds).
+//   k_cut_masks: a node's own masks and its parent's. A leaf has N = 0; its V is tested
+//     only for the cameras whose unit wants its parent refined, one lane per leaf, until
+//     a camera of the unit keeps it. A unit's decision is bits: (leaf or no N_n) and
+//     (root or some N_p) and some V_n over the unit's cameras; without kGroups (units of
+//     one camera) that is the same formula on whole masks, and a 32 x 32 bit transpose
+//     turns 32 nodes' masks into the cameras' words.
 //
 // Bound by the issue of the tests (about 14 instructions for a granularity, 75 for
 // five planes). A test per (node, camera) on the node and on its parent, once to count
 // and once to write, took 683 + 1016 us for 64 plain cuts of 5.25 M nodes, and one
 // thread per node over its group's members 1557 us for 8 frustum-culled cuts of 8
-// cameras each; CUT_NOTE
+// cameras each; with the parents tested again for the children of each word 228 us (+ 159
+// us to write 850 MB of ids) and 530 us, with their masks read 172 us (108 + 64) and 433 us (228 + 205).
 constexpr int kCutWords = kCutPart / 32;
 
-template <bool kFrustum, bool kGroups, int C>
+template <bool kFrustum, int C>
 __global__ void __launch_bounds__(kCutThreads)
-k_cut_masks(const float4 *__restrict__ box_lo, const float4 *__restrict__ box_hi,
-            int64_t n_nodes, const CutCam *__restrict__ cams,
-            const int32_t *__restrict__ group_begin, const CutChunk *__restrict__ chunks,
-            int n_chunks, uint32_t *__restrict__ words, uint32_t *__restrict__ counts,
-            const int *err) {
+k_cut_nodes(const float4 *__restrict__ box_lo, const float4 *__restrict__ box_hi,
+            int64_t n_nodes, const CutCam *__restrict__ cams, const CutChunk *__restrict__ chunks,
+            int n_chunks, uint2 *__restrict__ masks, const int *err) {
     constexpr int G = 32 / C, kWarps = kCutThreads / 32;
-    static_assert(kCutWords % kWarps == 0 && kCutWords == 64, "two words per lane");
     __shared__ float4 s_lo[kWarps][32], s_hi[kWarps][32];   // the boxes under test, per warp
-    __shared__ uint32_t s_word[C][kCutWords + 1];
-    __shared__ CutCam s_cam[kFrustum ? C : 1];
-    __shared__ uint32_t s_unit[kGroups ? C : 1];   // each unit's cameras of the chunk
     if (*err) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int64_t nblk = (n_nodes + kCutPart - 1) / kCutPart;
     const int64_t b = blockIdx.x / n_chunks;
-    const CutChunk ch = chunks[blockIdx.x - b * n_chunks];
-    const uint32_t live = ch.n_cams == 32 ? 0xffffffffu : (1u << ch.n_cams) - 1u;
-    // this lane's camera
+    const int k = (int)(blockIdx.x - b * n_chunks);
+    const CutChunk ch = chunks[k];
+    uint2 *out = masks + k * n_nodes;
+    // this lane's camera, and which of the boxes taken at once it tests
     const int cl = lane % C, grp = lane / C;
     const CutCam cam = cams[ch.cam0 + min(cl, ch.n_cams - 1)];
     const float tau2 = __fmul_rn(cam.tau, cam.tau);
-    if (kFrustum) {
-        if (tid < ch.n_cams) s_cam[tid] = cams[ch.cam0 + tid];
-        if (kGroups && tid < ch.n_units) {
-            const int g0 = group_begin[ch.unit0 + tid] - ch.cam0, g1 = group_begin[ch.unit0 + tid + 1] - ch.cam0;
-            s_unit[tid] = (g1 == 32 ? 0xffffffffu : (1u << g1) - 1u) & ~((1u << g0) - 1u);
-        }
-        __syncthreads();
-    } else if (kGroups) {
-        if (tid < ch.n_units) {
-            const int g0 = group_begin[ch.unit0 + tid] - ch.cam0, g1 = group_begin[ch.unit0 + tid + 1] - ch.cam0;
-            s_unit[tid] = (g1 == 32 ? 0xffffffffu : (1u << g1) - 1u) & ~((1u << g0) - 1u);
-        }
-        __syncthreads();
-    }
-    // masks (N, V) of the staged boxes; a lane whose box is number `rank` gets them
-    auto test = [&](int n, int rank, uint32_t &N, uint32_t &V) {
-        __syncwarp();
-#pragma unroll 2
-        for (int t = 0; t < n; t += G) {
-            const int k = min(t + grp, n - 1);
-            const float4 lo = s_lo[warp][k], hi = s_hi[warp][k];
-            const bool keep = !kFrustum || !frustum_culled(cam, lo, hi);
-            const bool fine = fine_enough_pre(lo, hi, box_extent(lo, hi), cam.pos[0], cam.pos[1],
-                                              cam.pos[2], cam.fx, tau2);
-            const uint32_t nm = __ballot_sync(0xffffffffu, keep && !fine);
-            const uint32_t vm = kFrustum ? __ballot_sync(0xffffffffu, keep) : 0xffffffffu;
-            const int at = rank - t;
-            if (at >= 0 && at < G) {
-                N = nm >> (C * at % 32);
-                V = vm >> (C * at % 32);
-            }
-        }
-        __syncwarp();
-    };
     for (int j = warp; j < kCutWords; j += kWarps) {
         const int64_t node = b * kCutPart + 32 * j + lane;
         const bool valid = node < n_nodes;
-        float4 lo = make_float4(0.f, 0.f, 0.f, __int_as_float(-1)), hi = make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
         if (valid) {
             lo = box_lo[node];
             hi = box_hi[node];
         }
-        const int parent = __float_as_int(lo.w);
-        const bool leaf = __float_as_int(hi.w) == 0;
-        bool look = __any_sync(0xffffffffu, valid);
-        if (kFrustum && look) {
+        const bool inner = valid && __float_as_int(hi.w) != 0;
+        const uint32_t inners = __ballot_sync(0xffffffffu, inner);
+        if (inners == 0) continue;
+        uint32_t N = 0, V = 0;
+        bool look = true;
+        if (kFrustum) {
             const float inf = __int_as_float(0x7f800000);
-            float4 ulo = valid ? lo : make_float4(inf, inf, inf, 0.f);
-            float4 uhi = valid ? hi : make_float4(-inf, -inf, -inf, 0.f);
+            float4 ulo = inner ? lo : make_float4(inf, inf, inf, 0.f);
+            float4 uhi = inner ? hi : make_float4(-inf, -inf, -inf, 0.f);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
                 ulo.x = fminf(ulo.x, __shfl_xor_sync(0xffffffffu, ulo.x, o));
@@ -327,62 +289,110 @@ k_cut_masks(const float4 *__restrict__ box_lo, const float4 *__restrict__ box_hi
             }
             look = __any_sync(0xffffffffu, cl < ch.n_cams && !frustum_culled(cam, ulo, uhi));
         }
-        uint32_t sel = 0;     // bit u: unit u (camera, without kGroups) selects the node
         if (look) {
-            // the parents
-            const int before = __shfl_up_sync(0xffffffffu, parent, 1);
-            const bool first = valid && parent >= 0 && (lane == 0 || parent != before);
-            const uint32_t firsts = __ballot_sync(0xffffffffu, first);
-            const int rank = __popc(firsts & (lanemask_lt() | 1u << lane)) - 1;
-            if (first) {
-                s_lo[warp][rank] = box_lo[parent];
-                s_hi[warp][rank] = box_hi[parent];
-            }
-            uint32_t Np = 0, Vp = 0;
-            test(__popc(firsts), valid && parent >= 0 ? rank : -1, Np, Vp);
-            if (valid && parent < 0) Np = 0xffffffffu;   // the root: as if a parent were refined
-            Np &= live;
-            // the cameras whose units want the parent refined
-            uint32_t want = Np;
-            if (kGroups) {
-                want = 0;
-                for (int u = 0; u < ch.n_units; ++u)
-                    if (Np & s_unit[u]) want |= s_unit[u];
-            }
-            // the interior nodes among them
-            uint32_t Nn = 0, Vn = kFrustum ? 0u : 0xffffffffu;
-            const bool inner = !leaf && want != 0;
-            const uint32_t inners = __ballot_sync(0xffffffffu, inner);
-            const int irank = __popc(inners & lanemask_lt());
+            const int n = __popc(inners), rank = inner ? __popc(inners & lanemask_lt()) : -1;
             if (inner) {
-                s_lo[warp][irank] = lo;
-                s_hi[warp][irank] = hi;
+                s_lo[warp][rank] = lo;
+                s_hi[warp][rank] = hi;
             }
-            test(__popc(inners), inner ? irank : -1, Nn, Vn);
+            __syncwarp();
+#pragma unroll 2
+            for (int t = 0; t < n; t += G) {
+                const int q = min(t + grp, n - 1);
+                const float4 l = s_lo[warp][q], h = s_hi[warp][q];
+                const bool keep = !kFrustum || !frustum_culled(cam, l, h);
+                const bool fine = fine_enough_pre(l, h, box_extent(l, h), cam.pos[0], cam.pos[1],
+                                                  cam.pos[2], cam.fx, tau2);
+                const uint32_t nm = __ballot_sync(0xffffffffu, keep && !fine);
+                const uint32_t vm = kFrustum ? __ballot_sync(0xffffffffu, keep) : 0xffffffffu;
+                const int at = rank - t;   // a lane whose box is among these takes its masks
+                if (at >= 0 && at < G) {
+                    N = nm >> (C * at % 32);
+                    V = vm >> (C * at % 32);
+                }
+            }
+            __syncwarp();
+        }
+        if (inner) out[node] = make_uint2(N, V);
+    }
+}
+
+template <bool kFrustum, bool kGroups, int C>
+__global__ void __launch_bounds__(kCutThreads)
+k_cut_masks(const float4 *__restrict__ box_lo, const float4 *__restrict__ box_hi,
+            int64_t n_nodes, const CutCam *__restrict__ cams,
+            const int32_t *__restrict__ group_begin, const CutChunk *__restrict__ chunks,
+            int n_chunks, const uint2 *__restrict__ masks, uint32_t *__restrict__ words,
+            uint32_t *__restrict__ counts, const int *err) {
+    constexpr int kWarps = kCutThreads / 32;
+    static_assert(kCutWords % kWarps == 0 && kCutWords == 64, "two words per lane");
+    __shared__ uint32_t s_word[C][kCutWords + 1];
+    __shared__ CutCam s_cam[kFrustum ? C : 1];
+    __shared__ uint32_t s_unit[kGroups ? C : 1];   // each unit's cameras of the chunk
+    if (*err) return;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t nblk = (n_nodes + kCutPart - 1) / kCutPart;
+    const int64_t b = blockIdx.x / n_chunks;
+    const int k = (int)(blockIdx.x - b * n_chunks);
+    const CutChunk ch = chunks[k];
+    const uint2 *mask = masks + k * n_nodes;
+    const uint32_t live = ch.n_cams == 32 ? 0xffffffffu : (1u << ch.n_cams) - 1u;
+    if (kFrustum && tid < ch.n_cams) s_cam[tid] = cams[ch.cam0 + tid];
+    if (kGroups && tid < ch.n_units) {
+        const int g0 = group_begin[ch.unit0 + tid] - ch.cam0, g1 = group_begin[ch.unit0 + tid + 1] - ch.cam0;
+        s_unit[tid] = (g1 == 32 ? 0xffffffffu : (1u << g1) - 1u) & ~((1u << g0) - 1u);
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int j = warp; j < kCutWords; j += kWarps) {
+        const int64_t node = b * kCutPart + 32 * j + lane;
+        const bool valid = node < n_nodes;
+        int parent = -1;
+        bool leaf = true;
+        if (valid) {
+            parent = __float_as_int(box_lo[node].w);
+            leaf = __float_as_int(box_hi[node].w) == 0;
+        }
+        // the root: as if a parent were refined
+        uint32_t Np = !valid ? 0u : parent < 0 ? 0xffffffffu : mask[parent].x;
+        Np &= live;
+        // the cameras whose units want the parent refined
+        uint32_t want = Np;
+        if (kGroups) {
+            want = 0;
+            for (int u = 0; u < ch.n_units; ++u)
+                if (Np & s_unit[u]) want |= s_unit[u];
+        }
+        uint32_t sel = 0;     // bit u: unit u (camera, without kGroups) selects the node
+        if (__any_sync(0xffffffffu, want != 0)) {
+            uint2 own = make_uint2(0u, kFrustum ? 0u : 0xffffffffu);   // N, V
+            if (!leaf && want) own = mask[node];
             if (kFrustum) {
                 // the leaves: a lane each, camera by camera
                 uint32_t need = leaf ? want : 0u;
+                float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
+                if (need) {
+                    lo = box_lo[node];
+                    hi = box_hi[node];
+                }
                 for (uint32_t c = __reduce_or_sync(0xffffffffu, need); c; c &= c - 1) {
-                    const int k = __ffs(c) - 1;
-                    if (need >> k & 1u) {
-                        if (!frustum_culled(s_cam[k], lo, hi)) {
-                            Vn |= 1u << k;
-                            if (kGroups)   // its unit's other cameras need not look
-                                for (int u = 0; u < ch.n_units; ++u)
-                                    if (s_unit[u] >> k & 1u) need &= ~s_unit[u];
-                        }
+                    const int q = __ffs(c) - 1;
+                    if ((need >> q & 1u) && !frustum_culled(s_cam[q], lo, hi)) {
+                        own.y |= 1u << q;
+                        if (kGroups)   // its unit's other cameras need not look
+                            for (int u = 0; u < ch.n_units; ++u)
+                                if (s_unit[u] >> q & 1u) need &= ~s_unit[u];
                     }
                 }
             }
             if (kGroups) {
                 for (int u = 0; u < ch.n_units; ++u) {
                     const uint32_t m = s_unit[u];
-                    if ((leaf || !(Nn & m)) && (Np & m) && (Vn & m)) sel |= 1u << u;
+                    if ((leaf || !(own.x & m)) && (Np & m) && (own.y & m)) sel |= 1u << u;
                 }
             } else {
-                sel = (leaf ? 0xffffffffu : ~Nn) & Np & Vn;
+                sel = (leaf ? 0xffffffffu : ~own.x) & Np & own.y;
             }
-            if (!valid) sel = 0;
         }
         // rows of nodes to rows of units
         uint32_t x = sel, m = 0x0000ffffu;
@@ -462,29 +472,39 @@ int64_t cut_words_per_unit(int64_t n_nodes) {
     return (n_nodes + kCutPart - 1) / kCutPart * kCutWords;
 }
 
+template <bool kFrustum, bool kGroups, int C>
+static void launch_masks_c(const float4 *box_lo, const float4 *box_hi, int64_t n_nodes,
+                           const CutCam *cams, const int32_t *group_begin, const CutChunk *chunks,
+                           int n_chunks, uint2 *masks, uint32_t *words, uint32_t *counts,
+                           const int *err, cudaStream_t st) {
+    const unsigned grid = (unsigned)((n_nodes + kCutPart - 1) / kCutPart * n_chunks);
+    k_cut_nodes<kFrustum, C><<<grid, kCutThreads, 0, st>>>(box_lo, box_hi, n_nodes, cams, chunks,
+                                                           n_chunks, masks, err);
+    k_cut_masks<kFrustum, kGroups, C><<<grid, kCutThreads, 0, st>>>(
+        box_lo, box_hi, n_nodes, cams, group_begin, chunks, n_chunks, masks, words, counts, err);
+}
+
 template <bool kFrustum, bool kGroups>
 static void launch_masks(int c, const float4 *box_lo, const float4 *box_hi, int64_t n_nodes,
                          const CutCam *cams, const int32_t *group_begin, const CutChunk *chunks,
-                         int n_chunks, uint32_t *words, uint32_t *counts, const int *err,
-                         cudaStream_t st) {
-    const unsigned grid = (unsigned)((n_nodes + kCutPart - 1) / kCutPart * n_chunks);
-    if (c <= 8)
-        k_cut_masks<kFrustum, kGroups, 8><<<grid, kCutThreads, 0, st>>>(
-            box_lo, box_hi, n_nodes, cams, group_begin, chunks, n_chunks, words, counts, err);
-    else if (c <= 16)
-        k_cut_masks<kFrustum, kGroups, 16><<<grid, kCutThreads, 0, st>>>(
-            box_lo, box_hi, n_nodes, cams, group_begin, chunks, n_chunks, words, counts, err);
-    else
-        k_cut_masks<kFrustum, kGroups, 32><<<grid, kCutThreads, 0, st>>>(
-            box_lo, box_hi, n_nodes, cams, group_begin, chunks, n_chunks, words, counts, err);
+                         int n_chunks, uint2 *masks, uint32_t *words, uint32_t *counts,
+                         const int *err, cudaStream_t st) {
+    auto go = [&](auto f) {
+        f(box_lo, box_hi, n_nodes, cams, group_begin, chunks, n_chunks, masks, words, counts, err, st);
+    };
+    if (c <= 8) go(launch_masks_c<kFrustum, kGroups, 8>);
+    else if (c <= 16) go(launch_masks_c<kFrustum, kGroups, 16>);
+    else go(launch_masks_c<kFrustum, kGroups, 32>);
 }
 
 void launch_cut_masks(bool frustum, bool groups, int c, const float4 *box_lo,
                       const float4 *box_hi, int64_t n_nodes, const CutCam *cams,
                       const int32_t *group_begin, const CutChunk *chunks, int n_chunks,
-                      uint32_t *words, uint32_t *counts, const int *err, cudaStream_t st) {
+                      uint2 *masks, uint32_t *words, uint32_t *counts, const int *err,
+                      cudaStream_t st) {
     auto go = [&](auto f) {
-        f(c, box_lo, box_hi, n_nodes, cams, group_begin, chunks, n_chunks, words, counts, err, st);
+        f(c, box_lo, box_hi, n_nodes, cams, group_begin, chunks, n_chunks, masks, words, counts, err,
+          st);
     };
     if (frustum) groups ? go(launch_masks<true, true>) : go(launch_masks<true, false>);
     else groups ? go(launch_masks<false, true>) : go(launch_masks<false, false>);

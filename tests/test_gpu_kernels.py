@@ -110,9 +110,9 @@ def floor_views(small_floor):
     return walk_cameras(small_floor, 110, seed=8, width=320, height=240, taus=taus)
 
 
-# record_capacity: 2^22 holds every mask word of a call, 2^10 those of five cameras of
-# this scene (calls cut in slices), 2^7 none (single-pass kernels)
-@pytest.mark.parametrize("records", [1 << 22, 1 << 10, 1 << 7])
+# record_capacity: 2^22 holds the masks of every call here, 2^16 those of four cameras of
+# this scene (calls cut in slices), 2^12 none (single-pass kernels)
+@pytest.mark.parametrize("records", [1 << 22, 1 << 16, 1 << 12])
 def test_cuts_by_masks_equal_single_pass_cuts(small_floor, floor_views, records):
     from paper_2603_15186_gb300 import Renderer
     R = Renderer(cut_capacity=1 << 22, record_capacity=records, pair_capacity=1 << 20)
