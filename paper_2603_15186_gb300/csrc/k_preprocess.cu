@@ -35,7 +35,12 @@
 namespace ngs {
 
 constexpr int kPreThreads = 256;
-constexpr int kPreItems = 4;                          // phase-A nodes per thread
+// Phase-A nodes per thread. Finer partitions cull better and spread a few views' groups
+// over the SMs; their tables and scans grow. k_cutpre + key gather with 4, 2, 1: 5987 +
+// 945, 5721 + 889, 5914 + 914 us on 256 mixed views of a 4M-leaf floor; 87 + 22, 56 + 14,
+// 52 + 12 us on eight 333x187 views of a 1M-leaf floor; 44 + 21, 40 + 14, 40 + 11 us on one
+// 720p view of the former, whose partition scan takes 6, 10, 19 us.
+constexpr int kPreItems = 2;
 constexpr int kPrePart = kPreThreads * kPreItems;     // nodes per partition
 
 
