@@ -134,11 +134,16 @@ struct CompLayout {
 
 __device__ __forceinline__ float finite_or_max(float v) { return fminf(v, 3.402823466e38f); }
 
-// at least five 128-thread CTAs per SM (at most 102 registers): measured
-// faster than both more registers (4 CTAs) and fewer (6 or 7, with spills)
+// 128-thread CTAs per SM that the registers leave room for: six with 32-byte records
+// (80 registers; 256 mixed views 18.47 ms against 19.00 with five), five with 48-byte
+// ones (96; four 640x480 views 174 us against 181 with six)
+// and in 8-pixel-wide tiles (whose warps gather up to eight records a lane)
+template <typename R, int TW>
+constexpr int kCompCtas = sizeof(R) == sizeof(Rec16) && TW >= 16 ? 6 : 5;
+
 template <typename R, int TW, int TH, int BATCH>
 __global__ void __launch_bounds__(CompLayout<R, TW, TH, BATCH>::NT,
-                                  (5 * 128) / CompLayout<R, TW, TH, BATCH>::NT)
+                                  (kCompCtas<R, TW> * 128) / CompLayout<R, TW, TH, BATCH>::NT)
 k_composite(const DevCamera *__restrict__ cams, int n_cams, uint32_t n_tiles,
             const uint2 *__restrict__ ranges, const uint32_t *__restrict__ pval,
             const R *__restrict__ rec, uint32_t *ticket, int persistent, const int *err,
