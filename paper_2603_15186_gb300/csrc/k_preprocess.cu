@@ -683,7 +683,7 @@ struct CutPreSmem {
     uint32_t ncand[kGroupCams], nvis[kGroupCams], sel[kGroupCams];
     CamLite cam[kGroupCams];
     uint32_t gcam[kGroupCams];
-    uint32_t wsum[kPreThreads / 32];
+    uint32_t wsum[kPreItems][kPreThreads / 32]; // entries per (item, warp)
     uint32_t goff, gcnt;
 };
 static_assert(kGroupCams <= 16 && kPrePart <= 4096, "entries pack node and camera in 16 bits");
@@ -802,6 +802,22 @@ k_cutpre(SceneDev sc, const DevCamera *__restrict__ cams, int n_cams, R *__restr
             }
             mask[k] = m;
         }
+        // node-major entry list: node v = k * kPreThreads + tid has popc(mask[k])
+        // entries, one per candidate camera in camera order; here those before it in
+        // its warp
+        uint32_t ent0[kPreItems];
+#pragma unroll
+        for (int k = 0; k < kPreItems; ++k) {
+            const uint32_t v = __popc(mask[k]);
+            uint32_t incl = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
+            }
+            if (lane == 31) S.wsum[k][warp] = incl;
+            ent0[k] = incl - v;
+        }
         __syncthreads();
         // per camera: candidates before each (item, warp) in node order, and
         // the partition's output space
@@ -824,33 +840,22 @@ k_cutpre(SceneDev sc, const DevCamera *__restrict__ cams, int n_cams, R *__restr
                 S.off[i] = off;
             }
         }
-        // node-major entry list: node v = k * kPreThreads + tid has popc(mask[k])
-        // entries, one per candidate camera in camera order
         uint32_t base = 0;
 #pragma unroll
         for (int k = 0; k < kPreItems; ++k) {
-            const uint32_t v = __popc(mask[k]);
-            uint32_t incl = v;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += t;
-            }
-            if (lane == 31) S.wsum[warp] = incl;
-            __syncthreads();
             uint32_t wb = 0, tot = 0;
 #pragma unroll
             for (int w = 0; w < kPreThreads / 32; ++w) {
-                if (w < warp) wb += S.wsum[w];
-                tot += S.wsum[w];
+                if (w < warp) wb += S.wsum[k][w];
+                tot += S.wsum[k][w];
             }
-            uint32_t e = base + wb + incl - v;
+            uint32_t e = base + wb + ent0[k];
             const uint32_t nodev = (uint32_t)(k * kPreThreads + tid);
             for (uint32_t mm = mask[k]; mm; mm &= mm - 1)
                 S.ent[e++] = (uint16_t)((nodev << 4) | (uint32_t)(__ffs(mm) - 1));
             base += tot;
-            __syncthreads();   // S.wsum is reused by the next item
         }
+        __syncthreads();
         const int nent = (int)base;
         // phase B: preprocess every (node, camera) candidate straight into its slot
         for (int e = tid; e < nent; e += kPreThreads) {
