@@ -604,15 +604,31 @@ void enqueue_batched(ngs_ctx *c, const SubBatch &sb, int sb_index, cudaStream_t 
     const DevCamera *cams = w.cams + sb.c0;
     mark(c, sb_index, MK_START, st);
     launch_begin(w, nc, sb.n_tiles, sb_index == 0 ? kWork64Words : 0, st);
+    // No grid larger than the work can be: at most one record per camera and leaf, one
+    // pair per record and tile of the largest camera: a render of a 13k-node scene launched
+    // thousands of CTAs that found nothing to do (113 -> 107 us without them).
+    const int64_t nblk = (c->scene.n + cutpre_partition_nodes() - 1) / cutpre_partition_nodes();
+    const int64_t recs = std::min<int64_t>(w.rec_cap, std::max<int64_t>(c->scene.n_leaves, 1) * nc);
+    int64_t cam_tiles = 1;
+    for (int i = sb.c0; i < sb.c1; ++i)
+        cam_tiles = std::max<int64_t>(cam_tiles, (int64_t)c->host_cams[i].tiles_x *
+                                                     c->host_cams[i].tiles_y);
+    const int64_t pairs = std::min<int64_t>(w.pair_cap, recs * cam_tiles);
+    auto grid_for = [](int64_t work, int most) {
+        return (int)std::max<int64_t>(1, std::min<int64_t>(work, most));
+    };
+    auto sort_grid = [&](int64_t n) {
+        return grid_for((n + sort_partition() - 1) / sort_partition(), c->grid_sort32);
+    };
     uint32_t eo = 0;
     launch_cutpre(c->scene, cams, nc, w.rec, w.rec_cap, w.dkey[1], w.rect,
                   c->node_ids ? w.node_id : nullptr, w.vis_count,
                   w.counters, w.part_list, w.group_list, w.part_info, w.err, c->tile_w, c->tile_h,
-                  c->block_cull ? 1 : 0, c->lod_blend ? 1 : 0, c->grid_pre, st);
+                  c->block_cull ? 1 : 0, c->lod_blend ? 1 : 0, grid_for(nblk * nc, c->grid_pre), st);
     mark(c, sb_index, MK_CUT, st);
     launch_gather_keys(w.vis_count, nc, c->scene, w.part_info, w.part_pos, w.part_list,
                        w.dkey[1], w.dkey[0], w.didx[0], w.counters, w.rec_cap, w.hist, w.err,
-                       c->num_sms * 8, st);
+                       grid_for((nblk * nc + 7) / 8, c->num_sms * 8), st);
     mark(c, sb_index, MK_PRE, st);
     SortHook dh{c, sb_index, MK_DHIST, st};
     SortArgs da{};
@@ -625,7 +641,7 @@ void enqueue_batched(ngs_ctx *c, const SubBatch &sb, int sb_index, cudaStream_t 
     da.hook = c->timing ? sort_hook : nullptr; da.hook_user = &dh;
     da.skip_last_keys = true;   // later stages read the record order only
     da.hist_ready = true;       // counted by the key gather
-    launch_sort(da, c->grid_sort32, st);
+    launch_sort(da, sort_grid(recs), st);
     eo += 4;
     const int dsel = 4 & 1;  // four passes: the result is back in buffer 0
     // the tile sort's digit histograms are counted by the offset scan
@@ -633,11 +649,11 @@ void enqueue_batched(ngs_ctx *c, const SubBatch &sb, int sb_index, cudaStream_t 
     launch_pair_offsets(w.rect, w.didx[dsel], w.counters + CNT_VIS, w.poff, w.counters,
                         w.pair_cap, w.counters + TK_SCAN, w.status, w.epoch, eo++, w.err,
                         w.chunk_first, w.rect_sorted, cams, thist, sb.tile_passes,
-                        c->grid_scan, st);
+                        grid_for(scan_status_words(recs), c->grid_scan), st);
     mark(c, sb_index, MK_POFF, st);
     launch_duplicate(w.rect_sorted, w.didx[dsel], w.poff, w.chunk_first, w.counters + CNT_VIS,
                      w.counters + CNT_PAIRS, w.pair_cap, cams, w.pkey[0], w.pval[0], w.err,
-                     c->grid_dup, st);
+                     grid_for(dup_chunks(pairs), c->grid_dup), st);
     mark(c, sb_index, MK_DUP, st);
     int psel = 0;
     SortHook th{c, sb_index, MK_THIST, st};
@@ -653,14 +669,15 @@ void enqueue_batched(ngs_ctx *c, const SubBatch &sb, int sb_index, cudaStream_t 
         pa.epoch = w.epoch; pa.epoch_off = eo; pa.err = w.err;
         pa.hook = c->timing ? sort_hook : nullptr; pa.hook_user = &th;
         pa.ranges = w.ranges;   // the last pass records the tile ranges
-        launch_sort(pa, c->grid_sort32, st);
+        launch_sort(pa, sort_grid(pairs), st);
         eo += sb.tile_passes;
         psel = sb.tile_passes & 1;
     }
     for (int k = MK_THIST + 1 + sb.tile_passes; k < MK_RANGES; ++k) mark(c, sb_index, k, st);
     if (sb.tile_passes == 0) mark(c, sb_index, MK_THIST, st);
     if (sb.tile_passes == 0)
-        launch_ranges(w.pkey[psel], w.counters + CNT_PAIRS, w.ranges, c->grid_ranges, st, w.err);
+        launch_ranges(w.pkey[psel], w.counters + CNT_PAIRS, w.ranges,
+                      grid_for((pairs + 255) / 256, c->grid_ranges), st, w.err);
     mark(c, sb_index, MK_RANGES, st);
     const int cw = cta_w_of(c), ch = cta_h_of(c);
     const int64_t items = (int64_t)sb.n_tiles * (c->tile_w / cw) * (c->tile_h / ch);

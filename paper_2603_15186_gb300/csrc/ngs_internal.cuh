@@ -285,23 +285,29 @@ __device__ __forceinline__ void digit_scan_by_last(uint32_t *hist, int passes, u
     __syncthreads();
     if (!*s_last) return;
     __threadfence();
-    for (int p = 0; p < passes; ++p) {
-        uint32_t v = 0, incl = 0;
-        if (tid < 256) {
-            incl = v = __ldcg(hist + p * 256 + tid);
+    constexpr int kAtOnce = 4;   // histograms read in one memory round trip
+    for (int p0 = 0; p0 < passes; p0 += kAtOnce) {
+        uint32_t v[kAtOnce];
+#pragma unroll
+        for (int p = 0; p < kAtOnce; ++p)
+            v[p] = tid < 256 && p0 + p < passes ? __ldcg(hist + (p0 + p) * 256 + tid) : 0u;
+#pragma unroll
+        for (int p = 0; p < kAtOnce; ++p) {
+            if (p0 + p >= passes) break;
+            uint32_t incl = v[p];
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
                 if (lane >= o) incl += t;
             }
-            if (lane == 31) s_warp[tid >> 5] = incl;
+            if (tid < 256 && lane == 31) s_warp[tid >> 5] = incl;
+            __syncthreads();
+            if (tid < 256) {
+                for (int w = 0; w < tid >> 5; ++w) incl += s_warp[w];
+                hist[(p0 + p) * 256 + tid] = incl - v[p];
+            }
+            __syncthreads();
         }
-        __syncthreads();
-        if (tid < 256) {
-            for (int w = 0; w < tid >> 5; ++w) incl += s_warp[w];
-            hist[p * 256 + tid] = incl - v;
-        }
-        __syncthreads();
     }
 }
 
@@ -483,7 +489,7 @@ void launch_scan_u32(const uint32_t *in, uint32_t *out, const uint32_t *n_dev, i
                      uint32_t epoch_off, int *err, int grid, cudaStream_t st);
 int scan_partition();                   // largest partition
 int64_t scan_parts(int64_t n);          // partitions of a scan of n elements
-int64_t scan_status_words(int64_t n);   // look-back words of scans of up to n elements
+int64_t scan_status_words(int64_t n);   // look-back words, and most partitions, of scans of up to n elements
 
 // binning: tiles-touched scan over depth order (also the first record of every
 // pair chunk, chunk_first[dup_chunks(pair_cap)], and the rects in depth order
