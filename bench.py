@@ -261,9 +261,10 @@ def stage_bytes(st, n_nodes, n_cams, pixels, tiles, attr="f16"):
         "cut_preprocess": st["sub_batches"] * n_nodes * 32 + V * (rec + 4 + 8),
         "gather_keys": 12 * V,
         "depth_hist": 4 * V,
-        # the last depth pass writes values only; the last tile pass writes
-        # values and each tile's range (8 B per tile) instead of keys
-        "depth_pass0": 16 * V, "depth_pass1": 16 * V, "depth_pass2": 16 * V, "depth_pass3": 12 * V,
+        # the last depth pass (the third: no depth of this scene needs a fourth) writes
+        # values only; the last tile pass writes values and each tile's range (8 B
+        # per tile) instead of keys
+        "depth_pass0": 16 * V, "depth_pass1": 16 * V, "depth_pass2": 12 * V, "depth_pass3": 0,
         # pair offsets: index, gathered 8-byte rect and offset per Gaussian,
         # plus the rect written in depth order for the pair emission, which
         # reads it, the offset and the index back sequentially
@@ -391,8 +392,8 @@ def run_ours(args, world, rank, local, pg):
             # the common path (exponent from per-row coefficients 2, threshold
             # compare 1, threshold factor 1, clamp 1, weight alpha T 1, colour 3,
             # T - alpha T 1, and the stop test's two compares once per group of
-            # four records: 0.5) and one exp2 (a group in which a pixel stops is
-            # redone with the stop factor: extra work on top of this bound)
+            # four records: 0.5) and one exp2 (the later weights of a group in
+            # which a pixel stops are set to 0: extra work on top of this bound)
             sms = torch.cuda.get_device_properties(local).multi_processor_count
             mhz = float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["sm_max_mhz"]) \
                 if os.path.exists(os.path.join(ROOT, "MEASURED_PEAKS.json")) else 2070.0

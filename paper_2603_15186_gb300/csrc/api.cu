@@ -36,6 +36,7 @@ struct SubBatch {
     int c0, c1;          // cameras [c0, c1)
     uint32_t n_tiles;
     int tile_passes;     // radix passes over the tile id
+    bool near_depths;    // three passes over the depth (near_depths) instead of four
 };
 
 float half_to_float(uint16_t h) {
@@ -327,6 +328,7 @@ ngs_status ensure_work(ngs_ctx *c) {
     sw = std::max<int64_t>(sw, (w.rec_cap + scan_partition() - 1) / scan_partition());
     w.status_limit = sw;
     sw = std::max<int64_t>(sw, scan_status_words(w.rec_cap));
+    sw = std::max<int64_t>(sw, (w.rec_cap + 8191) / 8192 * 512);   // depth sort, 512 digits
     w.status_words = sw;
     ngs_status st = NGS_OK;
     auto A = [&](ngs_status s) { if (st == NGS_OK) st = s; };
@@ -557,6 +559,23 @@ int bits_for(uint32_t n) {
     return b;
 }
 
+// Whether no view depth of the camera can reach kDepthNear: the depth of every mean (and
+// of every blend of two) is at most that of the means' bounds' farthest corner.
+bool near_depths(const ngs_ctx *c, const DevCamera &d) {
+    double z = 0.0;
+    for (int k = 0; k < 3; ++k)
+        z += std::fabs(d.R[6 + k]) * std::max(std::fabs((double)c->scene.mean_lo[k] - d.pos[k]),
+                                              std::fabs((double)c->scene.mean_hi[k] - d.pos[k]));
+    return z * (1.0 + 1e-5) < kDepthNear;   // false for NaN
+}
+
+void set_depth_bits(SortArgs &a, bool near) {
+    a.key_bytes = 4;
+    a.begin_bit = 0;
+    a.end_bit = near ? 27 : 32;
+    a.digit_bits = near ? 9 : 8;
+}
+
 // Splits cameras into sub-batches: at most kMaxCamsPerBatch cameras, at most
 // max_tiles tiles (one camera alone may exceed it), cut and record bounds
 // (a camera's cut is an antichain of the tree, so it holds at most as many
@@ -572,7 +591,7 @@ std::vector<SubBatch> plan(ngs_ctx *c, std::vector<DevCamera> &cams, int max_cam
     int i = 0;
     const int N = (int)cams.size();
     while (i < N) {
-        SubBatch sb{i, i, 0, 0};
+        SubBatch sb{i, i, 0, 0, true};
         int64_t tiles = 0;
         double pairs = 0;
         while (sb.c1 < N) {
@@ -584,6 +603,7 @@ std::vector<SubBatch> plan(ngs_ctx *c, std::vector<DevCamera> &cams, int max_cam
                             cnt + 1 > cams_by_cut || pairs + p > (double)c->w.pair_cap))
                 break;
             cams[sb.c1].tile_base = (uint32_t)tiles;
+            sb.near_depths = sb.near_depths && near_depths(c, d);
             tiles += t;
             pairs += p;
             ++sb.c1;
@@ -627,15 +647,15 @@ void enqueue_batched(ngs_ctx *c, const SubBatch &sb, int sb_index, cudaStream_t 
                   c->block_cull ? 1 : 0, c->lod_blend ? 1 : 0, grid_for(nblk * nc, c->grid_pre), st);
     mark(c, sb_index, MK_CUT, st);
     launch_gather_keys(w.vis_count, nc, c->scene, w.part_info, w.part_pos, w.part_list,
-                       w.dkey[1], w.dkey[0], w.didx[0], w.counters, w.rec_cap, w.hist, w.err,
-                       grid_for((nblk * nc + 7) / 8, c->num_sms * 8), st);
+                       w.dkey[1], w.dkey[0], w.didx[0], w.counters, w.rec_cap, w.hist, sb.near_depths,
+                       w.err, grid_for((nblk * nc + 7) / 8, c->num_sms * 8), st);
     mark(c, sb_index, MK_PRE, st);
     SortHook dh{c, sb_index, MK_DHIST, st};
     SortArgs da{};
     da.keys[0] = w.dkey[0]; da.keys[1] = w.dkey[1];
     da.vals[0] = w.didx[0]; da.vals[1] = w.didx[1];
     da.n_dev = w.counters + CNT_VIS; da.n_host = -1; da.n_max = w.rec_cap;
-    da.key_bytes = 4; da.begin_bit = 0; da.end_bit = 32; da.vals_identity = false;
+    set_depth_bits(da, sb.near_depths);
     da.hist = w.hist; da.tickets = w.counters + TK_SORT0; da.status = w.status;
     da.epoch = w.epoch; da.epoch_off = eo; da.err = w.err;
     da.hook = c->timing ? sort_hook : nullptr; da.hook_user = &dh;
@@ -643,7 +663,8 @@ void enqueue_batched(ngs_ctx *c, const SubBatch &sb, int sb_index, cudaStream_t 
     da.hist_ready = true;       // counted by the key gather
     launch_sort(da, sort_grid(recs), st);
     eo += 4;
-    const int dsel = 4 & 1;  // four passes: the result is back in buffer 0
+    const int dsel = sb.near_depths ? 1 : 0;   // three or four passes
+    if (sb.near_depths) mark(c, sb_index, MK_DPASS0 + 3, st);
     // the tile sort's digit histograms are counted by the offset scan
     uint32_t *thist = w.hist + kTileHist;
     launch_pair_offsets(w.rect, w.didx[dsel], w.counters + CNT_VIS, w.poff, w.counters,
@@ -663,7 +684,7 @@ void enqueue_batched(ngs_ctx *c, const SubBatch &sb, int sb_index, cudaStream_t 
         pa.vals[0] = w.pval[0]; pa.vals[1] = w.pval[1];
         pa.n_dev = w.counters + CNT_PAIRS; pa.n_host = -1; pa.n_max = w.pair_cap;
         pa.key_bytes = 4; pa.begin_bit = 0; pa.end_bit = 8 * sb.tile_passes;
-        pa.vals_identity = false;
+        pa.digit_bits = 8;
         pa.hist_ready = true;   // counted by the offset scan
         pa.hist = thist; pa.tickets = w.counters + TK_SORT0 + 4; pa.status = w.status;
         pa.epoch = w.epoch; pa.epoch_off = eo; pa.err = w.err;
@@ -700,12 +721,12 @@ void enqueue_batched(ngs_ctx *c, const SubBatch &sb, int sb_index, cudaStream_t 
 
 int kernels_of(const SubBatch &sb, bool batched, bool order) {
     // start, live partitions, fused cut + preprocess, partition scan and key
-    // gather (which also counts the depth histograms); depth sort (4 passes);
+    // gather (which also counts the depth histograms); depth sort (3 or 4 passes);
     // pair offsets, duplication; tile sort (the last pass writing the tile
     // ranges) or, with a single tile, the ranges kernel; compositing; and in the
     // batched path the tile order, or else the stats copy
     (void)order;
-    return 5 + 4 + 2 + std::max(sb.tile_passes, 1) + 1 + (batched ? 1 : 0);
+    return 5 + (sb.near_depths ? 3 : 4) + 2 + std::max(sb.tile_passes, 1) + 1 + (batched ? 1 : 0);
 }
 
 ngs_status check_err(ngs_ctx *c) {
@@ -766,11 +787,12 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
     if (es0 != NGS_OK) return es0;
     c->kernels_per_render = 0;
     for (int ci = 0; ci < n_cams; ++ci) {
-        SubBatch sb{ci, ci + 1, 0, 0};
+        SubBatch sb{ci, ci + 1, 0, 0, false};
         DevCamera &d = c->host_cams[ci];
         d.tile_base = 0;
         sb.n_tiles = (uint32_t)d.tiles_x * d.tiles_y;
         sb.tile_passes = (bits_for(sb.n_tiles) + 7) / 8;
+        sb.near_depths = near_depths(c, d);
         CK(cudaMemcpyAsync(w.cams + ci, &d, sizeof(DevCamera), cudaMemcpyHostToDevice, st));
         const DevCamera *cams = w.cams + ci;
         ngs_status es = epoch_guard(c, st, kEpochStride);
@@ -787,7 +809,8 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
         eo++;
         mark(c, ci, MK_CUT, st);
         launch_gather_keys(w.vis_count, 1, c->scene, w.part_info, w.part_pos, w.part_list,
-                           w.dkey[1], w.dkey[0], w.didx[0], w.counters, w.rec_cap, w.hist, w.err,
+                           w.dkey[1], w.dkey[0], w.didx[0], w.counters, w.rec_cap, w.hist,
+                           sb.near_depths, w.err,
                            (int)std::max<int64_t>(1, std::min<int64_t>(nblk / 8 + 1,
                                                                        8 * c->num_sms)), st);
         mark(c, ci, MK_PRE, st);
@@ -802,7 +825,7 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
         da.keys[0] = w.dkey[0]; da.keys[1] = w.dkey[1];
         da.vals[0] = w.didx[0]; da.vals[1] = w.didx[1];
         da.n_dev = nullptr; da.n_host = n_vis; da.n_max = w.rec_cap;
-        da.key_bytes = 4; da.begin_bit = 0; da.end_bit = 32; da.vals_identity = false;
+        set_depth_bits(da, sb.near_depths);
         da.hist = w.hist; da.tickets = w.counters + TK_SORT0; da.status = w.status;
         da.epoch = w.epoch; da.epoch_off = eo; da.err = w.err;
         SortHook dh{c, ci, MK_DHIST, st};
@@ -811,9 +834,11 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
         da.hist_ready = true;       // counted by the key gather
         launch_sort(da, std::min(gsort_v, c->grid_sort32), st);
         eo += 4;
+        const int dsel = sb.near_depths ? 1 : 0;   // three or four passes
+        if (sb.near_depths) mark(c, ci, MK_DPASS0 + 3, st);
         const int gscan = (int)std::max<int64_t>(1, scan_parts(n_vis));
         uint32_t *thist = w.hist + kTileHist;
-        launch_pair_offsets(w.rect, w.didx[0], w.counters + CNT_VIS, w.poff, w.counters,
+        launch_pair_offsets(w.rect, w.didx[dsel], w.counters + CNT_VIS, w.poff, w.counters,
                             w.pair_cap, w.counters + TK_SCAN, w.status, w.epoch, eo++, w.err,
                             w.chunk_first, w.rect_sorted, cams, thist, sb.tile_passes, gscan,
                             st);
@@ -823,7 +848,7 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
         if ((int64_t)n_pairs > w.pair_cap) return NGS_ERR_CAPACITY;
         const int gdup = (int)std::max<int64_t>(
             1, std::min<int64_t>(((int64_t)n_pairs + 2047) / 2048, 8 * (int64_t)c->num_sms));
-        launch_duplicate(w.rect_sorted, w.didx[0], w.poff, w.chunk_first, w.counters + CNT_VIS,
+        launch_duplicate(w.rect_sorted, w.didx[dsel], w.poff, w.chunk_first, w.counters + CNT_VIS,
                          w.counters + CNT_PAIRS, w.pair_cap, cams, w.pkey[0], w.pval[0], w.err,
                          gdup, st);
         mark(c, ci, MK_DUP, st);
@@ -837,7 +862,7 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
             pa.vals[0] = w.pval[0]; pa.vals[1] = w.pval[1];
             pa.n_dev = nullptr; pa.n_host = n_pairs; pa.n_max = w.pair_cap;
             pa.key_bytes = 4; pa.begin_bit = 0; pa.end_bit = 8 * sb.tile_passes;
-            pa.vals_identity = false;
+            pa.digit_bits = 8;
             pa.hist_ready = true;   // counted by the offset scan
             pa.hist = thist; pa.tickets = w.counters + TK_SORT0 + 4; pa.status = w.status;
             pa.epoch = w.epoch; pa.epoch_off = eo; pa.err = w.err;
@@ -888,6 +913,7 @@ ngs_status render_batched(ngs_ctx *c, int n_cams, cudaStream_t st) {
     key.push_back(cta_w_of(c)); key.push_back(cta_h_of(c));
     key.push_back(c->lod_blend ? 1 : 0);
     key.push_back(c->composite_order ? 1 : 0);
+    for (const SubBatch &sb : sbs) key.push_back(sb.near_depths ? 1 : 0);
     for (int i = 0; i < n_cams; ++i) {
         key.push_back(c->host_cams[i].width);
         key.push_back(c->host_cams[i].height);
@@ -1290,6 +1316,14 @@ NGS_API ngs_status ngs_load_scene(ngs_ctx *c, const ngs_gaussians *g, const ngs_
     CK(cudaMemcpy(d.blk_hi_b, bhi_b.data(), nb * sizeof(float4), cudaMemcpyHostToDevice));
     d.nblk = nb;
     d.n = n;
+    for (int k = 0; k < 3; ++k) {
+        d.mean_lo[k] = INFINITY;
+        d.mean_hi[k] = -INFINITY;
+        for (int64_t b = 0; b < nb; ++b) {
+            d.mean_lo[k] = std::min(d.mean_lo[k], (&blo[b].x)[k]);
+            d.mean_hi[k] = std::max(d.mean_hi[k], (&bhi[b].x)[k]);
+        }
+    }
     d.n_leaves = 0;
     for (int64_t i = 0; i < n; ++i) d.n_leaves += h->child_count[i] == 0 ? 1 : 0;
     d.attr_dtype = g->attr_dtype;
@@ -1812,7 +1846,7 @@ NGS_API ngs_status ngs_sort_pairs(ngs_ctx *c, void *d_keys, uint32_t *d_vals, in
     a.vals[0] = d_vals; a.vals[1] = c->sort_tmp_vals;
     a.n_dev = nullptr; a.n_host = n; a.n_max = n;
     a.key_bytes = key_bytes; a.begin_bit = begin_bit; a.end_bit = end_bit;
-    a.vals_identity = false;
+    a.digit_bits = 8;
     a.hist = c->w.hist; a.tickets = c->w.counters + TK_SORT0; a.status = c->w.status;
     a.epoch = c->w.epoch; a.epoch_off = 0; a.err = c->w.err;
     const int grid = (int)std::min<int64_t>(parts, key_bytes == 8 ? c->grid_sort64 : c->grid_sort32);

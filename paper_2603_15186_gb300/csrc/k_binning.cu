@@ -333,7 +333,7 @@ k_scan(const uint32_t *__restrict__ in, const uint2 *__restrict__ rect,
             const uint32_t v = S.td.hh[q - 1][tid];
             if (v) atomicAdd(&hist[q * 256 + tid], v);
         }
-        digit_scan_by_last(hist, passes, done, &S.part, S.warp);
+        digit_scan_by_last<256>(hist, passes, done, &S.part, S.warp);
     }
 }
 

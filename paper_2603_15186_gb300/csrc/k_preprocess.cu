@@ -954,21 +954,23 @@ k_part_scan(const uint32_t *__restrict__ vis_count, int n_cams, int64_t nblk,
 // Dense depth-sort input, part 2: one warp per live partition copies the keys
 // of its visible Gaussians (skipping holes) and writes their record indices at
 // the partition's dense position. On the
-// way it counts the digit histograms of the four 8-bit passes of the depth
-// sort into hist[4][256] (zeroed beforehand; the last CTA scans them): positive float depths share
+// way it counts the digit histograms of the depth sort's passes (four of 8 bits, or, with
+// kNear, three of 9 bits on keys less their base) into hist[passes][digits] (zeroed beforehand; the last CTA scans them): positive float depths share
 // their high digits, so a warp whose keys agree on a digit adds its count once
 // instead of contending on one shared-memory counter.
+template <bool kNear>
 __global__ void __launch_bounds__(256)
 k_part_gather(const uint32_t *__restrict__ part_list, int n_cams, int64_t nblk,
               const uint2 *__restrict__ part_info, const uint32_t *__restrict__ part_pos,
               const uint32_t *__restrict__ dkey_sparse, uint32_t *__restrict__ dkey,
               uint32_t *__restrict__ didx, uint32_t *counters, int64_t cap,
               uint32_t *hist, const int *err) {
-    __shared__ uint32_t s_h[4][256];
+    constexpr int kPasses = kNear ? 3 : 4, kBits = kNear ? 9 : 8, kDigits = 1 << kBits;
+    __shared__ uint32_t s_h[kPasses][kDigits];
     __shared__ uint32_t s_last, s_warp[8];
     if (*err) return;
     const int tid = threadIdx.x;
-    for (int i = tid; i < 4 * 256; i += blockDim.x) (&s_h[0][0])[i] = 0;
+    for (int i = tid; i < kPasses * kDigits; i += blockDim.x) (&s_h[0][0])[i] = 0;
     __syncthreads();
     const uint32_t n_live = counters[CNT_LIVE];
     const int lane = tid & 31;
@@ -997,8 +999,8 @@ k_part_gather(const uint32_t *__restrict__ part_list, int n_cams, int64_t nblk,
 #pragma unroll
             for (int u = 0; u < kRows; ++u) {
                 const uint32_t k = k0 + 32 * u + lane;
-                const uint32_t key = keys[u];
-                const bool vis = key != kKeyHole;
+                const bool vis = keys[u] != kKeyHole;
+                const uint32_t key = kNear ? keys[u] - kDepthKeyBase : keys[u];
                 const uint32_t vb = __ballot_sync(0xffffffffu, vis);
                 const int64_t dst = pos + __popc(vb & lanemask_lt());
                 const bool valid = vis && dst < cap;
@@ -1011,8 +1013,8 @@ k_part_gather(const uint32_t *__restrict__ part_list, int n_cams, int64_t nblk,
                 if (vmask) {
                     const int leader = __ffs(vmask) - 1;
 #pragma unroll
-                    for (int qd = 0; qd < 4; ++qd) {
-                        const uint32_t d = (key >> (8 * qd)) & 255u;
+                    for (int qd = 0; qd < kPasses; ++qd) {
+                        const uint32_t d = (key >> (kBits * qd)) & (kDigits - 1u);
                         const uint32_t dl = __shfl_sync(0xffffffffu, d, leader);
                         if (__all_sync(0xffffffffu, !valid || d == dl)) {
                             if (lane == leader) atomicAdd(&s_h[qd][d], (uint32_t)__popc(vmask));
@@ -1025,11 +1027,11 @@ k_part_gather(const uint32_t *__restrict__ part_list, int n_cams, int64_t nblk,
         }
     }
     __syncthreads();
-    for (int i = tid; i < 4 * 256; i += blockDim.x) {
+    for (int i = tid; i < kPasses * kDigits; i += blockDim.x) {
         const uint32_t v = (&s_h[0][0])[i];
         if (v) atomicAdd(&hist[i], v);
     }
-    digit_scan_by_last(hist, 4, counters + CNT_DONE + 1, &s_last, s_warp);
+    digit_scan_by_last<kDigits>(hist, kPasses, counters + CNT_DONE + 1, &s_last, s_warp);
 }
 
 template <bool kBlend>
@@ -1085,13 +1087,14 @@ void launch_cutpre(const SceneDev &sc, const DevCamera *cams, int n_cams, void *
 void launch_gather_keys(const uint32_t *vis_count, int n_cams, const SceneDev &sc,
                         const uint2 *part_info, uint32_t *part_pos, const uint32_t *part_list,
                         const uint32_t *dkey_sparse, uint32_t *dkey, uint32_t *didx,
-                        uint32_t *counters, int64_t cap, uint32_t *hist, int *err, int grid,
-                        cudaStream_t st) {
+                        uint32_t *counters, int64_t cap, uint32_t *hist, bool near, int *err,
+                        int grid, cudaStream_t st) {
     const int64_t nblk = (sc.n + kPrePart - 1) / kPrePart;
     k_part_scan<<<n_cams, 1024, 0, st>>>(vis_count, n_cams, nblk, part_info, part_pos, counters,
                                          cap, err);
-    k_part_gather<<<grid, 256, 0, st>>>(part_list, n_cams, nblk, part_info, part_pos, dkey_sparse,
-                                        dkey, didx, counters, cap, hist, err);
+    auto gather = near ? k_part_gather<true> : k_part_gather<false>;
+    gather<<<grid, 256, 0, st>>>(part_list, n_cams, nblk, part_info, part_pos, dkey_sparse, dkey,
+                                 didx, counters, cap, hist, err);
 }
 
 int cutpre_partition_nodes() { return kPrePart; }

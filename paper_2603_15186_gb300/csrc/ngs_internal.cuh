@@ -39,6 +39,13 @@ constexpr float kLog2AlphaMin = -7.9943534368588578f;
 // margin far above float32 error, so no pixel that could reach 1/255 is lost)
 constexpr float kTileMarginLog2 = 0.014426950408889634f;
 
+// Depth keys are the bits of view depths above kNearZ. Those of depths below 13107 m
+// (kDepthNear) lie within 2^27 of the bits of kNearZ: three 9-bit digits instead of four of
+// 8 bits.
+constexpr uint32_t kDepthKeyBase = 0x3e4ccccdu;   // the bits of kNearZ
+constexpr uint32_t kDepthKeyEnd = kDepthKeyBase + (1u << 27);
+constexpr float kDepthNear = 13100.0f;            // its bits are below kDepthKeyEnd
+
 constexpr uint32_t kNodeCullOpacity = 1u;    // pos4.w flag: 255 * opacity < 1
 
 // error codes latched in the device status word (same values as ngs_status)
@@ -113,6 +120,7 @@ struct SceneDev {
     // selects more Gaussians than this
     int64_t n_leaves = 0;
     int32_t attr_dtype = NGS_F32;
+    float mean_lo[3] = {0.f, 0.f, 0.f}, mean_hi[3] = {0.f, 0.f, 0.f};   // the means' bounds
     float4 *box_lo = nullptr, *box_hi = nullptr, *pos4 = nullptr, *quat = nullptr;
     void *sop = nullptr;     // [n][4] of attr type
     void *sh = nullptr;      // [n][48] of attr type
@@ -272,12 +280,14 @@ __device__ __forceinline__ bool look_back(const uint64_t *status, int64_t part, 
     return true;
 }
 
-// Exclusive prefix over the 256 digits of each of `passes` histograms, by the CTA (of
-// at least 256 threads) that added its counts last; every CTA of the launch calls it
-// after its own. done: one word, zero before the launch. s_last, s_warp: shared, 1 and 8
-// words.
+// Exclusive prefix over the kDigits (256 or 512) digits of each of `passes` histograms,
+// by the CTA (of at least 256 threads) that added its counts last; every CTA of the launch
+// calls it after its own. done: one word, zero before the launch. s_last, s_warp:
+// shared, 1 and 8 words.
+template <int kDigits>
 __device__ __forceinline__ void digit_scan_by_last(uint32_t *hist, int passes, uint32_t *done,
                                                    uint32_t *s_last, uint32_t *s_warp) {
+    constexpr int kPer = kDigits / 256;   // consecutive digits per thread
     const int tid = threadIdx.x, lane = tid & 31;
     __threadfence();
     __syncthreads();
@@ -287,14 +297,20 @@ __device__ __forceinline__ void digit_scan_by_last(uint32_t *hist, int passes, u
     __threadfence();
     constexpr int kAtOnce = 4;   // histograms read in one memory round trip
     for (int p0 = 0; p0 < passes; p0 += kAtOnce) {
-        uint32_t v[kAtOnce];
+        uint32_t v[kAtOnce][kPer];
 #pragma unroll
         for (int p = 0; p < kAtOnce; ++p)
-            v[p] = tid < 256 && p0 + p < passes ? __ldcg(hist + (p0 + p) * 256 + tid) : 0u;
+#pragma unroll
+            for (int k = 0; k < kPer; ++k)
+                v[p][k] = tid < 256 && p0 + p < passes
+                              ? __ldcg(hist + (p0 + p) * kDigits + tid * kPer + k) : 0u;
 #pragma unroll
         for (int p = 0; p < kAtOnce; ++p) {
             if (p0 + p >= passes) break;
-            uint32_t incl = v[p];
+            uint32_t sum = 0;
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) sum += v[p][k];
+            uint32_t incl = sum;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
@@ -304,7 +320,12 @@ __device__ __forceinline__ void digit_scan_by_last(uint32_t *hist, int passes, u
             __syncthreads();
             if (tid < 256) {
                 for (int w = 0; w < tid >> 5; ++w) incl += s_warp[w];
-                hist[(p0 + p) * 256 + tid] = incl - v[p];
+                uint32_t at = incl - sum;
+#pragma unroll
+                for (int k = 0; k < kPer; ++k) {
+                    hist[(p0 + p) * kDigits + tid * kPer + k] = at;
+                    at += v[p][k];
+                }
             }
             __syncthreads();
         }
@@ -375,8 +396,9 @@ struct Work {
     uint32_t *pval[2] = {nullptr, nullptr};
     int64_t pair_cap = 0;
     uint2 *ranges = nullptr;          int64_t ranges_cap = 0;
-    uint32_t *hist = nullptr;         // kHistWords: [4][256] of the depth sort, at kTileHist
-                                      // [3][256] of the tile sort; standalone sorts: [8][256]
+    // kHistWords: [3][512] or [4][256] of the depth sort, at kTileHist [3][256] of the
+    // tile sort; standalone sorts: [8][256]
+    uint32_t *hist = nullptr;
     DevCamera *cams = nullptr;        int64_t cams_cap = 0;
     // compositing work counters: [0] records staged, [1] pixel-Gaussian
     // evaluations, then per sub-batch (up to kTailSlots) the tail words of its
@@ -388,7 +410,8 @@ struct Work {
 constexpr int kTailSlots = 64;
 constexpr int kWork64Words = 2 + 2 * kTailSlots;
 
-constexpr uint32_t kHistWords = 8 * 256, kTileHist = 4 * 256;
+constexpr uint32_t kTileHist = 3 * 512, kHistWords = kTileHist + 3 * 256;
+static_assert(kHistWords >= 8 * 256, "a standalone sort's histograms");
 
 // ticket slots in Work::counters
 enum : int {
@@ -439,13 +462,15 @@ void launch_cutpre(const SceneDev &sc, const DevCamera *cams, int n_cams, void *
 int cutpre_partition_nodes();
 void cutpre_init_attributes();
 // dense depth keys (camera-major, node order) and their record indices for the
-// sort, and the exclusive prefixes of the depth sort's digit histograms in hist[4][256];
+// sort, and the exclusive prefixes of the depth sort's digit histograms: of the bits'
+// four 8-bit digits in hist[4][256], or, near, of the bits less kDepthKeyBase's three
+// 9-bit digits in hist[3][512] (near: every depth is below kDepthNear);
 // counters[CNT_VIS], [CNT_DONE + 1]
 void launch_gather_keys(const uint32_t *vis_count, int n_cams, const SceneDev &sc,
                         const uint2 *part_info, uint32_t *part_pos, const uint32_t *part_list,
                         const uint32_t *dkey_sparse, uint32_t *dkey, uint32_t *didx,
-                        uint32_t *counters, int64_t cap, uint32_t *hist, int *err, int grid,
-                        cudaStream_t st);
+                        uint32_t *counters, int64_t cap, uint32_t *hist, bool near, int *err,
+                        int grid, cudaStream_t st);
 
 // radix sort (onesweep) of (uint32 | uint64 key, uint32 value) pairs; n from
 // device memory (*n_dev) or host (n_host >= 0). Result lands in buffer
@@ -458,9 +483,9 @@ struct SortArgs {
     int64_t n_max;            // bound on n (status array and grid sizing)
     int key_bytes;
     int begin_bit, end_bit;
-    bool vals_identity;       // first pass takes value = input index
+    int digit_bits;           // 8, or 9 (32-bit keys with hist_ready, no ranges)
     bool hist_ready;          // hist already holds the digit counts' exclusive prefixes
-    uint32_t *hist;           // [passes][256]
+    uint32_t *hist;           // [passes][256 or 512]
     // last pass: skip_last_keys writes the values only (the sorted keys are
     // not needed afterwards); a non-null ranges (32-bit tile keys only) also
     // records every key's [first, end) there, encoded as in k_ranges (x holds
@@ -479,7 +504,6 @@ struct SortArgs {
 };
 int sort_passes(int begin_bit, int end_bit);
 int sort_partition();
-size_t sort_smem_bytes(int key_bytes);
 void sort_init_attributes();
 void launch_sort(const SortArgs &a, int grid, cudaStream_t st);
 

@@ -205,3 +205,36 @@ def test_sort_key_widths_share_the_scratch():
         torch.cuda.synchronize()
         assert torch.equal(keys, want) and torch.equal(vals, order.to(torch.int32))
     r.close()
+
+
+@pytest.mark.parametrize("mode", ["batched", "plain"])
+def test_depths_beyond_the_short_keys(mode):
+    """Three passes over 27 bits of depth while no mean can lie 13.1 km away, four over
+    all bits otherwise: large Gaussians 20 and 30 km away are blended behind the near
+    ones and in their order, and the near ones as without them."""
+    import oracle as O
+    from paper_2603_15186_gb300 import Renderer
+    from scenegen import camera_c0, make_uniform_box_scene
+    from scenegen.scene import build_hierarchy
+    near = make_uniform_box_scene(600, seed=12)
+    leaf = near.child_count == 0
+    cam = camera_c0(0.0)
+    r = Renderer(cut_capacity=1 << 20, record_capacity=1 << 20, pair_capacity=1 << 22)
+    r.set_mode(mode)
+    for far in (0, 2):
+        pos = np.concatenate([near.pos[leaf], np.float32([[30_000, 2, 1.2], [20_000, 2, 1.2]])[:far]])
+        quat = np.concatenate([near.quat[leaf], np.float32([[1, 0, 0, 0]] * far).reshape(far, 4)])
+        logs = np.concatenate([near.log_scale[leaf], np.full((far, 3), np.log(4000.0), np.float32)])
+        opac = np.concatenate([near.opacity[leaf], np.full(far, 0.8, np.float32)])
+        sh = np.concatenate([near.sh[leaf], np.zeros((far, 16, 3), np.float32)])
+        for k in range(far):
+            sh[600 + k, 0, k] = 1.5          # red behind green
+        scene = build_hierarchy(pos, quat, logs, opac, sh)
+        r.load_scene(scene)
+        got = r.render([cam])[0].cpu().numpy().astype(np.float64)
+        ref = O.render(scene, cam)
+        ok = ref.flags == 0
+        assert ok.mean() > 0.5 and np.abs(got - ref.image)[:, ok].max() <= 2e-3
+        if far:
+            assert ref.image[1].mean() > ref.image[0].mean()
+    r.close()
