@@ -464,6 +464,8 @@ __device__ __forceinline__ uint32_t length_class(uint2 rg) {
     return 62u - min(62u, 2u * (uint32_t)lg + half);
 }
 
+constexpr int kOrderAtOnce = 4;
+
 __global__ void __launch_bounds__(1024)
 k_tile_order(const uint2 *__restrict__ ranges, uint32_t n_tiles, uint32_t *__restrict__ order,
              const int *err, const uint32_t *counters, uint32_t *stats) {
@@ -472,8 +474,16 @@ k_tile_order(const uint2 *__restrict__ ranges, uint32_t n_tiles, uint32_t *__res
     if (*err) return;
     if (threadIdx.x < 64) s_hist[threadIdx.x] = 0;
     __syncthreads();
-    for (uint32_t t = threadIdx.x; t < n_tiles; t += blockDim.x)
-        atomicAdd(&s_hist[length_class(ranges[t])], 1u);
+    // kOrderAtOnce tiles per thread in one memory round trip
+    for (uint32_t t0 = threadIdx.x; t0 < n_tiles; t0 += kOrderAtOnce * blockDim.x) {
+        uint2 rg[kOrderAtOnce];
+#pragma unroll
+        for (int u = 0; u < kOrderAtOnce; ++u)
+            rg[u] = t0 + u * blockDim.x < n_tiles ? ranges[t0 + u * blockDim.x] : make_uint2(0u, 0u);
+#pragma unroll
+        for (int u = 0; u < kOrderAtOnce; ++u)
+            if (t0 + u * blockDim.x < n_tiles) atomicAdd(&s_hist[length_class(rg[u])], 1u);
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         uint32_t acc = 0;
@@ -483,8 +493,19 @@ k_tile_order(const uint2 *__restrict__ ranges, uint32_t n_tiles, uint32_t *__res
         }
     }
     __syncthreads();
-    for (uint32_t t = threadIdx.x; t < n_tiles; t += blockDim.x)
-        order[atomicAdd(&s_cur[length_class(ranges[t])], 1u)] = t;
+    for (uint32_t t0 = threadIdx.x; t0 < n_tiles; t0 += kOrderAtOnce * blockDim.x) {
+        uint2 rg[kOrderAtOnce];
+#pragma unroll
+        for (int u = 0; u < kOrderAtOnce; ++u)
+            rg[u] = t0 + u * blockDim.x < n_tiles ? ranges[t0 + u * blockDim.x] : make_uint2(0u, 0u);
+        uint32_t at[kOrderAtOnce];
+#pragma unroll
+        for (int u = 0; u < kOrderAtOnce; ++u)
+            if (t0 + u * blockDim.x < n_tiles) at[u] = atomicAdd(&s_cur[length_class(rg[u])], 1u);
+#pragma unroll
+        for (int u = 0; u < kOrderAtOnce; ++u)
+            if (t0 + u * blockDim.x < n_tiles) order[at[u]] = t0 + u * blockDim.x;
+    }
 }
 
 void launch_tile_order(const uint2 *ranges, uint32_t n_tiles, uint32_t *order, const int *err,
