@@ -349,7 +349,10 @@ __device__ __forceinline__ bool look_back_warp(const uint64_t *status, int64_t p
         const uint32_t prefix = __ballot_sync(0xffffffffu, known && flag == kFlagPrefix);
         const int n_known = unknown ? __ffs(unknown) - 1 : 32;
         const int to = prefix ? __ffs(prefix) : 33;    // lanes up to the first prefix
-        acc += __reduce_add_sync(0xffffffffu, lane < min(n_known, to) ? (uint32_t)w : 0u);
+        uint32_t sum = lane < min(n_known, to) ? (uint32_t)w : 0u;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        acc += sum;
         if (to <= n_known) break;
         j -= n_known;
         if (unknown && ++spins > kSpinLimit) {
