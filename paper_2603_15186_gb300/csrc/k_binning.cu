@@ -23,9 +23,8 @@ namespace ngs {
 constexpr int kScanThreads = 256;
 constexpr int kScanItems = 8;
 constexpr int kScanPart = kScanThreads * kScanItems;
-// inputs of up to kScanFew elements (partitions for up to three waves of CTAs) take
-// partitions of 2 elements per thread
-constexpr int kScanItemsFew = 2;
+// inputs of up to kScanFew elements take partitions of 1 element per thread
+constexpr int kScanItemsFew = 1;
 constexpr int64_t kScanFew = 1 << 20;
 
 int scan_partition() { return kScanPart; }
@@ -130,13 +129,13 @@ __device__ __forceinline__ void tile_digits_add(TileDigits &H, uint32_t k0, uint
 // A chain of at most this many partitions (they all run at once) is looked back over
 // by a warp, 32 partitions per round trip; on longer chains, where a look-back ends
 // after a window or two, one thread took 8% less time than a warp.
-constexpr int kScanShortChain = 2048;
+constexpr int kScanShortChain = 4096;
 // Rects of up to this many tile rows are counted by their own thread; a warp that has
 // a larger one deals all its rows to its lanes. 260k records of a 720p view on
 // 16-pixel tiles (25 tiles each, up to 45 rows): 73 us for the kernel with a loop per
-// thread and the chain walked by one thread, 61 us so, and 38 us with partitions of 512
-// records (kScanFew), as the nearest 2048 records alone hold a twentieth of the rows; 473k records of 16 views:
-// 86 us with partitions of 2048, 32 us with 512.
+// thread and the chain walked by one thread, 61 us so. Partitions of few records (kScanFew)
+// spread the nearest, tallest rects: 38 us with 512 records, 30 us with 256 (473k records of
+// 16 views: 86, 32, 25 us; 258k of small views: 18, 17, 19 us).
 constexpr uint32_t kScanFewRows = 4;
 
 struct ScanSmem {

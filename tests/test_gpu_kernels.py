@@ -159,8 +159,8 @@ def test_sort_histogram_sizes(R, key_bytes, n):
     assert torch.equal(keys, want) and torch.equal(vals, order.to(torch.int32))
 
 
-# partitions of 512 elements up to 152 * 2048, of 2048 beyond
-@pytest.mark.parametrize("n", [511, 512, 513, 16_385, 311_296, 311_297, 4_000_001])
+# partitions of 256 elements up to 2^20, of 2048 beyond; chains of more partitions than CTAs
+@pytest.mark.parametrize("n", [255, 256, 257, 8_193, 311_297, 1 << 20, (1 << 20) + 1, 4_000_001])
 def test_scan_partition_sizes(R, n):
     x = torch.randint(0, 1000, (n,), device="cuda", dtype=torch.int32)
     out, total = R.scan_u32(x)
