@@ -165,6 +165,17 @@ k_onesweep(const K *__restrict__ kin, const uint32_t *__restrict__ vin, K *__res
             const int64_t idx = base + i * 32 + lane;
             key[i] = idx < n ? kin[idx] : (K)0;
         }
+        // kOut == 2: the keys come in the order of their lower digits. Where the partition
+        // has one value of them (nearly all of a large sort's), a digit's run is one key's
+        // and the digit's owner records it; else every key looks at its neighbours in the
+        // write-out. 431 M pairs: 2496 us with the look at the neighbours everywhere, 2326 us.
+        K low = 0;
+        bool one_low = false;
+        if (kOut == 2) {
+            const K lows = ((K)1 << shift) - 1;
+            low = kin[part * PART] & lows;
+            one_low = low == (kin[min(n, (part + 1) * PART) - 1] & lows);
+        }
         // rank of each item among the warp's earlier items with its digit:
         // the lanes sharing a digit (peers) are found by one shared-memory OR
         // of the lane bits into the warp's mask of that digit (the lowest
@@ -246,6 +257,14 @@ k_onesweep(const K *__restrict__ kin, const uint32_t *__restrict__ vin, K *__res
                 publish(slot, pack_status(kFlagPrefix, epoch, prev + run));
             }
             S.gstart[tid] = digit_base[tid] + prev - ds;
+            if (kOut == 2 && one_low && run) {
+                const uint32_t g0 = digit_base[tid] + prev;
+                const uint32_t t = (uint32_t)(low | (K)tid << shift);
+                if (g0 < n) {
+                    atomicMax(&ranges[t].x, ~g0);
+                    atomicMax(&ranges[t].y, g0 + min(run, (uint32_t)n - g0));
+                }
+            }
         }
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i)
@@ -262,7 +281,7 @@ k_onesweep(const K *__restrict__ kin, const uint32_t *__restrict__ vin, K *__res
             if (g >= n) continue;
             if (kOut == 0) kout[g] = k;
             vout[g] = S.vals[j];
-            if (kOut == 2) {
+            if (kOut == 2 && !one_low) {
                 const uint32_t t = (uint32_t)k;
                 if (j == 0 || S.keys[j - 1] != k) atomicMax(&ranges[t].x, ~(uint32_t)g);
                 if (j + 1 == cnt || S.keys[j + 1] != k) atomicMax(&ranges[t].y, (uint32_t)g + 1u);

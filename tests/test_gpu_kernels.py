@@ -238,3 +238,28 @@ def test_depths_beyond_the_short_keys(mode):
         if far:
             assert ref.image[1].mean() > ref.image[0].mean()
     r.close()
+
+
+# pairs: less than a partition of the last tile pass; partitions with one value of the
+# tiles' low digit and with several; three passes over 76800 tiles
+@pytest.mark.parametrize("leaves,grow,width,height", [(40, 0.0, 640, 480), (3000, 1.0, 640, 480),
+                                                      (20_000, 1.5, 640, 480), (3000, 1.5, 2560, 1920)])
+def test_tile_ranges_from_the_last_pass(leaves, grow, width, height):
+    from paper_2603_15186_gb300 import Renderer
+    from scenegen import look_camera, make_uniform_box_scene
+    R = Renderer(cut_capacity=1 << 22, record_capacity=1 << 20, pair_capacity=1 << 27)
+    scene = make_uniform_box_scene(leaves, seed=leaves)
+    scene.log_scale[scene.child_count == 0] += np.float32(grow)
+    R.load_scene(scene)
+    cam = look_camera((2.0, 2.0, 1.2), 0.4, width, height, tau=0.0)
+    images = []
+    for t in (8, 32):
+        R.set_tile(t, t)
+        images.append(R.render([cam])[0].clone())
+        ranges, pairs = R.tile_ranges(0, -(-width // t) * -(-height // t), 1 << 27)
+        some = ranges[ranges[:, 1] > ranges[:, 0]]
+        # the tiles' runs lie end to end in tile order
+        assert some[0, 0] == 0 and some[-1, 1] == pairs == R.stats()["pair_total"]
+        assert np.array_equal(some[1:, 0], some[:-1, 1])
+    assert torch.equal(*images)
+    R.close()
