@@ -616,12 +616,20 @@ __device__ __forceinline__ void store_rec(Rec16 *rec, int64_t i, const PreOut &o
 // block through L2. Culled partitions get an empty entry in the partition
 // table.
 constexpr int kGroupCams = 16;
+// A group is one CTA's work, and the ones of blocks close to the cameras are many times
+// the others': with few of them the launch ends waiting for a few CTAs. Groups are
+// therefore of 16, 8, 4, 2 or 1 cameras, the most that leave kGroupsPerCta groups per CTA
+// (nodes are loaded once per group). Cut + preprocess with 0 (always 16), 8, 16, 32 and always
+// 1: eight 333x187 views of a 1M-leaf floor 149, 138, 157, 205, 205 us; 16 blended 640x480
+// views 422, 376, 385, 431, 543 us; 256 mixed views of a 4M-leaf floor 6057 us for the first
+// four (groups of 16), 9897 us with 1.
+constexpr int kGroupsPerCta = 8;
 
 __global__ void k_live_parts(SceneDev sc, const DevCamera *__restrict__ cams, int n_cams,
                              int64_t nblk, uint32_t *__restrict__ part_list,
                              uint2 *__restrict__ group_list, uint2 *__restrict__ part_info,
                              uint32_t *counters, int tile_w, int tile_h, int use_block_cull,
-                             int blend, const int *err) {
+                             int blend, uint32_t group_cams, const int *err) {
     // with level-of-detail blending a node's Gaussian may move toward its
     // parent: the bounds then cover the block's nodes and their parents
     const float4 *__restrict__ blo = blend ? sc.blk_lo_b : sc.blk_lo;
@@ -647,14 +655,22 @@ __global__ void k_live_parts(SceneDev sc, const DevCamera *__restrict__ cams, in
         }
         const uint32_t bal = __ballot_sync(0xffffffffu, live);
         const uint32_t n_lo = __popc(bal & 0xffffu), n_hi = __popc(bal >> 16);
+        const uint32_t g_lo = (n_lo + group_cams - 1) / group_cams,
+                       g_hi = (n_hi + group_cams - 1) / group_cams;
         uint32_t base = 0, gbase = 0;
         if (lane == 0 && bal) {
             base = atomicAdd(&counters[CNT_LIVE], (uint32_t)__popc(bal));
-            gbase = atomicAdd(&counters[CNT_GROUPS], (n_lo ? 1u : 0u) + (n_hi ? 1u : 0u));
-            if (n_lo) group_list[gbase++] = make_uint2(base, n_lo);
-            if (n_hi) group_list[gbase] = make_uint2(base + n_lo, n_hi);
+            gbase = atomicAdd(&counters[CNT_GROUPS], g_lo + g_hi);
         }
         base = __shfl_sync(0xffffffffu, base, 0);
+        gbase = __shfl_sync(0xffffffffu, gbase, 0);
+        // each half's live partitions in groups of equal size, a lane per group
+        const uint32_t n = half ? n_hi : n_lo, g = half ? g_hi : g_lo;
+        if ((uint32_t)hl < g) {
+            const uint32_t size = (n + g - 1) / g, first = min((uint32_t)hl * size, n);
+            group_list[gbase + (half ? g_lo : 0u) + hl] =
+                make_uint2(base + (half ? n_lo : 0u) + first, min(size, n - first));
+        }
         if (live) part_list[base + __popc(bal & lanemask_lt())] = t;
     }
 }
@@ -1092,11 +1108,16 @@ void launch_cutpre(const SceneDev &sc, const DevCamera *cams, int n_cams, void *
                    cudaStream_t st) {
     const int64_t nblk = (sc.n + kPrePart - 1) / kPrePart;
     const int64_t nq = nblk * ((n_cams + kGroupCams - 1) / kGroupCams);
+    int group_cams = kGroupCams;
+    while (group_cams > 1 &&
+           nblk * ((n_cams + group_cams - 1) / group_cams) < (int64_t)kGroupsPerCta * grid)
+        group_cams /= 2;
     // 8 warps per CTA, two (block, camera chunk) items per warp and iteration
     const int lgrid = (int)std::min<int64_t>((nq + 15) / 16, 8 * 1024);
     k_live_parts<<<std::max(lgrid, 1), 256, 0, st>>>(sc, cams, n_cams, nblk, part_list,
                                                      group_list, part_info, counters, tile_w,
-                                                     tile_h, use_block_cull, blend, err);
+                                                     tile_h, use_block_cull, blend,
+                                                     (uint32_t)group_cams, err);
     if (blend)
         launch_cutpre_t<true>(sc, cams, n_cams, rec, rec_cap, dkey_sparse, rect, node_id,
                               vis_count, counters, part_list, group_list, part_info, err,

@@ -263,3 +263,17 @@ def test_tile_ranges_from_the_last_pass(leaves, grow, width, height):
         assert np.array_equal(some[1:, 0], some[:-1, 1])
     assert torch.equal(*images)
     R.close()
+
+
+@pytest.mark.parametrize("n", [2, 16, 64, 70, 140, 290])
+def test_camera_groups_of_all_sizes(R, n):
+    """Cut + preprocess in groups of one to sixteen cameras of a node block (the fewer the
+    cameras, the smaller): the pixels are those of each view alone."""
+    from scenegen import look_camera, make_uniform_box_scene
+    if not hasattr(R, "box120k"):
+        R.box120k = make_uniform_box_scene(120_000, seed=4)
+    R.load_scene(R.box120k)
+    cams = [look_camera((1.0 + 2.0 * k / n, 2.0, 1.2), 0.37 * k, 64, 48, tau=4.0 + k % 5) for k in range(n)]
+    images = [x.clone() for x in R.render(cams)]
+    for k in range(0, n, max(1, n // 12)):
+        assert torch.equal(R.render([cams[k]])[0], images[k]), k
