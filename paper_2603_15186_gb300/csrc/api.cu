@@ -786,6 +786,10 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
     ngs_status es0 = ensure_events(c, n_cams);
     if (es0 != NGS_OK) return es0;
     c->kernels_per_render = 0;
+    // kernel after kernel without a graph: each one's launch overlaps the end of the one
+    // before (four 640x480 views 1170 -> 1086 us); in the batched path's graph the same
+    // changed nothing. Events stand between the kernels of a timed render.
+    const LaunchOn on(st, !c->timing);
     for (int ci = 0; ci < n_cams; ++ci) {
         SubBatch sb{ci, ci + 1, 0, 0, false};
         DevCamera &d = c->host_cams[ci];
@@ -805,14 +809,14 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
                       c->node_ids ? w.node_id : nullptr, w.vis_count,
                       w.counters, w.part_list, w.group_list, w.part_info, w.err, c->tile_w, c->tile_h,
                       c->block_cull ? 1 : 0, c->lod_blend ? 1 : 0,
-                      (int)std::min<int64_t>(nblk, c->grid_pre), st);
+                      (int)std::min<int64_t>(nblk, c->grid_pre), on);
         eo++;
         mark(c, ci, MK_CUT, st);
         launch_gather_keys(w.vis_count, 1, c->scene, w.part_info, w.part_pos, w.part_list,
                            w.dkey[1], w.dkey[0], w.didx[0], w.counters, w.rec_cap, w.hist,
                            sb.near_depths, w.err,
                            (int)std::max<int64_t>(1, std::min<int64_t>(nblk / 8 + 1,
-                                                                       8 * c->num_sms)), st);
+                                                                       8 * c->num_sms)), on);
         mark(c, ci, MK_PRE, st);
         eo++;
         // the counts so far, and the errors (one wait for both)
@@ -832,7 +836,7 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
         da.hook = c->timing ? sort_hook : nullptr; da.hook_user = &dh;
         da.skip_last_keys = true;   // later stages read the record order only
         da.hist_ready = true;       // counted by the key gather
-        launch_sort(da, std::min(gsort_v, c->grid_sort32), st);
+        launch_sort(da, std::min(gsort_v, c->grid_sort32), on);
         eo += 4;
         const int dsel = sb.near_depths ? 1 : 0;   // three or four passes
         if (sb.near_depths) mark(c, ci, MK_DPASS0 + 3, st);
@@ -841,7 +845,7 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
         launch_pair_offsets(w.rect, w.didx[dsel], w.counters + CNT_VIS, w.poff, w.counters,
                             w.pair_cap, w.counters + TK_SCAN, w.status, w.epoch, eo++, w.err,
                             w.chunk_first, w.rect_sorted, cams, thist, sb.tile_passes, gscan,
-                            st);
+                            on);
         mark(c, ci, MK_POFF, st);
         if ((s = read_counts(c, st)) != NGS_OK) return s;
         const uint32_t n_pairs = c->h_counts[CNT_PAIRS];
@@ -850,7 +854,7 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
             1, std::min<int64_t>(((int64_t)n_pairs + 2047) / 2048, 8 * (int64_t)c->num_sms));
         launch_duplicate(w.rect_sorted, w.didx[dsel], w.poff, w.chunk_first, w.counters + CNT_VIS,
                          w.counters + CNT_PAIRS, w.pair_cap, cams, w.pkey[0], w.pval[0], w.err,
-                         gdup, st);
+                         gdup, on);
         mark(c, ci, MK_DUP, st);
         int psel = 0;
         SortHook th{c, ci, MK_THIST, st};
@@ -868,7 +872,7 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
             pa.epoch = w.epoch; pa.epoch_off = eo; pa.err = w.err;
             pa.hook = c->timing ? sort_hook : nullptr; pa.hook_user = &th;
             pa.ranges = w.ranges;   // the last pass records the tile ranges
-            launch_sort(pa, std::min(gsort_p, c->grid_sort32), st);
+            launch_sort(pa, std::min(gsort_p, c->grid_sort32), on);
             eo += sb.tile_passes;
             psel = sb.tile_passes & 1;
         }
@@ -877,14 +881,14 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
         for (int k = MK_THIST + 1 + sb.tile_passes; k < MK_RANGES; ++k) mark(c, ci, k, st);
         if (sb.tile_passes == 0) mark(c, ci, MK_THIST, st);
         if (sb.tile_passes == 0)
-            launch_ranges(w.pkey[psel], w.counters + CNT_PAIRS, w.ranges, grng, st, w.err);
+            launch_ranges(w.pkey[psel], w.counters + CNT_PAIRS, w.ranges, grng, on, w.err);
         mark(c, ci, MK_RANGES, st);
         const int cw = cta_w_of(c), ch = cta_h_of(c);
         const uint32_t items = sb.n_tiles * (uint32_t)((c->tile_w / cw) * (c->tile_h / ch));
         launch_composite(c->scene.attr_dtype, c->tile_w, c->tile_h, cw, ch, c->batch, false,
                          cams, 1, sb.n_tiles, w.ranges, w.pval[psel], w.rec,
                          w.counters + TK_COMPOSITE, (int)std::max<uint32_t>(items, 1), w.err,
-                         w.work64, nullptr, nullptr, st);
+                         w.work64, nullptr, nullptr, on);
         mark(c, ci, MK_COMPOSITE, st);
         CK(cudaGetLastError());
         c->kernels_per_render += kernels_of(sb, false, false);

@@ -293,6 +293,7 @@ k_scan(const uint32_t *__restrict__ in, const uint2 *__restrict__ rect,
        int64_t chunk_cap, uint2 *__restrict__ rect_out, const DevCamera *__restrict__ cams,
        uint32_t *hist, int passes, uint32_t *done) {
     __shared__ ScanSmem S;
+    after_previous();
     if (*err) return;
     const int tid = threadIdx.x;
     if (kGather && hist) {
@@ -349,13 +350,11 @@ void launch_pair_offsets(const uint2 *rect, const uint32_t *sorted_idx, const ui
                          uint32_t *poff, uint32_t *counters, int64_t pair_cap, uint32_t *ticket,
                          uint64_t *status, const uint32_t *epoch, uint32_t epoch_off, int *err,
                          uint32_t *chunk_first, uint2 *rect_sorted, const DevCamera *cams,
-                         uint32_t *hist, int passes, int grid, cudaStream_t st) {
-    k_scan<true><<<grid, kScanThreads, 0, st>>>(nullptr, rect, sorted_idx, poff, n_vis, -1,
-                                                counters + CNT_PAIRS, pair_cap, ticket, status,
-                                                epoch, epoch_off, err, chunk_first,
-                                                dup_chunks(pair_cap), rect_sorted, cams,
-                                                passes > 0 ? hist : nullptr, passes,
-                                                counters + CNT_DONE + 2);
+                         uint32_t *hist, int passes, int grid, const LaunchOn &st) {
+    launch_on(st, k_scan<true>, grid, kScanThreads, 0, nullptr, rect, sorted_idx, poff, n_vis, -1,
+              counters + CNT_PAIRS, pair_cap, ticket, status, epoch, epoch_off, err, chunk_first,
+              dup_chunks(pair_cap), rect_sorted, cams, passes > 0 ? hist : nullptr, passes,
+              counters + CNT_DONE + 2);
 }
 
 // K4: the pair array is cut into chunks of kDupChunk pairs, so every CTA
@@ -385,6 +384,7 @@ k_duplicate(const uint2 *__restrict__ rect_sorted, const uint32_t *__restrict__ 
     __shared__ uint16_t s_map[kDupChunk];  // window index of each pair's record
     __shared__ uint32_t s_warp[kDupThreads / 32];
     static_assert(kDupWindow <= 65536 && kDupChunk % kDupThreads == 0, "map layout");
+    after_previous();
     if (*err) return;
     const uint32_t n_vis = *n_vis_p, n_pairs = *n_pairs_p;
     if ((int64_t)n_pairs > pair_cap) {
@@ -472,9 +472,9 @@ k_duplicate(const uint2 *__restrict__ rect_sorted, const uint32_t *__restrict__ 
 void launch_duplicate(const uint2 *rect_sorted, const uint32_t *sorted_idx, const uint32_t *poff,
                       const uint32_t *chunk_first, const uint32_t *n_vis, const uint32_t *n_pairs,
                       int64_t pair_cap, const DevCamera *cams, uint32_t *pkey, uint32_t *pval,
-                      int *err, int grid, cudaStream_t st) {
-    k_duplicate<<<grid, kDupThreads, 0, st>>>(rect_sorted, sorted_idx, poff, chunk_first, n_vis,
-                                              n_pairs, pair_cap, cams, pkey, pval, err);
+                      int *err, int grid, const LaunchOn &st) {
+    launch_on(st, k_duplicate, grid, kDupThreads, 0, rect_sorted, sorted_idx, poff, chunk_first,
+              n_vis, n_pairs, pair_cap, cams, pkey, pval, err);
 }
 
 // K6: ranges[t] = [first, end) of tile t in the sorted pair keys, stored as
@@ -484,6 +484,7 @@ void launch_duplicate(const uint2 *rect_sorted, const uint32_t *sorted_idx, cons
 // kernel covers sub-batches of a single tile, which need no tile sort.
 __global__ void k_ranges(const uint32_t *__restrict__ pkey, const uint32_t *n_pairs_p,
                          uint2 *__restrict__ ranges, const int *err) {
+    after_previous();
     if (*err) return;
     const int64_t n = *n_pairs_p;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -495,8 +496,8 @@ __global__ void k_ranges(const uint32_t *__restrict__ pkey, const uint32_t *n_pa
 }
 
 void launch_ranges(const uint32_t *pkey, const uint32_t *n_pairs, uint2 *ranges, int grid,
-                   cudaStream_t st, const int *err) {
-    k_ranges<<<grid, 256, 0, st>>>(pkey, n_pairs, ranges, err);
+                   const LaunchOn &st, const int *err) {
+    launch_on(st, k_ranges, grid, 256, 0, pkey, n_pairs, ranges, err);
 }
 
 }  // namespace ngs

@@ -170,6 +170,7 @@ k_composite(const DevCamera *__restrict__ cams, int n_cams, uint32_t n_tiles,
     float4 *s_box = reinterpret_cast<float4 *>(sm + Lay::box_off);
     uint32_t *s_list = reinterpret_cast<uint32_t *>(sm + Lay::list_off);
     __shared__ uint32_t s_tile;
+    after_previous();
     if (*err) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // warp -> WBW x BH pixel block of the tile; thread -> the pixels (lx, ly)
@@ -470,6 +471,7 @@ __global__ void __launch_bounds__(1024)
 k_tile_order(const uint2 *__restrict__ ranges, uint32_t n_tiles, uint32_t *__restrict__ order,
              const int *err, const uint32_t *counters, uint32_t *stats) {
     __shared__ uint32_t s_hist[64], s_cur[64];
+    after_previous();
     if (stats) keep_stats(counters, stats);   // also of a sub-batch that overflowed
     if (*err) return;
     if (threadIdx.x < 64) s_hist[threadIdx.x] = 0;
@@ -509,8 +511,8 @@ k_tile_order(const uint2 *__restrict__ ranges, uint32_t n_tiles, uint32_t *__res
 }
 
 void launch_tile_order(const uint2 *ranges, uint32_t n_tiles, uint32_t *order, const int *err,
-                       const uint32_t *counters, uint32_t *stats, cudaStream_t st) {
-    k_tile_order<<<1, 1024, 0, st>>>(ranges, n_tiles, order, err, counters, stats);
+                       const uint32_t *counters, uint32_t *stats, const LaunchOn &st) {
+    launch_on(st, k_tile_order, 1, 1024, 0, ranges, n_tiles, order, err, counters, stats);
 }
 
 template <typename R, int TW, int TH, int BATCH>
@@ -553,15 +555,15 @@ struct CompLaunch {
     int sub_x, sub_y;
     const uint32_t *order;
     unsigned long long *tail;
-    cudaStream_t st;
+    LaunchOn st;
 };
 
 template <typename R, int TW, int TH, int BATCH>
 static void launch_one(const CompLaunch &a) {
-    k_composite<R, TW, TH, BATCH>
-        <<<a.grid, CompLayout<R, TW, TH, BATCH>::NT, comp_smem<R, TW, TH, BATCH>(), a.st>>>(
-            a.cams, a.n_cams, a.n_tiles, a.ranges, a.pval, (const R *)a.rec, a.ticket,
-            a.persistent, a.err, a.work64, a.sub_x, a.sub_y, a.order, a.tail);
+    launch_on(a.st, k_composite<R, TW, TH, BATCH>, a.grid, CompLayout<R, TW, TH, BATCH>::NT,
+              comp_smem<R, TW, TH, BATCH>(), a.cams, a.n_cams, a.n_tiles, a.ranges, a.pval,
+              (const R *)a.rec, a.ticket, a.persistent, a.err, a.work64, a.sub_x, a.sub_y, a.order,
+              a.tail);
 }
 
 template <typename R, int TW, int TH>
@@ -585,7 +587,7 @@ void launch_composite(int attr_dtype, int tile_w, int tile_h, int cta_w, int cta
                       bool persistent, const DevCamera *cams, int n_cams, uint32_t n_tiles,
                       const uint2 *ranges, const uint32_t *pval, const void *rec,
                       uint32_t *ticket, int grid, const int *err, unsigned long long *work64,
-                      const uint32_t *order, unsigned long long *tail, cudaStream_t st) {
+                      const uint32_t *order, unsigned long long *tail, const LaunchOn &st) {
     const CompLaunch a{cams, n_cams, n_tiles, ranges, pval, rec, ticket, persistent ? 1 : 0,
                        grid, err, work64, tile_w / cta_w, tile_h / cta_h, order, tail, st};
     if (attr_dtype == NGS_F32) launch_r<Rec32>(cta_w, cta_h, batch, a);

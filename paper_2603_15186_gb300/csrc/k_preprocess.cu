@@ -634,6 +634,7 @@ __global__ void k_live_parts(SceneDev sc, const DevCamera *__restrict__ cams, in
     // parent: the bounds then cover the block's nodes and their parents
     const float4 *__restrict__ blo = blend ? sc.blk_lo_b : sc.blk_lo;
     const float4 *__restrict__ bhi = blend ? sc.blk_hi_b : sc.blk_hi;
+    after_previous();
     if (*err) return;
     const int lane = threadIdx.x & 31, half = lane >> 4, hl = lane & 15;
     const int64_t nch = (n_cams + kGroupCams - 1) / kGroupCams;
@@ -714,6 +715,7 @@ k_cutpre(SceneDev sc, const DevCamera *__restrict__ cams, int n_cams, R *__restr
          uint2 *__restrict__ part_info, int *err, int tile_w, int tile_h) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     CutPreSmem<R> &S = *reinterpret_cast<CutPreSmem<R> *>(smem_raw);
+    after_previous();
     if (*err) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t nblk = (sc.n + kPrePart - 1) / kPrePart;
@@ -921,6 +923,7 @@ k_part_scan(const uint32_t *__restrict__ vis_count, int n_cams, int64_t nblk,
     __shared__ uint32_t s_val[kScanBlocks + kScanBlocks / 32];
     __shared__ uint32_t s_w[32];
     __shared__ uint32_t s_base, s_total;
+    after_previous();
     if (*err) return;
     const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // exclusive scan of the (at most 1024) per-camera counts
@@ -1007,6 +1010,7 @@ k_part_gather(const uint32_t *__restrict__ part_list, int n_cams, int64_t nblk,
     constexpr int kPasses = kNear ? 3 : 4, kBits = kNear ? 9 : 8, kDigits = 1 << kBits;
     __shared__ uint32_t s_h[kPasses][kDigits];
     __shared__ uint32_t s_last, s_warp[8];
+    after_previous();
     if (*err) return;
     const int tid = threadIdx.x;
     for (int i = tid; i < kPasses * kDigits; i += blockDim.x) (&s_h[0][0])[i] = 0;
@@ -1079,23 +1083,22 @@ static void launch_cutpre_t(const SceneDev &sc, const DevCamera *cams, int n_cam
                             uint32_t *node_id, uint32_t *vis_count, uint32_t *counters,
                             uint32_t *part_list,
                             uint2 *group_list, uint2 *part_info, int *err, int tile_w, int tile_h,
-                            int grid, cudaStream_t st) {
+                            int grid, const LaunchOn &st) {
     switch (sc.attr_dtype) {
     case NGS_F16:
-        k_cutpre<__half, Rec16, kBlend><<<grid, kPreThreads, sizeof(CutPreSmem<Rec16>), st>>>(
-            sc, cams, n_cams, (Rec16 *)rec, rec_cap, dkey_sparse, rect, node_id, vis_count,
-            counters, part_list, group_list, part_info, err, tile_w, tile_h);
+        launch_on(st, k_cutpre<__half, Rec16, kBlend>, grid, kPreThreads, sizeof(CutPreSmem<Rec16>),
+                  sc, cams, n_cams, (Rec16 *)rec, rec_cap, dkey_sparse, rect, node_id, vis_count,
+                  counters, part_list, group_list, part_info, err, tile_w, tile_h);
         break;
     case NGS_BF16:
-        k_cutpre<__nv_bfloat16, Rec16, kBlend>
-            <<<grid, kPreThreads, sizeof(CutPreSmem<Rec16>), st>>>(
-                sc, cams, n_cams, (Rec16 *)rec, rec_cap, dkey_sparse, rect, node_id, vis_count,
-                counters, part_list, group_list, part_info, err, tile_w, tile_h);
+        launch_on(st, k_cutpre<__nv_bfloat16, Rec16, kBlend>, grid, kPreThreads,
+                  sizeof(CutPreSmem<Rec16>), sc, cams, n_cams, (Rec16 *)rec, rec_cap, dkey_sparse,
+                  rect, node_id, vis_count, counters, part_list, group_list, part_info, err, tile_w, tile_h);
         break;
     default:
-        k_cutpre<float, Rec32, kBlend><<<grid, kPreThreads, sizeof(CutPreSmem<Rec32>), st>>>(
-            sc, cams, n_cams, (Rec32 *)rec, rec_cap, dkey_sparse, rect, node_id, vis_count,
-            counters, part_list, group_list, part_info, err, tile_w, tile_h);
+        launch_on(st, k_cutpre<float, Rec32, kBlend>, grid, kPreThreads, sizeof(CutPreSmem<Rec32>),
+                  sc, cams, n_cams, (Rec32 *)rec, rec_cap, dkey_sparse, rect, node_id, vis_count,
+                  counters, part_list, group_list, part_info, err, tile_w, tile_h);
         break;
     }
 }
@@ -1105,7 +1108,7 @@ void launch_cutpre(const SceneDev &sc, const DevCamera *cams, int n_cams, void *
                    uint32_t *vis_count, uint32_t *counters, uint32_t *part_list,
                    uint2 *group_list, uint2 *part_info,
                    int *err, int tile_w, int tile_h, int use_block_cull, int blend, int grid,
-                   cudaStream_t st) {
+                   const LaunchOn &st) {
     const int64_t nblk = (sc.n + kPrePart - 1) / kPrePart;
     const int64_t nq = nblk * ((n_cams + kGroupCams - 1) / kGroupCams);
     int group_cams = kGroupCams;
@@ -1114,7 +1117,7 @@ void launch_cutpre(const SceneDev &sc, const DevCamera *cams, int n_cams, void *
         group_cams /= 2;
     // 8 warps per CTA, two (block, camera chunk) items per warp and iteration
     const int lgrid = (int)std::min<int64_t>((nq + 15) / 16, 8 * 1024);
-    k_live_parts<<<std::max(lgrid, 1), 256, 0, st>>>(sc, cams, n_cams, nblk, part_list,
+    launch_on(st, k_live_parts, std::max(lgrid, 1), 256, 0, sc, cams, n_cams, nblk, part_list,
                                                      group_list, part_info, counters, tile_w,
                                                      tile_h, use_block_cull, blend,
                                                      (uint32_t)group_cams, err);
@@ -1132,13 +1135,13 @@ void launch_gather_keys(const uint32_t *vis_count, int n_cams, const SceneDev &s
                         const uint2 *part_info, uint32_t *part_pos, const uint32_t *part_list,
                         const uint32_t *dkey_sparse, uint32_t *dkey, uint32_t *didx,
                         uint32_t *counters, int64_t cap, uint32_t *hist, bool near, int *err,
-                        int grid, cudaStream_t st) {
+                        int grid, const LaunchOn &st) {
     const int64_t nblk = (sc.n + kPrePart - 1) / kPrePart;
-    k_part_scan<<<n_cams, 1024, 0, st>>>(vis_count, n_cams, nblk, part_info, part_pos, counters,
-                                         cap, err);
+    launch_on(st, k_part_scan, n_cams, 1024, 0, vis_count, n_cams, nblk, part_info, part_pos,
+              counters, cap, err);
     auto gather = near ? k_part_gather<true> : k_part_gather<false>;
-    gather<<<grid, 256, 0, st>>>(part_list, n_cams, nblk, part_info, part_pos, dkey_sparse, dkey,
-                                 didx, counters, cap, hist, err);
+    launch_on(st, gather, grid, 256, 0, part_list, n_cams, nblk, part_info, part_pos, dkey_sparse,
+              dkey, didx, counters, cap, hist, err);
 }
 
 int cutpre_partition_nodes() { return kPrePart; }

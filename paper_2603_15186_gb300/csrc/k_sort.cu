@@ -133,6 +133,7 @@ k_onesweep(const K *__restrict__ kin, const uint32_t *__restrict__ vin, K *__res
     static_assert(kRadix <= kOsThreads, "a thread per digit");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem &S = *reinterpret_cast<Smem *>(smem_raw);
+    after_previous();
     if (*err) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t n = n_dev ? (int64_t)*n_dev : n_host;
@@ -308,22 +309,22 @@ void sort_init_attributes() {
 }
 
 template <typename K, int kOut, int BITS>
-static void launch_pass(int grid, const SortArgs &a, int p, uint32_t mask, cudaStream_t st) {
+static void launch_pass(int grid, const SortArgs &a, int p, uint32_t mask, const LaunchOn &st) {
     const int src = p & 1, dst = src ^ 1;
-    k_onesweep<K, kOut, BITS><<<grid, kOsThreads, sizeof(SortSmem<K, BITS>), st>>>(
+    launch_on(st, k_onesweep<K, kOut, BITS>, grid, kOsThreads, sizeof(SortSmem<K, BITS>),
         (const K *)a.keys[src], a.vals[src], (K *)a.keys[dst], a.vals[dst], a.n_dev, a.n_host,
         a.begin_bit + BITS * p, mask, a.hist + (p << BITS), a.status, a.tickets + p, a.epoch,
         a.epoch_off + p, a.err, a.ranges);
 }
 
 template <typename K, int BITS>
-static void launch_sort_t(const SortArgs &a, int grid, cudaStream_t st) {
+static void launch_sort_t(const SortArgs &a, int grid, const LaunchOn &st) {
     const int passes = (a.end_bit - a.begin_bit + BITS - 1) / BITS;
     if (!a.hist_ready) {
-        cudaMemsetAsync(a.hist, 0, sizeof(uint32_t) * kRadix * passes, st);
+        cudaMemsetAsync(a.hist, 0, sizeof(uint32_t) * kRadix * passes, st.st);
         const int ugrid = (int)std::max<int64_t>(
             1, std::min<int64_t>((a.n_max + kSortThreads * kUp - 1) / (kSortThreads * kUp), 8 * 152));
-        k_upsweep<K><<<ugrid, kSortThreads, 0, st>>>((const K *)a.keys[0], a.n_dev, a.n_host,
+        k_upsweep<K><<<ugrid, kSortThreads, 0, st.st>>>((const K *)a.keys[0], a.n_dev, a.n_host,
                                                      a.begin_bit, a.end_bit, a.hist,
                                                      a.tickets + kMaxPasses, a.err);
     }
@@ -345,7 +346,7 @@ static void launch_sort_t(const SortArgs &a, int grid, cudaStream_t st) {
     }
 }
 
-void launch_sort(const SortArgs &a, int grid, cudaStream_t st) {
+void launch_sort(const SortArgs &a, int grid, const LaunchOn &st) {
     if (a.key_bytes == 8) launch_sort_t<uint64_t, 8>(a, grid, st);
     else if (a.digit_bits == 9) launch_sort_t<uint32_t, 9>(a, grid, st);
     else launch_sort_t<uint32_t, 8>(a, grid, st);

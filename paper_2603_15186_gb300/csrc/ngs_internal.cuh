@@ -439,6 +439,41 @@ __device__ __forceinline__ void keep_stats(const uint32_t *counters, uint32_t *s
 // ---------------------------------------------------------------------------
 // kernel launchers (one translation unit each)
 // ---------------------------------------------------------------------------
+// Where a launch goes. early: its CTAs may take their places while the kernel before it on
+// the stream ends (programmatic dependent launch); they go no further than
+// after_previous() until that kernel is complete and its writes are visible.
+struct LaunchOn {
+    cudaStream_t st;
+    bool early;
+    LaunchOn(cudaStream_t s, bool e = false) : st(s), early(e) {}
+};
+
+template <typename... P, typename... A>
+inline void launch_on(const LaunchOn &on, void (*kernel)(P...), int grid, int block, size_t smem,
+                      A... args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = on.st;
+    cfg.attrs = &at;
+    cfg.numAttrs = on.early ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// First statement of every kernel that launch_on may launch early: nothing before it
+// touches memory, and no CTA leaves before it, so a kernel's completion still means that of
+// all before it. (With griddepcontrol.launch_dependents here, so that the next kernel's CTAs
+// wait beside this one's, 256 mixed views took 38.9 ms instead of 36.8.)
+__device__ __forceinline__ void after_previous() {
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 900
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+#endif
+}
+
 // cut: cameras [0, n_cams) of the table; writes ids (ascending per camera),
 // offsets [n_cams + 1] and counters[CNT_CUT]
 void launch_cut(const SceneDev &sc, const DevCamera *cams, int n_cams, uint32_t *ids,
@@ -461,7 +496,7 @@ void launch_cutpre(const SceneDev &sc, const DevCamera *cams, int n_cams, void *
                    uint32_t *vis_count,
                    uint32_t *counters, uint32_t *part_list, uint2 *group_list, uint2 *part_info,
                    int *err, int tile_w, int tile_h, int use_block_cull, int blend, int grid,
-                   cudaStream_t st);
+                   const LaunchOn &st);
 int cutpre_partition_nodes();
 void cutpre_init_attributes();
 // dense depth keys (camera-major, node order) and their record indices for the
@@ -473,7 +508,7 @@ void launch_gather_keys(const uint32_t *vis_count, int n_cams, const SceneDev &s
                         const uint2 *part_info, uint32_t *part_pos, const uint32_t *part_list,
                         const uint32_t *dkey_sparse, uint32_t *dkey, uint32_t *didx,
                         uint32_t *counters, int64_t cap, uint32_t *hist, bool near, int *err,
-                        int grid, cudaStream_t st);
+                        int grid, const LaunchOn &st);
 
 // radix sort (onesweep) of (uint32 | uint64 key, uint32 value) pairs; n from
 // device memory (*n_dev) or host (n_host >= 0). Result lands in buffer
@@ -508,7 +543,7 @@ struct SortArgs {
 int sort_passes(int begin_bit, int end_bit);
 int sort_partition();
 void sort_init_attributes();
-void launch_sort(const SortArgs &a, int grid, cudaStream_t st);
+void launch_sort(const SortArgs &a, int grid, const LaunchOn &st);
 
 // exclusive scan of uint32 (device-count or host-count)
 void launch_scan_u32(const uint32_t *in, uint32_t *out, const uint32_t *n_dev, int64_t n_host,
@@ -528,16 +563,16 @@ void launch_pair_offsets(const uint2 *rect, const uint32_t *sorted_idx, const ui
                          uint32_t *poff, uint32_t *counters, int64_t pair_cap, uint32_t *ticket,
                          uint64_t *status, const uint32_t *epoch, uint32_t epoch_off, int *err,
                          uint32_t *chunk_first, uint2 *rect_sorted, const DevCamera *cams,
-                         uint32_t *hist, int passes, int grid, cudaStream_t st);
+                         uint32_t *hist, int passes, int grid, const LaunchOn &st);
 int64_t dup_chunks(int64_t pair_cap);
 // emits the pairs from the depth-ordered rects and their record indices
 // (sorted_idx, as given to launch_pair_offsets)
 void launch_duplicate(const uint2 *rect_sorted, const uint32_t *sorted_idx, const uint32_t *poff,
                       const uint32_t *chunk_first, const uint32_t *n_vis, const uint32_t *n_pairs,
                       int64_t pair_cap, const DevCamera *cams, uint32_t *pkey, uint32_t *pval,
-                      int *err, int grid, cudaStream_t st);
+                      int *err, int grid, const LaunchOn &st);
 void launch_ranges(const uint32_t *pkey, const uint32_t *n_pairs, uint2 *ranges, int grid,
-                   cudaStream_t st, const int *err);
+                   const LaunchOn &st, const int *err);
 
 // compositing of tiles [0, n_tiles) of a sub-batch
 // GS-slice occupancy grid (see include/ngs.h, ngs_slice_grid)
@@ -561,11 +596,11 @@ void launch_composite(int attr_dtype, int tile_w, int tile_h, int cta_w, int cta
                       bool persistent, const DevCamera *cams, int n_cams, uint32_t n_tiles,
                       const uint2 *ranges, const uint32_t *pval, const void *rec,
                       uint32_t *ticket, int grid, const int *err, unsigned long long *work64,
-                      const uint32_t *order, unsigned long long *tail, cudaStream_t st);
+                      const uint32_t *order, unsigned long long *tail, const LaunchOn &st);
 // the tiles [0, n_tiles) of a sub-batch, longest list first (classes of half
 // an octave), into order[n_tiles]; with stats, also keep_stats
 void launch_tile_order(const uint2 *ranges, uint32_t n_tiles, uint32_t *order, const int *err,
-                       const uint32_t *counters, uint32_t *stats, cudaStream_t st);
+                       const uint32_t *counters, uint32_t *stats, const LaunchOn &st);
 int composite_blocks_per_sm(int attr_dtype, int tile_w, int tile_h, int batch);
 void composite_init_attributes();
 
