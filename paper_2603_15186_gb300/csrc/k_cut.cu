@@ -226,31 +226,41 @@ k_cut_shared(const float4 *__restrict__ box_lo, const float4 *__restrict__ box_h
 // and use bit masks over the chunk's cameras: N (the camera keeps the node's box and it
 // is not fine enough) and, with kFrustum, V (the camera keeps it).
 //   k_cut_nodes: one lane per camera, 32 / C boxes at a time, so that a ballot is a box's
-//     mask. With kFrustum 32 nodes whose boxes' union every camera culls go without
-//     tests (a box outside a half-space has every box it contains outside too, also in
-//     float32: the tests are monotone in the bounds).
+//     mask. With kFrustum the union of 32 nodes' boxes is tested first, a lane per camera:
+//     those that cull it cull them all (a box outside a half-space has every box it
+//     contains outside too, also in float32: the tests are monotone in the bounds). With
+//     chunks of 32 cameras the others are put side by side, W of them, 32 / W boxes at a
+//     time, where that saves two rounds (with 16 or 8 cameras it cost what it saved).
 //   k_cut_masks: a node's own masks and its parent's. A leaf has N = 0; its V is tested
-//     only for the cameras whose unit wants its parent refined, one lane per leaf, until
-//     a camera of the unit keeps it. A unit's decision is bits: (leaf or no N_n) and
-//     (root or some N_p) and some V_n over the unit's cameras; without kGroups (units of
-//     one camera) that is the same formula on whole masks, and a 32 x 32 bit transpose
-//     turns 32 nodes' masks into the cameras' words.
+//     only for the cameras whose unit wants its parent refined and that keep the parent,
+//     one lane per leaf: with groups each lane takes its own cameras, until one of a unit
+//     keeps the leaf, else the word's cameras in turn. A unit's decision is bits: (leaf or
+//     no N_n) and (root or some N_p) and some V_n over the unit's cameras; without kGroups
+//     (units of one camera) that is the same formula on whole masks, and a 32 x 32 bit
+//     transpose turns 32 nodes' masks into the cameras' words.
 //
 // Bound by the issue of the tests (about 14 instructions for a granularity, 75 for
 // five planes). A test per (node, camera) on the node and on its parent, once to count
 // and once to write, took 683 + 1016 us for 64 plain cuts of 5.25 M nodes, and one
 // thread per node over its group's members 1557 us for 8 frustum-culled cuts of 8
 // cameras each; with the parents tested again for the children of each word 228 us (+ 159
-// us to write 850 MB of ids) and 530 us, with their masks read 172 us (108 + 64) and 433 us (228 + 205).
+// us to write 850 MB of ids) and 530 us, with their masks read 172 us (108 + 64) and 433 us
+// (228 + 205). With live cameras side by side and each lane at its own cameras the call of
+// 8 shared cuts takes 390 - 447 us (by where the cameras are; 515 - 645 before), that of 64
+// culled cuts of one camera each 505 - 588 us (555 - 675).
 constexpr int kCutWords = kCutPart / 32;
 
 template <bool kFrustum, int C>
-__global__ void __launch_bounds__(kCutThreads)
+__global__ void __launch_bounds__(kCutThreads, kFrustum ? 4 : 1)
 k_cut_nodes(const float4 *__restrict__ box_lo, const float4 *__restrict__ box_hi,
             int64_t n_nodes, const CutCam *__restrict__ cams, const CutChunk *__restrict__ chunks,
             int n_chunks, uint2 *__restrict__ masks, const int *err) {
-    constexpr int G = 32 / C, kWarps = kCutThreads / 32;
+    constexpr int kWarps = kCutThreads / 32;
     __shared__ float4 s_lo[kWarps][32], s_hi[kWarps][32];   // the boxes under test, per warp
+    constexpr bool kNarrow = kFrustum && C == 32;
+    constexpr int kCamWords = 21;   // the planes, b0, pos, fx, tau
+    __shared__ float s_cam[kNarrow ? kCamWords : 1][C];
+    __shared__ int s_from[kNarrow ? kWarps : 1][32];       // lanes of the cameras under test
     if (*err) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t b = blockIdx.x / n_chunks;
@@ -259,8 +269,24 @@ k_cut_nodes(const float4 *__restrict__ box_lo, const float4 *__restrict__ box_hi
     uint2 *out = masks + k * n_nodes;
     // this lane's camera, and which of the boxes taken at once it tests
     const int cl = lane % C, grp = lane / C;
-    const CutCam cam = cams[ch.cam0 + min(cl, ch.n_cams - 1)];
-    const float tau2 = __fmul_rn(cam.tau, cam.tau);
+    CutCam cam = cams[ch.cam0 + min(cl, ch.n_cams - 1)];
+    float tau2 = __fmul_rn(cam.tau, cam.tau);
+    if (kNarrow) {
+        if (tid < C) {
+            const float *from = reinterpret_cast<const float *>(&cam);
+#pragma unroll
+            for (int k = 0; k < kCamWords; ++k) s_cam[k][tid] = from[k];
+        }
+        __syncthreads();
+    }
+    // camera c of the chunk becomes this lane's
+    auto take = [&](int c) {
+        float *to = reinterpret_cast<float *>(&cam);
+#pragma unroll
+        for (int k = 0; k < kCamWords; ++k) to[k] = s_cam[k][c];
+        tau2 = __fmul_rn(cam.tau, cam.tau);
+    };
+    bool moved = false;   // `cam` is another than cl's
     for (int j = warp; j < kCutWords; j += kWarps) {
         const int64_t node = b * kCutPart + 32 * j + lane;
         const bool valid = node < n_nodes;
@@ -273,7 +299,8 @@ k_cut_nodes(const float4 *__restrict__ box_lo, const float4 *__restrict__ box_hi
         const uint32_t inners = __ballot_sync(0xffffffffu, inner);
         if (inners == 0) continue;
         uint32_t N = 0, V = 0;
-        bool look = true;
+        // the lanes of one camera set that have a box to test
+        uint32_t live = C == 32 ? 0xffffffffu : (1u << C) - 1u;
         if (kFrustum) {
             const float inf = __int_as_float(0x7f800000);
             float4 ulo = inner ? lo : make_float4(inf, inf, inf, 0.f);
@@ -287,18 +314,38 @@ k_cut_nodes(const float4 *__restrict__ box_lo, const float4 *__restrict__ box_hi
                 uhi.y = fmaxf(uhi.y, __shfl_xor_sync(0xffffffffu, uhi.y, o));
                 uhi.z = fmaxf(uhi.z, __shfl_xor_sync(0xffffffffu, uhi.z, o));
             }
-            look = __any_sync(0xffffffffu, cl < ch.n_cams && !frustum_culled(cam, ulo, uhi));
+            if (kNarrow && moved) {
+                take(cl);
+                moved = false;
+            }
+            live &= __ballot_sync(0xffffffffu, cl < ch.n_cams && !frustum_culled(cam, ulo, uhi));
         }
-        if (look) {
+        if (live) {
             const int n = __popc(inners), rank = inner ? __popc(inners & lanemask_lt()) : -1;
             if (inner) {
                 s_lo[warp][rank] = lo;
                 s_hi[warp][rank] = hi;
             }
             __syncwarp();
+            // the cameras that do not cull all of these boxes, W of them (a power of two)
+            // side by side: 32 / W boxes at a time
+            int W = C, box = grp;
+            if (kNarrow) {
+                const int n_live = __popc(live);
+                const int w = n_live == 1 ? 1 : 1 << (32 - __clz(n_live - 1));
+                if ((n * C + 31) / 32 - (n * w + 31) / 32 >= 2) {   // rounds saved
+                    W = w;
+                    if (live >> lane & 1u) s_from[warp][__popc(live & lanemask_lt())] = lane;
+                    __syncwarp();
+                    box = lane / W;
+                    moved = true;
+                    take(s_from[warp][min(lane & (W - 1), n_live - 1)]);
+                }
+            }
+            const int boxes = 32 / W;
 #pragma unroll 2
-            for (int t = 0; t < n; t += G) {
-                const int q = min(t + grp, n - 1);
+            for (int t = 0; t < n; t += boxes) {
+                const int q = min(t + box, n - 1);
                 const float4 l = s_lo[warp][q], h = s_hi[warp][q];
                 const bool keep = !kFrustum || !frustum_culled(cam, l, h);
                 const bool fine = fine_enough_pre(l, h, box_extent(l, h), cam.pos[0], cam.pos[1],
@@ -306,10 +353,21 @@ k_cut_nodes(const float4 *__restrict__ box_lo, const float4 *__restrict__ box_hi
                 const uint32_t nm = __ballot_sync(0xffffffffu, keep && !fine);
                 const uint32_t vm = kFrustum ? __ballot_sync(0xffffffffu, keep) : 0xffffffffu;
                 const int at = rank - t;   // a lane whose box is among these takes its masks
-                if (at >= 0 && at < G) {
-                    N = nm >> (C * at % 32);
-                    V = vm >> (C * at % 32);
+                if (at >= 0 && at < boxes) {
+                    N = nm >> (W * at % 32);
+                    V = vm >> (W * at % 32);
                 }
+            }
+            if (kNarrow && W < C) {   // from the cameras side by side to the chunk's
+                uint32_t n_all = 0, v_all = 0;
+                int k = 0;
+                for (uint32_t m = live; m; m &= m - 1, ++k) {
+                    const int to = __ffs(m) - 1;
+                    n_all |= (N >> k & 1u) << to;
+                    v_all |= (V >> k & 1u) << to;
+                }
+                N = n_all;
+                V = v_all;
             }
             __syncwarp();
         }
@@ -327,7 +385,11 @@ k_cut_masks(const float4 *__restrict__ box_lo, const float4 *__restrict__ box_hi
     constexpr int kWarps = kCutThreads / 32;
     static_assert(kCutWords % kWarps == 0 && kCutWords == 64, "two words per lane");
     __shared__ uint32_t s_word[C][kCutWords + 1];
-    __shared__ CutCam s_cam[kFrustum ? C : 1];
+    // with groups every lane reads the camera that it is at (no bank conflicts by fields)
+    constexpr int kCamWords = 19;   // the planes, b0, pos
+    __shared__ float s_field[kFrustum && kGroups ? kCamWords : 1][C];
+    __shared__ CutCam s_cam[kFrustum && !kGroups ? C : 1];
+    __shared__ uint32_t s_peers[kFrustum && kGroups ? C : 1];   // each camera's unit
     __shared__ uint32_t s_unit[kGroups ? C : 1];   // each unit's cameras of the chunk
     if (*err) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -337,10 +399,20 @@ k_cut_masks(const float4 *__restrict__ box_lo, const float4 *__restrict__ box_hi
     const CutChunk ch = chunks[k];
     const uint2 *mask = masks + k * n_nodes;
     const uint32_t live = ch.n_cams == 32 ? 0xffffffffu : (1u << ch.n_cams) - 1u;
-    if (kFrustum && tid < ch.n_cams) s_cam[tid] = cams[ch.cam0 + tid];
+    if (kFrustum && tid < ch.n_cams) {
+        if (kGroups) {
+            const float *from = reinterpret_cast<const float *>(cams + ch.cam0 + tid);
+#pragma unroll
+            for (int w = 0; w < kCamWords; ++w) s_field[w][tid] = from[w];
+        } else {
+            s_cam[tid] = cams[ch.cam0 + tid];
+        }
+    }
     if (kGroups && tid < ch.n_units) {
         const int g0 = group_begin[ch.unit0 + tid] - ch.cam0, g1 = group_begin[ch.unit0 + tid + 1] - ch.cam0;
         s_unit[tid] = (g1 == 32 ? 0xffffffffu : (1u << g1) - 1u) & ~((1u << g0) - 1u);
+        if (kFrustum)
+            for (int c = g0; c < g1; ++c) s_peers[c] = s_unit[tid];
     }
     __syncthreads();
 #pragma unroll 2
@@ -353,8 +425,16 @@ k_cut_masks(const float4 *__restrict__ box_lo, const float4 *__restrict__ box_hi
             parent = __float_as_int(box_lo[node].w);
             leaf = __float_as_int(box_hi[node].w) == 0;
         }
-        // the root: as if a parent were refined
-        uint32_t Np = !valid ? 0u : parent < 0 ? 0xffffffffu : mask[parent].x;
+        // the parent's N (the root: as if one were refined) and, with groups, V (a unit of
+        // one camera that wants the parent refined keeps it)
+        uint32_t Np, Vp = 0xffffffffu;
+        if (kFrustum && kGroups) {
+            const uint2 up = parent >= 0 ? mask[parent] : make_uint2(valid ? 0xffffffffu : 0u, Vp);
+            Np = up.x;
+            Vp = up.y;
+        } else {
+            Np = !valid ? 0u : parent < 0 ? 0xffffffffu : mask[parent].x;
+        }
         Np &= live;
         // the cameras whose units want the parent refined
         uint32_t want = Np;
@@ -368,20 +448,33 @@ k_cut_masks(const float4 *__restrict__ box_lo, const float4 *__restrict__ box_hi
             uint2 own = make_uint2(0u, kFrustum ? 0u : 0xffffffffu);   // N, V
             if (!leaf && want) own = mask[node];
             if (kFrustum) {
-                // the leaves: a lane each, camera by camera
-                uint32_t need = leaf ? want : 0u;
+                // the leaves: a lane each, but for the cameras that cull its parent (they
+                // cull it too). With groups every lane takes its own cameras, as one that
+                // keeps the leaf ends its unit's; else all have to look, each camera of the
+                // word at a time
+                uint32_t need = leaf ? want & Vp : 0u;
                 float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
                 if (need) {
                     lo = box_lo[node];
                     hi = box_hi[node];
                 }
-                for (uint32_t c = __reduce_or_sync(0xffffffffu, need); c; c &= c - 1) {
-                    const int q = __ffs(c) - 1;
-                    if ((need >> q & 1u) && !frustum_culled(s_cam[q], lo, hi)) {
-                        own.y |= 1u << q;
-                        if (kGroups)   // its unit's other cameras need not look
-                            for (int u = 0; u < ch.n_units; ++u)
-                                if (s_unit[u] >> q & 1u) need &= ~s_unit[u];
+                if (kGroups) {
+                    while (need) {
+                        const int q = __ffs(need) - 1;
+                        need &= need - 1;
+                        CutCam cam;
+                        float *to = reinterpret_cast<float *>(&cam);
+#pragma unroll
+                        for (int w = 0; w < kCamWords; ++w) to[w] = s_field[w][q];
+                        if (!frustum_culled(cam, lo, hi)) {
+                            own.y |= 1u << q;
+                            need &= ~s_peers[q];   // its unit's others need not look
+                        }
+                    }
+                } else {
+                    for (uint32_t c = __reduce_or_sync(0xffffffffu, need); c; c &= c - 1) {
+                        const int q = __ffs(c) - 1;
+                        if ((need >> q & 1u) && !frustum_culled(s_cam[q], lo, hi)) own.y |= 1u << q;
                     }
                 }
             }

@@ -277,3 +277,25 @@ def test_camera_groups_of_all_sizes(R, n):
     images = [x.clone() for x in R.render(cams)]
     for k in range(0, n, max(1, n // 12)):
         assert torch.equal(R.render([cams[k]])[0], images[k]), k
+
+
+@pytest.mark.parametrize("sizes", [[1] * 5, [1] * 16, [1] * 40, [2, 5], [3, 12, 1], [8] * 8, [20, 30, 7]])
+def test_frustum_cuts_of_scattered_cameras(small_floor, sizes):
+    """Cameras that look everywhere, so that none to all of a chunk's keep a word of
+    nodes: the lists of the single-pass kernel."""
+    from paper_2603_15186_gb300 import Renderer
+    from scenegen import look_camera
+    R = Renderer(cut_capacity=1 << 22, record_capacity=1 << 22, pair_capacity=1 << 20)
+    R.load_scene(small_floor)
+    rng = np.random.default_rng(sum(sizes))
+    n = int(sum(sizes))
+    cams = [look_camera((rng.uniform(0.5, 7.5), rng.uniform(0.5, 5.5), 1.2), rng.uniform(-3.1, 3.1), 320,
+                        240, tau=float(rng.uniform(0.0, 30.0))) for _ in range(n + 33)]
+    gb = [0] + list(np.cumsum(sizes))
+    for guard in (0.0, 24.0):
+        ids, off = (t.cpu().numpy() for t in R.select_cut_shared(cams[:n], gb, True, guard))
+        # a group of 33 sends the whole call to the single-pass kernel
+        want, w_off = (t.cpu().numpy() for t in R.select_cut_shared(cams, gb + [n + 33], True, guard))
+        assert np.array_equal(off, w_off[:len(off)]) and np.array_equal(ids[:off[-1]], want[:off[-1]])
+        assert off[-1] > 0
+    R.close()
