@@ -245,9 +245,9 @@ k_cut_shared(const float4 *__restrict__ box_lo, const float4 *__restrict__ box_h
 // thread per node over its group's members 1557 us for 8 frustum-culled cuts of 8
 // cameras each; with the parents tested again for the children of each word 228 us (+ 159
 // us to write 850 MB of ids) and 530 us, with their masks read 172 us (108 + 64) and 433 us
-// (228 + 205). With live cameras side by side and each lane at its own cameras the call of
-// 8 shared cuts takes 390 - 447 us (by where the cameras are; 515 - 645 before), that of 64
-// culled cuts of one camera each 505 - 588 us (555 - 675).
+// (228 + 205). With live cameras side by side and each lane at its own cameras 253 us (139 +
+// 113), and the call of 8 shared cuts takes 390 - 447 us (by where the cameras are; 515 - 645
+// before), that of 64 culled cuts of one camera each 505 - 588 us (555 - 675).
 constexpr int kCutWords = kCutPart / 32;
 
 template <bool kFrustum, int C>
