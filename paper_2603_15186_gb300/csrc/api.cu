@@ -322,19 +322,14 @@ ngs_status ensure_work(ngs_ctx *c) {
     w.ranges_cap = 1 << 24;
     w.cams_cap = kMaxCamsPerCall;
     const int64_t nblk = (c->scene.n + cut_partition_nodes() - 1) / cut_partition_nodes();
-    int64_t sw = std::max<int64_t>(nblk * kMaxCamsPerBatch, 1);
-    sw = std::max<int64_t>(sw, (std::max(w.rec_cap, w.pair_cap) + sort_partition() - 1) /
-                                   sort_partition() * 256);
-    sw = std::max<int64_t>(sw, (w.rec_cap + scan_partition() - 1) / scan_partition());
-    w.status_limit = sw;
-    sw = std::max<int64_t>(sw, scan_status_words(w.rec_cap));
-    sw = std::max<int64_t>(sw, (w.rec_cap + 8191) / 8192 * 512);   // depth sort, 512 digits
-    w.status_words = sw;
+    const LookBack lb = look_back_words(nblk, kMaxCamsPerBatch, w.rec_cap, w.pair_cap);
+    w.status_limit = lb.limit;
+    w.status_words = lb.words;
     ngs_status st = NGS_OK;
     auto A = [&](ngs_status s) { if (st == NGS_OK) st = s; };
     A(dalloc(&w.counters, N_COUNTERS));
     A(dalloc(&w.epoch, 1));
-    A(dalloc(&w.status, (size_t)sw));
+    A(dalloc(&w.status, (size_t)w.status_words));
     A(dalloc(&w.err, 1));
     A(dalloc(&w.cut_ids, (size_t)w.cut_cap));
     A(dalloc(&w.cut_off, kMaxCamsPerBatch + 1));
@@ -373,7 +368,7 @@ ngs_status ensure_work(ngs_ctx *c) {
         free_work(c);
         return st;
     }
-    CK(cudaMemset(w.status, 0, (size_t)sw * sizeof(uint64_t)));
+    CK(cudaMemset(w.status, 0, (size_t)w.status_words * sizeof(uint64_t)));
     CK(cudaMemset(w.epoch, 0, sizeof(uint32_t)));
     CK(cudaMemset(w.err, 0, sizeof(int)));
     CK(cudaMemset(w.counters, 0, N_COUNTERS * sizeof(uint32_t)));
@@ -638,7 +633,7 @@ void enqueue_batched(ngs_ctx *c, const SubBatch &sb, int sb_index, cudaStream_t 
         return (int)std::max<int64_t>(1, std::min<int64_t>(work, most));
     };
     auto sort_grid = [&](int64_t n) {
-        return grid_for((n + sort_partition() - 1) / sort_partition(), c->grid_sort32);
+        return grid_for(parts_of(n, kSortPart), c->grid_sort32);
     };
     uint32_t eo = 0;
     launch_cutpre(c->scene, cams, nc, w.rec, w.rec_cap, w.dkey[1], w.rect,
@@ -823,8 +818,7 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
         ngs_status s = read_counts(c, st);
         if (s != NGS_OK) return s;
         const uint32_t n_cut = c->h_counts[CNT_CUT], n_vis = c->h_counts[CNT_VIS];
-        const int gsort_v = std::max<int64_t>(1, ((int64_t)n_vis + sort_partition() - 1) /
-                                                     sort_partition());
+        const int gsort_v = std::max<int64_t>(1, parts_of(n_vis, kSortPart));
         SortArgs da{};
         da.keys[0] = w.dkey[0]; da.keys[1] = w.dkey[1];
         da.vals[0] = w.didx[0]; da.vals[1] = w.didx[1];
@@ -859,8 +853,7 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
         int psel = 0;
         SortHook th{c, ci, MK_THIST, st};
         if (sb.tile_passes > 0) {
-            const int gsort_p = std::max<int64_t>(1, ((int64_t)n_pairs + sort_partition() - 1) /
-                                                         sort_partition());
+            const int gsort_p = std::max<int64_t>(1, parts_of(n_pairs, kSortPart));
             SortArgs pa{};
             pa.keys[0] = w.pkey[0]; pa.keys[1] = w.pkey[1];
             pa.vals[0] = w.pval[0]; pa.vals[1] = w.pval[1];
@@ -1826,8 +1819,8 @@ NGS_API ngs_status ngs_sort_pairs(ngs_ctx *c, void *d_keys, uint32_t *d_vals, in
     }
     ngs_status s = ensure_work(c);
     if (s != NGS_OK) return s;
-    const int64_t parts = (n + sort_partition() - 1) / sort_partition();
-    if (parts * 256 > c->w.status_limit) return NGS_ERR_CAPACITY;
+    if (!sort_accepted(n, c->w.status_limit)) return NGS_ERR_CAPACITY;
+    const int64_t parts = parts_of(n, kSortPart);
     if (n > c->sort_tmp_cap || (size_t)n * key_bytes > c->sort_tmp_key_bytes) {
         dfree(c->sort_tmp_keys);
         dfree(c->sort_tmp_vals);
@@ -1873,8 +1866,7 @@ NGS_API ngs_status ngs_scan_u32(ngs_ctx *c, const uint32_t *d_in, uint32_t *d_ou
     if (!c->loaded && !c->work_ready) c->scene.n = 1;
     ngs_status s = ensure_work(c);
     if (s != NGS_OK) return s;
-    const int64_t parts = (n + scan_partition() - 1) / scan_partition();
-    if (parts > c->w.status_limit) return NGS_ERR_CAPACITY;
+    if (!scan_accepted(n, c->w.status_limit)) return NGS_ERR_CAPACITY;
     if ((s = epoch_guard(c, st, kEpochStride)) != NGS_OK) return s;
     CK(cudaMemsetAsync(c->w.counters, 0, N_COUNTERS * sizeof(uint32_t), st));
     k_bump_epoch<<<1, 1, 0, st>>>(c->w.epoch, kEpochStride);

@@ -20,22 +20,6 @@
 
 namespace ngs {
 
-constexpr int kScanThreads = 256;
-constexpr int kScanItems = 8;
-constexpr int kScanPart = kScanThreads * kScanItems;
-// inputs of up to kScanFew elements take partitions of 1 element per thread
-constexpr int kScanItemsFew = 1;
-constexpr int64_t kScanFew = 1 << 20;
-
-int scan_partition() { return kScanPart; }
-int64_t scan_parts(int64_t n) {
-    const int64_t part = n <= kScanFew ? kScanThreads * kScanItemsFew : kScanPart;
-    return (n + part - 1) / part;
-}
-int64_t scan_status_words(int64_t n) {
-    return std::max(scan_parts(n), scan_parts(std::min(n, kScanFew)));
-}
-
 // K4 works on chunks of kDupChunk consecutive pairs
 constexpr int kDupThreads = 256;
 constexpr int kDupChunk = 2048;

@@ -34,12 +34,9 @@ namespace ngs {
 
 constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kSortItems = 16;
-constexpr int kSortPart = kSortThreads * kSortItems;   // 4096 keys
 constexpr int kRadix = 256;
 constexpr int kMaxPasses = 8;
 
-int sort_partition() { return kSortPart; }   // smallest partition of any key width
 int sort_passes(int begin_bit, int end_bit) { return (end_bit - begin_bit + 7) / 8; }
 
 template <typename K>
@@ -89,18 +86,12 @@ k_upsweep(const K *__restrict__ keys, const uint32_t *n_dev, int64_t n_host, int
     digit_scan_by_last<kRadix>(hist, passes, done, &s_last, s_warp);
 }
 
-// Partition shape per key width: 512 threads; 16 (32-bit keys) or 8 (64-bit
-// keys) items per thread, i.e. 8192 or 4096 keys per partition.
-template <typename K> struct SortShape;
-template <> struct SortShape<uint32_t> { static constexpr int kItems = 16; };
-template <> struct SortShape<uint64_t> { static constexpr int kItems = 8; };
-constexpr int kOsThreads = 512;
 constexpr int kOsWarps = kOsThreads / 32;
 
 // BITS: digit width, 8 or (depth keys) 9 bits.
 template <typename K, int BITS>
 struct SortSmem {
-    static constexpr int kPart = kOsThreads * SortShape<K>::kItems;
+    static constexpr int kPart = kOsPart<K>;
     static constexpr int kDigits = 1 << BITS;
     uint32_t whist[kOsWarps][kDigits];    // per-warp digit counts, then warp offsets
     // per-warp lane masks of one item's digits (kept 0); 512 digits' share the values'

@@ -19,6 +19,7 @@
 #include <stdint.h>
 
 #include "ngs.h"
+#include "lookback.h"
 
 namespace ngs {
 
@@ -541,7 +542,6 @@ struct SortArgs {
     void *hook_user;
 };
 int sort_passes(int begin_bit, int end_bit);
-int sort_partition();
 void sort_init_attributes();
 void launch_sort(const SortArgs &a, int grid, const LaunchOn &st);
 
@@ -549,9 +549,6 @@ void launch_sort(const SortArgs &a, int grid, const LaunchOn &st);
 void launch_scan_u32(const uint32_t *in, uint32_t *out, const uint32_t *n_dev, int64_t n_host,
                      uint32_t *total, uint32_t *ticket, uint64_t *status, const uint32_t *epoch,
                      uint32_t epoch_off, int *err, int grid, cudaStream_t st);
-int scan_partition();                   // largest partition
-int64_t scan_parts(int64_t n);          // partitions of a scan of n elements
-int64_t scan_status_words(int64_t n);   // look-back words, and most partitions, of scans of up to n elements
 
 // binning: tiles-touched scan over depth order (also the first record of every
 // pair chunk, chunk_first[dup_chunks(pair_cap)], and the rects in depth order

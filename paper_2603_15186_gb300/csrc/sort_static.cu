@@ -146,7 +146,7 @@ extern "C" NGS_API ngs_status ngs_sort_pairs_static(void *d_keys, uint32_t *d_va
     a.tickets = tickets; a.status = status;
     a.epoch = epoch; a.epoch_off = 0; a.err = err;
     a.hook = nullptr; a.hook_user = nullptr;
-    const int64_t parts = (n + sort_partition() - 1) / sort_partition();
+    const int64_t parts = parts_of(n, kSortPart);
     const int grid = (int)std::min<int64_t>(parts, 2 * (int64_t)sms);
     launch_sort(a, grid < 1 ? 1 : grid, st);
     if (passes & 1) {

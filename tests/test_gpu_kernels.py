@@ -170,6 +170,24 @@ def test_scan_partition_sizes(R, n):
     assert torch.equal(out.to(torch.int64) & 0xffffffff, (want - x) & 0xffffffff)
 
 
+def test_scans_on_a_context_of_small_capacities():
+    """A context of few records, without a scene, scans as many elements as any: its
+    look-back words are sized for what it accepts (1024 partitions of 2048, or the 4096
+    of 256 that 2^20 elements take)."""
+    from paper_2603_15186_gb300 import NgsError, Renderer
+    r = Renderer(cut_capacity=1 << 14, record_capacity=1 << 14, pair_capacity=1 << 14)
+    for n in (1, 262_145, 524_289, 1 << 20, (1 << 20) + 1, 1 << 21):
+        x = torch.randint(0, 1000, (n,), device="cuda", dtype=torch.int32)
+        out, total = r.scan_u32(x)
+        torch.cuda.synchronize()
+        want = torch.cumsum(x.to(torch.int64), 0)
+        assert int(total) == int(want[-1]) and torch.equal(out.to(torch.int64), want - x)
+    x = torch.zeros((1 << 21) + 1, device="cuda", dtype=torch.int32)
+    with pytest.raises(NgsError):
+        r.scan_u32(x)
+    r.close()
+
+
 @pytest.mark.parametrize("dtype,tile", [("f32", 16), ("f16", 8)])
 def test_tall_rects_next_to_small_ones(R, dtype, tile):
     """A view from among large Gaussians: rects of one to all of the tile rows in one
