@@ -96,7 +96,9 @@ struct ngs_ctx {
     uint32_t *cut_off32 = nullptr;     // scratch for ngs_select_cut offsets
     CutCam *cut_cams = nullptr;        // ngs_select_cut_shared: cameras and groups
     int32_t *cut_groups = nullptr;
-    CutChunk *cut_chunks = nullptr;    // cuts by masks: chunks of the cameras,
+    CutChunk *cut_chunks = nullptr;    // cuts by masks: chunks of the cameras
+    std::vector<CutChunk> host_chunks; // (their upload may still read it when the call that
+                                       // enqueued it has gone on),
     uint32_t *cut_counts = nullptr;    // (unit, block) counts
     uint32_t *cut_poff = nullptr;      // and their scanned offsets
 
@@ -501,7 +503,8 @@ ngs_status cut_by_masks(ngs_ctx *c, const std::vector<CutCam> &hc, const int32_t
     auto begin = [&](int u) { return group_begin ? group_begin[u] : u; };
     int lanes = n_cams <= 8 ? 8 : n_cams <= 16 ? 16 : 32;
     const int slice = (int)std::min<int64_t>(n_units, cut_slice_units(c));
-    std::vector<CutChunk> chunks;
+    std::vector<CutChunk> &chunks = c->host_chunks;
+    chunks.clear();
     std::vector<int> first_chunk;   // of each slice
     for (int u0 = 0; u0 < n_units; u0 += slice) {
         first_chunk.push_back((int)chunks.size());
