@@ -97,8 +97,9 @@ struct ngs_ctx {
     CutCam *cut_cams = nullptr;        // ngs_select_cut_shared: cameras and groups
     int32_t *cut_groups = nullptr;
     CutChunk *cut_chunks = nullptr;    // cuts by masks: chunks of the cameras
-    std::vector<CutChunk> host_chunks; // (their upload may still read it when the call that
+    CutPlan cut_plan;                  // (their upload may still read it when the call that
                                        // enqueued it has gone on),
+    uint2 *cut_scratch = nullptr;      // masks and words where the record buffer is small,
     uint32_t *cut_counts = nullptr;    // (unit, block) counts
     uint32_t *cut_poff = nullptr;      // and their scanned offsets
 
@@ -230,6 +231,7 @@ void free_work(ngs_ctx *c) {
     dfree(c->cut_cams);
     dfree(c->cut_groups);
     dfree(c->cut_chunks);
+    dfree(c->cut_scratch);
     dfree(c->cut_counts);
     dfree(c->cut_poff);
     c->w = Work();
@@ -238,6 +240,7 @@ void free_work(ngs_ctx *c) {
     c->cut_cams = nullptr;
     c->cut_groups = nullptr;
     c->cut_chunks = nullptr;
+    c->cut_scratch = nullptr;
     c->cut_counts = nullptr;
     c->cut_poff = nullptr;
     c->work_ready = false;
@@ -474,77 +477,75 @@ void fill_cut_cam(CutCam &d, const ngs_camera &k, float guard) {
     d.tau = k.tau;
 }
 
-// Units whose words and nodes' masks fit in the record buffer at once (they live there
-// between the passes of a cut: no render is in flight), each with a chunk of its own.
-int64_t cut_slice_units(const ngs_ctx *c) {
-    return c->w.rec_cap * (int64_t)sizeof(Rec32) /
-           (cut_words_per_unit(c->scene.n) * (int64_t)sizeof(uint32_t) +
-            c->scene.n * (int64_t)sizeof(uint2));
+int64_t cut_mask_bytes(const ngs_ctx *c) { return c->scene.n * (int64_t)sizeof(uint2); }
+int64_t cut_word_bytes(const ngs_ctx *c) {
+    return cut_words_per_unit(c->scene.n) * (int64_t)sizeof(uint32_t);
+}
+
+// Where the masks and words of a cut live between its passes: in the record buffer (no
+// render is in flight), or, where that is too small for any plan (12 bytes a node), in a
+// buffer of that size which the context keeps; null without memory for it. *room: bytes.
+uint2 *cut_room(ngs_ctx *c, int64_t *room) {
+    const int64_t least = cut_least_bytes(cut_mask_bytes(c), cut_word_bytes(c));
+    *room = c->w.rec_cap * (int64_t)sizeof(Rec32);
+    if (*room >= least) return (uint2 *)c->w.rec;
+    *room = least;
+    if (!c->cut_scratch) dalloc(&c->cut_scratch, (size_t)(least / (int64_t)sizeof(uint2)));
+    return c->cut_scratch;
 }
 
 // Whether a cut goes by masks: enough cameras for a lane each, groups that fit a
-// mask, and room for at least one unit's words.
-bool cut_masks_ok(const ngs_ctx *c, int n_cams, const int32_t *group_begin, int n_units) {
-    if (n_cams < kCutMasksMinCams || cut_slice_units(c) < 1) return false;
+// mask, and room for the masks.
+bool cut_masks_ok(ngs_ctx *c, int n_cams, const int32_t *group_begin, int n_units) {
+    if (n_cams < kCutMasksMinCams) return false;
     if (group_begin)
         for (int g = 0; g < n_units; ++g)
             if (group_begin[g + 1] - group_begin[g] > 32) return false;
-    return true;
+    int64_t room;
+    return cut_room(c, &room) != nullptr;
 }
 
 // The cuts of n_units cameras (group_begin null) or groups, enqueued on st: as
-// many units at a time as their mask words fit.
+// many units at a time as their words fit, their chunks as their masks do. 64 cuts of
+// 1.31 M nodes, plain / frustum-culled, us by record capacity: 154 / 274 with 2^26, 149 /
+// 276 with 2^22, 154 / 273 with 2^20, 203 / 376 with 2^17 (the cut's own buffer). With an
+// array of masks reserved for every unit: 153 / 271, 321 / 503, 1020 / 1030, and the
+// single-pass kernels' 849 / 984.
 ngs_status cut_by_masks(ngs_ctx *c, const std::vector<CutCam> &hc, const int32_t *group_begin,
                         int n_units, bool frustum, int32_t *d_ids, int64_t *d_offsets, int64_t cap,
                         cudaStream_t st) {
     Work &w = c->w;
     const SceneDev &sc = c->scene;
     const int n_cams = (int)hc.size();
-    auto begin = [&](int u) { return group_begin ? group_begin[u] : u; };
-    int lanes = n_cams <= 8 ? 8 : n_cams <= 16 ? 16 : 32;
-    const int slice = (int)std::min<int64_t>(n_units, cut_slice_units(c));
-    std::vector<CutChunk> &chunks = c->host_chunks;
-    chunks.clear();
-    std::vector<int> first_chunk;   // of each slice
-    for (int u0 = 0; u0 < n_units; u0 += slice) {
-        first_chunk.push_back((int)chunks.size());
-        const int u1 = std::min(n_units, u0 + slice);
-        for (int u = u0; u < u1;) {
-            CutChunk ch{begin(u), 0, u - u0, 0};
-            while (u < u1 && begin(u + 1) - ch.cam0 <= lanes) {
-                ch.n_cams = begin(u + 1) - ch.cam0;
-                ++ch.n_units;
-                ++u;
-            }
-            chunks.push_back(ch);
-        }
-    }
-    first_chunk.push_back((int)chunks.size());
+    int64_t room;
+    uint2 *masks = cut_room(c, &room);
+    CutPlan &plan = c->cut_plan;
+    plan_cuts(n_cams, group_begin, n_units, cut_mask_bytes(c), cut_word_bytes(c), room, &plan);
     CK(cudaMemcpyAsync(c->cut_cams, hc.data(), sizeof(CutCam) * n_cams, cudaMemcpyHostToDevice,
                        st));
-    CK(cudaMemcpyAsync(c->cut_chunks, chunks.data(), sizeof(CutChunk) * chunks.size(),
+    CK(cudaMemcpyAsync(c->cut_chunks, plan.chunks.data(), sizeof(CutChunk) * plan.chunks.size(),
                        cudaMemcpyHostToDevice, st));
     if (group_begin)
         CK(cudaMemcpyAsync(c->cut_groups, group_begin, sizeof(int32_t) * (n_units + 1),
                            cudaMemcpyHostToDevice, st));
     const int64_t nblk = (sc.n + cut_partition_nodes() - 1) / cut_partition_nodes();
-    uint2 *masks = (uint2 *)w.rec;
-    uint32_t *words = (uint32_t *)(masks + (int64_t)slice * sc.n);
-    for (size_t k = 0; k + 1 < first_chunk.size(); ++k) {
-        const int u0 = (int)k * slice, nu = std::min(slice, n_units - u0);
+    for (size_t k = 0; k < plan.slices.size(); ++k) {
+        const CutSlice &sl = plan.slices[k];
+        uint32_t *words = (uint32_t *)(masks + sl.n_masks * sc.n);
         ngs_status s = epoch_guard(c, st, kEpochStride);
         if (s != NGS_OK) return s;
         CK(cudaMemsetAsync(w.counters, 0, N_COUNTERS * sizeof(uint32_t), st));
         k_bump_epoch<<<1, 1, 0, st>>>(w.epoch, kEpochStride);
-        launch_cut_masks(frustum, group_begin != nullptr, lanes, sc.box_lo, sc.box_hi, sc.n,
-                         c->cut_cams, c->cut_groups + u0, c->cut_chunks + first_chunk[k],
-                         first_chunk[k + 1] - first_chunk[k], masks, words, c->cut_counts, w.err, st);
-        const int64_t np = nblk * nu, sparts = scan_parts(np);
+        for (int j = 0; j < sl.n_chunks; j += sl.n_masks)
+            launch_cut_masks(frustum, group_begin != nullptr, plan.lanes, sc.box_lo, sc.box_hi, sc.n,
+                             c->cut_cams, c->cut_groups + sl.unit0, c->cut_chunks + sl.chunk0 + j,
+                             std::min(sl.n_masks, sl.n_chunks - j), masks, words, c->cut_counts, w.err, st);
+        const int64_t np = nblk * sl.n_units, sparts = scan_parts(np);
         launch_scan_u32(c->cut_counts, c->cut_poff, nullptr, np, c->cut_off32,
                         w.counters + TK_SCAN, w.status, w.epoch, 0, w.err,
                         (int)std::min<int64_t>(sparts, c->grid_scan), st);
-        launch_cut_write(words, c->cut_poff, c->cut_off32, sc.n, nu, k == 0,
-                         k + 2 == first_chunk.size(), cap, (uint32_t *)d_ids, d_offsets + u0,
+        launch_cut_write(words, c->cut_poff, c->cut_off32, sc.n, sl.n_units, k == 0,
+                         k + 1 == plan.slices.size(), cap, (uint32_t *)d_ids, d_offsets + sl.unit0,
                          w.counters, w.err, st);
     }
     CK(cudaGetLastError());

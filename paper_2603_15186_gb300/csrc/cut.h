@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "cut_plan.h"
+
 namespace ngs {
 
 struct DevCamera;
@@ -32,17 +34,12 @@ void launch_cut_shared(bool frustum, const float4 *box_lo, const float4 *box_hi,
                        uint32_t *ticket, uint64_t *status, const uint32_t *epoch,
                        uint32_t epoch_off, int *err, int grid, cudaStream_t st);
 
-// A chunk of a call's cameras, cams[cam0 .. cam0 + n_cams) (at most 32), and its
-// units (cameras or whole groups), unit0 counted within the slice.
-struct CutChunk {
-    int32_t cam0, n_cams, unit0, n_units;
-};
-
-// Cuts of many units, one slice of them at a time: launch_cut_masks decides, for
-// chunks of at most c <= 32 cameras, every (node, unit) into words[unit *
+// Cuts of many units, one slice of them at a time (cut_plan.h): launch_cut_masks
+// decides, for chunks of at most c <= 32 cameras, every (node, unit) into words[unit *
 // cut_words_per_unit() ...] and counts[unit * blocks + block] (blocks of
-// cut_partition_nodes() nodes), with masks[n_chunks][n_nodes] as scratch; after an exclusive scan of the counts into part_off
-// (its sum in *total), launch_cut_write writes the units' offsets (offsets[0] ..
+// cut_partition_nodes() nodes), with masks[n_chunks][n_nodes] as scratch; after all
+// chunks of the slice and an exclusive scan of the counts into part_off (its sum in
+// *total), launch_cut_write writes the units' offsets (offsets[0] ..
 // offsets[n_units], continuing from offsets[0] unless `first`) and ids; with `last`
 // also counters[CNT_CUT], and it latches the capacity error when the ids exceed cap.
 // group_begin (with groups): the slice's entries. Without groups a unit is a camera.

@@ -1,0 +1,66 @@
+// How the cameras of a cut by masks are split: slices of units whose words fit the
+// scratch at once, in each of them chunks of up to 32 cameras with an array of node
+// masks, as many arrays side by side as fit beside the words. Host arithmetic only.
+#ifndef NGS_CUT_PLAN_H
+#define NGS_CUT_PLAN_H
+
+#include <algorithm>
+#include <cstdint>
+#include <vector>
+
+namespace ngs {
+
+// A chunk of a call's cameras, cams[cam0 .. cam0 + n_cams) (at most 32), and its
+// units (cameras or whole groups), unit0 counted within the slice.
+struct CutChunk {
+    int32_t cam0, n_cams, unit0, n_units;
+};
+
+// Units [unit0, unit0 + n_units), of chunks [chunk0, chunk0 + n_chunks), decided n_masks
+// chunks at a time.
+struct CutSlice {
+    int unit0, n_units, chunk0, n_chunks, n_masks;
+};
+
+struct CutPlan {
+    int lanes;      // most cameras of a chunk: 8, 16 or 32
+    std::vector<CutChunk> chunks;
+    std::vector<CutSlice> slices;
+};
+
+// The least scratch: one array of masks and 32 units' words. mask_bytes: of a chunk's
+// array, word_bytes: of a unit's words.
+inline int64_t cut_least_bytes(int64_t mask_bytes, int64_t word_bytes) {
+    return mask_bytes + 32 * word_bytes;
+}
+
+// group_begin null: units of one camera each; groups of up to 32 cameras otherwise.
+// room: the scratch, at least cut_least_bytes. A slice has its own scan of counts and its
+// own write, a further pass of chunks only its two launches: so the words come first.
+inline void plan_cuts(int n_cams, const int32_t *group_begin, int n_units, int64_t mask_bytes,
+                      int64_t word_bytes, int64_t room, CutPlan *p) {
+    auto begin = [&](int u) { return group_begin ? group_begin[u] : u; };
+    p->lanes = n_cams <= 8 ? 8 : n_cams <= 16 ? 16 : 32;
+    p->chunks.clear();
+    p->slices.clear();
+    const int units = (int)std::min<int64_t>(n_units, (room - mask_bytes) / word_bytes);
+    for (int u0 = 0; u0 < n_units; u0 += units) {
+        CutSlice s{u0, std::min(units, n_units - u0), (int)p->chunks.size(), 0, 0};
+        for (int u = u0; u < u0 + s.n_units;) {
+            CutChunk ch{begin(u), 0, u - u0, 0};
+            while (u < u0 + s.n_units && begin(u + 1) - ch.cam0 <= p->lanes) {
+                ch.n_cams = begin(u + 1) - ch.cam0;
+                ++ch.n_units;
+                ++u;
+            }
+            p->chunks.push_back(ch);
+        }
+        s.n_chunks = (int)p->chunks.size() - s.chunk0;
+        s.n_masks = (int)std::min<int64_t>(s.n_chunks, (room - s.n_units * word_bytes) / mask_bytes);
+        p->slices.push_back(s);
+    }
+}
+
+}  // namespace ngs
+
+#endif

@@ -140,6 +140,34 @@ def test_cuts_by_masks_equal_single_pass_cuts(small_floor, floor_views, records)
     R.close()
 
 
+# this scene's masks take 0.6 MB an array, its words 10 KB a unit; records of 48 bytes.
+# 2^16: all words and three arrays; 2^15: one array, several slices; 1: a buffer of the cut's own
+@pytest.mark.parametrize("records", [1 << 16, 1 << 15, 1])
+def test_cuts_in_slices_equal_cuts_at_once(small_floor, floor_views, records):
+    from paper_2603_15186_gb300 import NgsError, Renderer
+    pair = [Renderer(cut_capacity=1 << 22, record_capacity=k, pair_capacity=1 << 20) for k in (1 << 22, records)]
+    for r in pair:
+        r.load_scene(small_floor)
+    rng = np.random.default_rng(6)
+
+    def same(call):
+        (ids, off), (ids1, off1) = (call(r) for r in pair)
+        assert torch.equal(off, off1)
+        assert torch.equal(ids[:int(off[-1])], ids1[:int(off[-1])]) and int(off[-1]) > 0
+
+    for n in (4, 32, 33, 110):
+        same(lambda r: r.select_cut(floor_views[:n]))
+        with pytest.raises(NgsError):
+            pair[1].select_cut(floor_views[:n], cap=100)
+    for frustum in (True, False):
+        for sizes in ([1] * 40, [20] * 5, list(rng.integers(1, 33, 6))):
+            n = int(sum(sizes))
+            gb = [0] + list(np.cumsum(sizes))
+            same(lambda r: r.select_cut_shared((floor_views * 2)[:n], gb, frustum))
+    for r in pair:
+        r.close()
+
+
 # one key into a second partition (4096 or 8192 keys), the keys that the histogram's
 # CTAs take at once (2048) and one more, several rounds of all its CTAs
 @pytest.mark.parametrize("key_bytes,n", [(4, 2048), (4, 2049), (4, 8193), (4, 311_297), (4, 6_000_001),

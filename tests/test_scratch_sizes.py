@@ -58,3 +58,54 @@ int main() {
 """)
     assert n > 100_000 and refused > 1000 and accepted > 1000
     assert short == 0
+
+
+def test_cut_plans_fill_their_slices(tmp_path):
+    """Every unit is in one chunk of one slice, in order; masks and words of a slice fit
+    the room; a slice holds as many units as words fit beside one array of masks (32 at the
+    least room, so that a call of n units takes at most n / 32 slices however small the
+    record buffer is), and its chunks as many arrays as fit then."""
+    calls, slices, bad = run_host(tmp_path, r"""
+#include <cstdio>
+#include <random>
+#include "cut_plan.h"
+using namespace ngs;
+int main() {
+  std::mt19937 rng(1);
+  long calls = 0, slices = 0, bad = 0;
+  for (int64_t nodes : {1, 2049, 1'310'000, 50'000'000}) for (int n_cams : {4, 8, 9, 16, 17, 64, 1023, 1024})
+    for (int most : {1, 3, 20, 32}) for (double scale : {1.0, 1.5, 3.0, 7.9, 40.0, 1e4}) {
+      std::vector<int32_t> begin{0};
+      while (begin.back() < n_cams)
+        begin.push_back(std::min<int>(n_cams, begin.back() + (most == 1 ? 1 : 1 + rng() % most)));
+      const int units = (int)begin.size() - 1;
+      const int64_t mask = 8 * nodes, word = (nodes + 2047) / 2048 * 256;
+      const int64_t room = (int64_t)(cut_least_bytes(mask, word) * scale);
+      CutPlan p;
+      plan_cuts(n_cams, most == 1 ? nullptr : begin.data(), units, mask, word, room, &p);
+      ++calls;
+      slices += (long)p.slices.size();
+      const int64_t full = (room - mask) / word;
+      bad += full < 32 || (int64_t)p.slices.size() != (units + full - 1) / full;
+      int u = 0, chunk = 0;
+      for (const CutSlice &s : p.slices) {
+        bad += s.unit0 != u || s.chunk0 != chunk || s.n_masks < 1 || s.n_masks > s.n_chunks;
+        bad += s.n_masks * mask + s.n_units * word > room;
+        bad += s.n_masks < s.n_chunks && (s.n_masks + 1) * mask + s.n_units * word <= room;
+        for (int k = 0; k < s.n_chunks; ++k, ++chunk) {
+          const CutChunk &c = p.chunks.at(chunk);
+          bad += c.cam0 != begin[u] || c.unit0 != u - s.unit0 || c.n_units < 1 || c.n_cams > p.lanes;
+          bad += c.n_cams != begin[u + c.n_units] - begin[u];
+          u += c.n_units;
+          // no unit of the slice would have fitted too
+          bad += u < s.unit0 + s.n_units && c.n_cams + begin[u + 1] - begin[u] <= p.lanes;
+        }
+        bad += u != s.unit0 + s.n_units;
+      }
+      bad += u != units || chunk != (int)p.chunks.size() || p.lanes > 32 || (p.lanes < n_cams && p.lanes < 32);
+    }
+  std::printf("%ld %ld %ld\n", calls, slices, bad);
+  return 0;
+}
+""")
+    assert calls > 500 and slices > calls and bad == 0
