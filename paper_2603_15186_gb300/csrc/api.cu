@@ -21,11 +21,7 @@ namespace {
 
 constexpr uint32_t kEpochStride = 32;   // epoch values reserved per sub-batch
 constexpr int kMaxCamsPerBatch = 1024;
-// cuts of this many cameras or more (and no group of more than 32) are decided as
-// masks over the cameras, the others by the single-pass kernels. Measured on a 1M-leaf
-// floor, masks / single pass: 4 cameras 93 / 120 us (plain), 117 / 177 us (frustum), 116 /
-// 119 us (one group of 4); the masks' cost is that of 8 cameras for fewer, the single
-// pass takes 73, 87, 110 us for 1, 2, 3
+// fewer cameras go to the single-pass kernels; more by masks where that pays (cut_plan.h)
 constexpr int kCutMasksMinCams = 4;
 constexpr int kMaxCamsPerCall = 1 << 16;
 constexpr int kTuneShapes = NGS_TUNE_SHAPES;
@@ -484,29 +480,35 @@ int64_t cut_word_bytes(const ngs_ctx *c) {
 
 // Where the masks and words of a cut live between its passes: in the record buffer (no
 // render is in flight), or, where that is too small for any plan (12 bytes a node), in a
-// buffer of that size which the context keeps; null without memory for it. *room: bytes.
-uint2 *cut_room(ngs_ctx *c, int64_t *room) {
-    const int64_t least = cut_least_bytes(cut_mask_bytes(c), cut_word_bytes(c));
-    *room = c->w.rec_cap * (int64_t)sizeof(Rec32);
-    if (*room >= least) return (uint2 *)c->w.rec;
-    *room = least;
-    if (!c->cut_scratch) dalloc(&c->cut_scratch, (size_t)(least / (int64_t)sizeof(uint2)));
+// buffer of that size which the context keeps; null without memory for it.
+int64_t cut_room_bytes(const ngs_ctx *c) {
+    return std::max(c->w.rec_cap * (int64_t)sizeof(Rec32),
+                    cut_least_bytes(cut_mask_bytes(c), cut_word_bytes(c)));
+}
+uint2 *cut_room(ngs_ctx *c) {
+    const int64_t room = cut_room_bytes(c);
+    if (room == c->w.rec_cap * (int64_t)sizeof(Rec32)) return (uint2 *)c->w.rec;
+    if (!c->cut_scratch) dalloc(&c->cut_scratch, (size_t)(room / (int64_t)sizeof(uint2)));
     return c->cut_scratch;
 }
 
-// Whether a cut goes by masks: enough cameras for a lane each, groups that fit a
-// mask, and room for the masks.
-bool cut_masks_ok(ngs_ctx *c, int n_cams, const int32_t *group_begin, int n_units) {
+// Whether a cut goes by masks (planned then in c->cut_plan): enough cameras for a lane
+// each, groups that fit a mask, enough work (cut_plan.h), and room for the masks.
+bool cut_masks_ok(ngs_ctx *c, int n_cams, const int32_t *group_begin, int n_units, bool frustum) {
     if (n_cams < kCutMasksMinCams) return false;
-    if (group_begin)
-        for (int g = 0; g < n_units; ++g)
-            if (group_begin[g + 1] - group_begin[g] > 32) return false;
-    int64_t room;
-    return cut_room(c, &room) != nullptr;
+    int largest = 1;
+    for (int g = 0; group_begin && g < n_units; ++g)
+        largest = std::max(largest, group_begin[g + 1] - group_begin[g]);
+    if (largest > 32) return false;
+    plan_cuts(n_cams, group_begin, n_units, cut_mask_bytes(c), cut_word_bytes(c),
+              cut_room_bytes(c), &c->cut_plan);
+    const int64_t nblk = (c->scene.n + cut_partition_nodes() - 1) / cut_partition_nodes();
+    return cut_masks_pay(c->cut_plan, nblk, n_cams, n_units, largest, frustum, c->grid_cut) &&
+           cut_room(c) != nullptr;
 }
 
-// The cuts of n_units cameras (group_begin null) or groups, enqueued on st: as
-// many units at a time as their words fit, their chunks as their masks do. 64 cuts of
+// The cuts of n_units cameras (group_begin null) or groups as c->cut_plan has them, enqueued
+// on st: as many units at a time as their words fit, their chunks as their masks do. 64 cuts of
 // 1.31 M nodes, plain / frustum-culled, us by record capacity: 154 / 274 with 2^26, 149 /
 // 276 with 2^22, 154 / 273 with 2^20, 203 / 376 with 2^17 (the cut's own buffer). With an
 // array of masks reserved for every unit: 153 / 271, 321 / 503, 1020 / 1030, and the
@@ -517,10 +519,8 @@ ngs_status cut_by_masks(ngs_ctx *c, const std::vector<CutCam> &hc, const int32_t
     Work &w = c->w;
     const SceneDev &sc = c->scene;
     const int n_cams = (int)hc.size();
-    int64_t room;
-    uint2 *masks = cut_room(c, &room);
-    CutPlan &plan = c->cut_plan;
-    plan_cuts(n_cams, group_begin, n_units, cut_mask_bytes(c), cut_word_bytes(c), room, &plan);
+    uint2 *masks = cut_room(c);
+    const CutPlan &plan = c->cut_plan;
     CK(cudaMemcpyAsync(c->cut_cams, hc.data(), sizeof(CutCam) * n_cams, cudaMemcpyHostToDevice,
                        st));
     CK(cudaMemcpyAsync(c->cut_chunks, plan.chunks.data(), sizeof(CutChunk) * plan.chunks.size(),
@@ -1351,7 +1351,7 @@ NGS_API ngs_status ngs_select_cut(ngs_ctx *c, const ngs_camera *cams, int32_t n_
     cudaStream_t st = (cudaStream_t)stream;
     Work &w = c->w;
     const int64_t cap32 = std::min<int64_t>(cap, (1ll << 32) - 1);
-    if (cut_masks_ok(c, n_cams, nullptr, n_cams)) {
+    if (cut_masks_ok(c, n_cams, nullptr, n_cams, false)) {
         std::vector<CutCam> hc(n_cams);
         for (int i = 0; i < n_cams; ++i) fill_cut_cam(hc[i], cams[i], 0.0f);
         if ((s = cut_by_masks(c, hc, nullptr, n_cams, false, d_ids, d_offsets, cap32, st)) != NGS_OK)
@@ -1400,9 +1400,10 @@ NGS_API ngs_status ngs_select_cut_shared(ngs_ctx *c, const ngs_camera *cams, int
     for (int i = 0; i < n_cams; ++i) fill_cut_cam(hc[i], cams[i], guard_px);
     Work &w = c->w;
     const int64_t cap32 = std::min<int64_t>(cap, (1ll << 32) - 1);
-    if (cut_masks_ok(c, n_cams, group_begin, n_groups)) {
-        s = cut_by_masks(c, hc, n_groups == n_cams ? nullptr : group_begin, n_groups,
-                         (flags & NGS_CUT_FRUSTUM) != 0, d_ids, d_offsets, cap32, st);
+    const int32_t *groups = n_groups == n_cams ? nullptr : group_begin;
+    const bool frustum = (flags & NGS_CUT_FRUSTUM) != 0;
+    if (cut_masks_ok(c, n_cams, groups, n_groups, frustum)) {
+        s = cut_by_masks(c, hc, groups, n_groups, frustum, d_ids, d_offsets, cap32, st);
         if (s != NGS_OK) return s;
         CK(cudaStreamSynchronize(st));
         return check_err(c);
@@ -1414,7 +1415,7 @@ NGS_API ngs_status ngs_select_cut_shared(ngs_ctx *c, const ngs_camera *cams, int
                        cudaMemcpyHostToDevice, st));
     CK(cudaMemsetAsync(w.counters, 0, N_COUNTERS * sizeof(uint32_t), st));
     k_bump_epoch<<<1, 1, 0, st>>>(w.epoch, kEpochStride);
-    launch_cut_shared((flags & NGS_CUT_FRUSTUM) != 0, c->scene.box_lo, c->scene.box_hi,
+    launch_cut_shared(frustum, c->scene.box_lo, c->scene.box_hi,
                       c->scene.n, c->cut_cams, c->cut_groups, n_groups, (uint32_t *)d_ids,
                       cap32, c->cut_off32, w.counters,
                       w.counters + TK_CUT, w.status, w.epoch, 0, w.err, c->grid_cut, st);

@@ -61,6 +61,39 @@ inline void plan_cuts(int n_cams, const int32_t *group_begin, int n_units, int64
     }
 }
 
+// Whether the plan's masks take less time than the single-pass kernels, by estimates in
+// us. blocks: of nodes; largest: cameras of the largest group; resident: CTAs of the
+// single-pass grid.
+//   The single-pass kernel goes in rounds of `resident` (unit, block) partitions; a
+// partition's time grows with its group, most under a frustum, where each member's five
+// planes are tested one after the other. The masks' two kernels are a chain of several
+// launches whose first CTAs take long (a CTA tests 2048 boxes for all cameras of a chunk),
+// but then the chunk's cameras cost little more than one; a pass of chunks takes another
+// launch of both.
+//   Measured, masks / single pass, us: 64 plain cuts of 2.6k nodes 68 / 48, 26k 81 / 68,
+// 79k 85 / 102, 1.31M 149 / 853; frustum-culled groups of 4 (64 cameras) 109 / 71, 142 / 83,
+// 148 / 94, 216 / 535, of 12 104 / 97, 129 / 122, 126 / 127, 196 / 485; one group of 4 cameras,
+// 1.31M nodes 77 / 68, with the frustum 97 / 96. On 945 such calls the choice is at most 8%
+// slower than the better of the two.
+inline bool cut_masks_pay(const CutPlan &p, int64_t blocks, int n_cams, int n_units, int largest,
+                          bool frustum, int64_t resident) {
+    // a last round of an eighth or less is hidden behind the others' ends
+    const int64_t parts = blocks * n_units - resident / 8;
+    const double rounds = (double)std::max<int64_t>(1, (parts + resident - 1) / resident);
+    const double mean = (double)n_cams / n_units;
+    const double cams = largest + (rounds - 1.0) * mean;   // one after the other
+    const double single = frustum ? 52.0 + 9.0 * rounds + 5.0 * cams
+                                  : 46.0 + 12.0 * rounds + 0.625 * cams;
+    const int k = p.lanes == 8 ? 0 : p.lanes == 16 ? 1 : 2;
+    constexpr double kPlain[3] = {70.0, 76.0, 86.0};
+    constexpr double kCulled[3] = {88.0, 100.0, 134.0}, kOfUnits[3] = {5.0, 20.0, 35.0};
+    double masks = frustum ? kCulled[k] + kOfUnits[k] / mean : kPlain[k];
+    int passes = 0;
+    for (const CutSlice &s : p.slices) passes += (s.n_chunks + s.n_masks - 1) / s.n_masks;
+    masks += 44.0 * (passes - 1);
+    return masks < single;
+}
+
 }  // namespace ngs
 
 #endif

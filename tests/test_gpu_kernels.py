@@ -168,6 +168,38 @@ def test_cuts_in_slices_equal_cuts_at_once(small_floor, floor_views, records):
         r.close()
 
 
+@pytest.fixture(scope="module")
+def larger_floor():
+    from scenegen import make_floor_scene, walk_cameras
+    scene = make_floor_scene(600_000, seed=12, size=(14.0, 10.0, 3.0), n_clusters=8, cluster_size=4000)
+    taus = np.random.default_rng(3).uniform(0.0, 40.0, 110)
+    return scene, walk_cameras(scene, 110, seed=8, width=320, height=240, taus=taus)
+
+
+# chunks of 8, 16 and 32 cameras, one and several; 2^13 records: slices in the cut's own buffer
+@pytest.mark.parametrize("records", [1 << 22, 1 << 13])
+def test_cuts_by_masks_of_a_larger_scene(larger_floor, records):
+    """A scene of enough nodes for masks at any number of cameras: the lists of the
+    single-pass kernels, which a group of 33 sends the whole call to."""
+    from paper_2603_15186_gb300 import Renderer
+    scene, cams = larger_floor
+    R = Renderer(cut_capacity=1 << 22, record_capacity=records, pair_capacity=1 << 20)
+    R.load_scene(scene)
+    for frustum, guard in ((True, 0.0), (True, 24.0), (False, 0.0)):
+        for sizes in ([1] * 4, [1] * 9, [1] * 16, [1] * 40, [3, 5], [3, 12, 1], [20, 30, 7], [32, 1, 31]):
+            n = int(sum(sizes))
+            gb = [0] + list(np.cumsum(sizes))
+            ids, off = R.select_cut_shared(cams[:n], gb, frustum, guard)
+            want, w_off = R.select_cut_shared(cams[:n + 33], gb + [n + 33], frustum, guard)
+            assert torch.equal(off, w_off[:len(off)]) and int(off[-1]) > 0
+            assert torch.equal(ids[:int(off[-1])], want[:int(off[-1])]), (frustum, guard, sizes)
+            if not frustum and len(sizes) == n:
+                plain, p_off = R.select_cut(cams[:n])
+                assert torch.equal(p_off, off) and torch.equal(plain[:int(off[-1])], ids[:int(off[-1])])
+            del ids, want
+    R.close()
+
+
 # one key into a second partition (4096 or 8192 keys), the keys that the histogram's
 # CTAs take at once (2048) and one more, several rounds of all its CTAs
 @pytest.mark.parametrize("key_bytes,n", [(4, 2048), (4, 2049), (4, 8193), (4, 311_297), (4, 6_000_001),

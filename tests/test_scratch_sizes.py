@@ -109,3 +109,45 @@ int main() {
 }
 """)
     assert calls > 500 and slices > calls and bad == 0
+
+
+# (blocks of 2048 nodes, group sizes, frustum, masks pay)
+CUT_ROUTES = [
+    # small scenes and few groups: the single-pass kernels, measured 1.1 to 2.2 times as fast
+    (2, [1] * 64, False, False), (13, [1] * 64, False, False), (39, [1] * 16, False, False),
+    (2, [4] * 16, True, False), (13, [2] * 32, True, False), (39, [4] * 16, True, False),
+    (39, [1] * 24, True, False), (97, [2] * 12, True, False), (97, [8] * 3, True, False),
+    (39, [4] * 8, False, False), (194, [8], False, False), (643, [4], False, False), (643, [12], False, False),
+    # large ones: the masks, 1.1 to 5 times as fast
+    (39, [1] * 128, False, True), (194, [1] * 6, False, True), (643, [1] * 4, False, True),
+    (643, [4] * 4, False, True), (2564, [4], False, True), (643, [1] * 4, True, True), (643, [8], True, True),
+    (13, [12], True, True), (39, [32], True, True), (39, [4] * 64, True, True), (194, [1] * 64, True, True),
+    (643, [4] * 16, True, True), (643, [12] * 5 + [4], True, True),
+    # the calls of test_cuts_by_masks_of_a_larger_scene
+    (381, [1] * 4, False, True), (381, [3, 5], False, True), (381, [32, 1, 31], False, True),
+    (381, [1] * 4, True, True), (381, [1] * 16, True, True), (381, [3, 5], True, True),
+    (381, [3, 12, 1], True, True), (381, [20, 30, 7], True, True)]
+
+
+def test_cuts_go_by_masks_where_they_pay(tmp_path):
+    calls = "".join("{%d, %d, {%s}},\n" % (b, f, ",".join(map(str, g))) for b, g, f, _ in CUT_ROUTES)
+    got = run_host(tmp_path, r"""
+#include <cstdio>
+#include "cut_plan.h"
+using namespace ngs;
+struct Call { int64_t blocks; int frustum; std::vector<int> groups; };
+int main() {
+  for (const Call &c : std::vector<Call>{""" + calls + r"""}) {
+    std::vector<int32_t> begin{0};
+    int largest = 0;
+    for (int g : c.groups) { begin.push_back(begin.back() + g); largest = std::max(largest, g); }
+    CutPlan p;
+    plan_cuts(begin.back(), begin.data(), (int)c.groups.size(), c.blocks * 16384, c.blocks * 256,
+              (int64_t)1 << 33, &p);
+    std::printf("%d\n", (int)cut_masks_pay(p, c.blocks, begin.back(), (int)c.groups.size(), largest,
+                                           c.frustum != 0, 608));
+  }
+  return 0;
+}
+""")
+    assert [bool(x) for x in got] == [pays for *_, pays in CUT_ROUTES]
