@@ -352,8 +352,9 @@ NGS_API ngs_status ngs_slice_occupancy(ngs_ctx *ctx, const ngs_slice_grid *grid,
  * free cells, 0xffffffff where unreachable (also everywhere when the goal is
  * blocked or outside the grid). Synchronous: returns once the fields are
  * complete. The context keeps a scratch buffer for it (two maps of the grid and,
- * for grids of more than about a million cells, two frontier queues of ny * nx
- * entries per goal), grown on demand. */
+ * for grids of more than about a million cells or more than some 75 to 230 goals
+ * (fewer the larger the grid), two frontier queues of ny * nx entries per goal),
+ * grown on demand. */
 NGS_API ngs_status ngs_nav_fields(ngs_ctx *ctx, const uint8_t *d_occ, int32_t nx, int32_t ny,
                                   int32_t nz, int32_t k_lo, int32_t k_hi, int32_t inflate,
                                   const int32_t *goals, int32_t n_goals, uint8_t *d_blocked,

@@ -134,7 +134,7 @@ struct ngs_ctx {
     cudaEvent_t ev_copied = nullptr;
 
     // navigation scratch (occupied-any map, goals, free-cell bits, and for
-    // maps beyond the search on bits frontier queues), grown on demand
+    // maps or goals beyond the search on bits frontier queues), grown on demand
     unsigned char *nav_tmp = nullptr;
     size_t nav_tmp_bytes = 0;
 
@@ -1767,8 +1767,8 @@ NGS_API ngs_status ngs_nav_fields(ngs_ctx *c, const uint8_t *d_occ, int32_t nx, 
     const size_t a_bytes = ((size_t)plane + 255) & ~(size_t)255;
     const size_t g_bytes = ((size_t)n_goals * sizeof(int2) + 255) & ~(size_t)255;
     const size_t f_bytes = ((size_t)nav_row_words(nx) * ny * sizeof(uint32_t) + 255) & ~(size_t)255;
-    const size_t need =
-        a_bytes + g_bytes + f_bytes + nav_queue_words(nx, ny, n_goals) * sizeof(uint32_t);
+    const size_t need = a_bytes + g_bytes + f_bytes +
+                        nav_queue_words(nx, ny, n_goals, c->num_sms) * sizeof(uint32_t);
     cudaStream_t st = (cudaStream_t)stream;
     if (need > c->nav_tmp_bytes) {
         CK(cudaStreamSynchronize(st));

@@ -6,7 +6,7 @@
 //    occupied at a cell within Chebyshev distance `inflate` of (i, j).
 //  - One distance field per goal: 4-connected breadth-first steps over free
 //    cells, UINT32_MAX where unreachable, level by level: on the map's bits, one
-//    cluster of CTAs per goal (k_nav_bfs), or, for maps too large for that, on a
+//    cluster of CTAs per goal (k_nav_bfs), or, for large maps and many goals, on a
 //    frontier queue, one CTA per goal (k_nav_bfs_queue: its threads expand the
 //    frontier's cells and admit each unreached free neighbour once, by an
 //    atomicCAS from UINT32_MAX to L + 1). Every cell enters a frontier at most
@@ -57,7 +57,8 @@ k_nav_dilate(const uint8_t *__restrict__ any, int nx, int ny, int r, int wpr,
     }
 }
 
-// Maps of more words than k_nav_bfs is built for (about a million cells).
+// Maps of more words than k_nav_bfs is built for (about a million cells), and many goals
+// (nav_words_per_thread).
 __global__ void __launch_bounds__(1024)
 k_nav_bfs_queue(const uint8_t *__restrict__ blocked, int nx, int ny, const int2 *__restrict__ goals,
           uint32_t *dist, uint32_t *queues) {
@@ -412,10 +413,21 @@ static int nav_grid(int64_t work, int num_sms) {
     return (int)std::max<int64_t>(1, std::min<int64_t>((work + 255) / 256, (int64_t)num_sms * 16));
 }
 
-// words per thread of k_nav_bfs, 0 for a map too large for it
-static int nav_words_per_thread(int ny, int wpr) {
+// Words per thread of k_nav_bfs, 0 where the queue searches: maps too large for the
+// bits, and more goals than the bits are faster for. A search on bits is the faster
+// one, but it holds eight CTAs that look at every word on every level, so that a few
+// dozen run at once; the queue's CTA looks at its frontier alone, and two run on each
+// SM. Bits / queue on open maps, us: 64 x 64 cells (1 word a thread) 128 goals 283 / 380,
+// 256 goals 484 / 388; 528 x 276 (1 word) 200 goals 2208 / 2401, 256 goals 2737 / 2418; 511 x 896
+// (2 words) 128 goals 4145 / 4727, 256 goals 8008 / 5692; 511 x 1920 (4 words) 64 goals 8023 /
+// 9280, 128 goals 13789 / 9510.
+static int nav_words_per_thread(int ny, int wpr, int n_goals, int num_sms) {
     const int64_t k = (nav_cta_words(ny, wpr) + kNavThreads - 1) / kNavThreads;
-    return k > 4 || nav_smem_bytes(ny, wpr) > kNavSmemMax ? 0 : k <= 2 ? (int)k : 4;
+    if (k > 4 || nav_smem_bytes(ny, wpr) > kNavSmemMax) return 0;
+    const int words = k <= 2 ? (int)k : 4;
+    const int most = words == 4 ? num_sms / 2 : words == 2 ? num_sms
+                     : ny * wpr < 512 ? num_sms * 5 / 4 : num_sms * 3 / 2;
+    return n_goals <= most ? words : 0;
 }
 
 template <int kWords>
@@ -427,8 +439,9 @@ static void launch_bfs(const uint32_t *free_bits, int nx, int ny, int wpr, const
         free_bits, nx, ny, wpr, goals, dist);
 }
 
-size_t nav_queue_words(int nx, int ny, int n_goals) {
-    return nav_words_per_thread(ny, nav_row_words(nx)) ? 0 : (size_t)n_goals * 2 * nx * ny;
+size_t nav_queue_words(int nx, int ny, int n_goals, int num_sms) {
+    return nav_words_per_thread(ny, nav_row_words(nx), n_goals, num_sms)
+               ? 0 : (size_t)n_goals * 2 * nx * ny;
 }
 
 // scratch: any [ny * nx] bytes, free_bits [ny * nav_row_words(nx)], queues
@@ -444,7 +457,7 @@ int launch_nav_fields(const uint8_t *occ, int nx, int ny, int k_lo, int k_hi, in
     k_nav_dilate<<<nav_grid(32 * words, num_sms), 256, 0, st>>>(any, nx, ny, inflate, wpr, blocked,
                                                                 free_bits);
     cudaMemsetAsync(dist, 0xff, (size_t)plane * n_goals * sizeof(uint32_t), st);   // kNavUnreached
-    switch (nav_words_per_thread(ny, wpr)) {
+    switch (nav_words_per_thread(ny, wpr, n_goals, num_sms)) {
     case 1: launch_bfs<1>(free_bits, nx, ny, wpr, d_goals, n_goals, dist, st); break;
     case 2: launch_bfs<2>(free_bits, nx, ny, wpr, d_goals, n_goals, dist, st); break;
     case 4: launch_bfs<4>(free_bits, nx, ny, wpr, d_goals, n_goals, dist, st); break;

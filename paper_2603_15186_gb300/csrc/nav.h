@@ -16,7 +16,7 @@ int launch_nav_fields(const uint8_t *occ, int nx, int ny, int k_lo, int k_hi, in
 // 32-bit words of a row of the free-cell map: at least one bit past the row's end
 inline int nav_row_words(int nx) { return nx / 32 + 1; }
 // words of the queues that launch_nav_fields takes for such a map (0: none)
-size_t nav_queue_words(int nx, int ny, int n_goals);
+size_t nav_queue_words(int nx, int ny, int n_goals, int num_sms);
 void launch_nav_paths(const uint32_t *dist, int nx, int ny, int n_goals, const int3 *starts,
                       int n, int max_len, int2 *paths, int32_t *lens, cudaStream_t st);
 

@@ -55,6 +55,21 @@ def test_nav_fields_and_paths_of_all_map_sizes(R, nx, ny):
             assert not paths[a, lens[a]:].any()
 
 
+# one, two and four words per thread: the most goals that search on bits and one more
+# (152 SMs), which the queue takes
+@pytest.mark.parametrize("nx,ny,n", [(64, 40, 190), (64, 40, 191), (300, 200, 228), (300, 200, 229),
+                                     (511, 385, 152), (511, 385, 153), (511, 900, 76), (511, 900, 77)])
+def test_nav_fields_of_many_goals(R, nx, ny, n):
+    """Every goal's field is the one that it has in a call of its own."""
+    rng = np.random.default_rng(n)
+    occ = torch.from_numpy((rng.random((2, ny, nx)) < 0.12).astype(np.uint8)).cuda()
+    goals = np.stack([rng.integers(-1, nx + 1, n), rng.integers(0, ny, n)], 1)
+    blocked, dist = R.nav_fields(occ, goals, 0, 1, 0)
+    for k in range(0, n, 10):
+        b1, d1 = R.nav_fields(occ, goals[k:k + 1], 0, 1, 0)
+        assert torch.equal(b1, blocked) and torch.equal(d1[0], dist[k]), k
+
+
 def test_nav_paths_of_other_fields(R):
     """A field that no breadth-first search gave is followed by the same rule: the
     first neighbour one less than the count so far, else stay and count on."""
