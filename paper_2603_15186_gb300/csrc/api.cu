@@ -1803,7 +1803,7 @@ NGS_API ngs_status ngs_nav_paths(ngs_ctx *c, const uint32_t *d_dist, int32_t nx,
     if ((int64_t)n * max_len >= ((int64_t)1 << 31)) return NGS_ERR_INVALID_ARG;
     cudaSetDevice(c->device);
     launch_nav_paths(d_dist, nx, ny, n_goals, reinterpret_cast<const int3 *>(d_starts), n, max_len,
-                     reinterpret_cast<int2 *>(d_paths), d_len, (cudaStream_t)stream);
+                     reinterpret_cast<int2 *>(d_paths), d_len, c->num_sms, (cudaStream_t)stream);
     CK(cudaGetLastError());
     return NGS_OK;
 }

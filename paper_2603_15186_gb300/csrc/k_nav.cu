@@ -13,7 +13,8 @@
 //    once, so the loop ends after at most one level per cell; the only waits are
 //    the barriers of a CTA and of its cluster.
 //  - A path descends a field from its start, taking the first neighbour in the
-//    order (+x, -x, +y, -y) whose distance is one less, one CTA per agent.
+//    order (+x, -x, +y, -y) whose distance is one less, one CTA per agent, or, of
+//    thousands of agents, one thread each.
 #include <cooperative_groups.h>
 
 #include "ngs_internal.cuh"
@@ -409,6 +410,37 @@ k_nav_paths(const uint32_t *__restrict__ dist, int nx, int ny, int n_goals,
     if (tid == 0) lens[a] = len;
 }
 
+// A thread per agent, reading the field in global memory: two memory round trips a
+// step, hidden by nothing but the other agents.
+__global__ void __launch_bounds__(128)
+k_nav_paths_each(const uint32_t *__restrict__ dist, int nx, int ny, int n_goals,
+                 const int3 *__restrict__ starts, int n, int max_len, int2 *__restrict__ paths,
+                 int32_t *__restrict__ lens) {
+    const int a = blockIdx.x * blockDim.x + threadIdx.x;
+    if (a >= n) return;
+    const int3 s = starts[a];
+    int len = 0;
+    if (s.z >= 0 && s.z < n_goals && s.x >= 0 && s.x < nx && s.y >= 0 && s.y < ny && max_len > 0) {
+        const uint32_t *dg = dist + (int64_t)s.z * nx * ny;
+        uint32_t d = dg[(int64_t)s.y * nx + s.x];
+        int i = s.x, j = s.y;
+        if (d != kNavUnreached) {
+            for (;;) {
+                paths[(int64_t)a * max_len + len] = make_int2(i, j);
+                ++len;
+                if (d == 0 || len >= max_len) break;
+                const int ni[4] = {i + 1, i - 1, i, i}, nj[4] = {j, j, j + 1, j - 1};
+                for (int e = 0; e < 4; ++e) {
+                    if (ni[e] < 0 || ni[e] >= nx || nj[e] < 0 || nj[e] >= ny) continue;
+                    if (dg[(int64_t)nj[e] * nx + ni[e]] == d - 1u) { i = ni[e]; j = nj[e]; break; }
+                }
+                --d;
+            }
+        }
+    }
+    lens[a] = len;
+}
+
 static int nav_grid(int64_t work, int num_sms) {
     return (int)std::max<int64_t>(1, std::min<int64_t>((work + 255) / 256, (int64_t)num_sms * 16));
 }
@@ -470,9 +502,19 @@ int launch_nav_fields(const uint8_t *occ, int nx, int ny, int k_lo, int k_hi, in
     return (int)e;
 }
 
+// Above this many agents a thread each: four CTAs run on an SM, and from the seventh
+// round of them on the windows take longer. CTAs / threads, us, on a 528 x 276 map: 64
+// paths of 286 cells on average 72 / 438, 4096 of 251 cells 284 / 437, 16384 981 / 466,
+// 131072 7453 / 605; of 53 cells 64 paths 22 / 65, 4096 72 / 70, 16384 232 / 71.
+static int nav_paths_few(int num_sms) { return 7 * 4 * num_sms; }
+
 void launch_nav_paths(const uint32_t *dist, int nx, int ny, int n_goals, const int3 *starts,
-                      int n, int max_len, int2 *paths, int32_t *lens, cudaStream_t st) {
-    if (n > 0)
+                      int n, int max_len, int2 *paths, int32_t *lens, int num_sms,
+                      cudaStream_t st) {
+    if (n > nav_paths_few(num_sms))
+        k_nav_paths_each<<<(n + 127) / 128, 128, 0, st>>>(dist, nx, ny, n_goals, starts, n, max_len,
+                                                          paths, lens);
+    else if (n > 0)
         k_nav_paths<<<n, kNavPathThreads, 0, st>>>(dist, nx, ny, n_goals, starts, n, max_len, paths, lens);
 }
 

@@ -18,7 +18,8 @@ inline int nav_row_words(int nx) { return nx / 32 + 1; }
 // words of the queues that launch_nav_fields takes for such a map (0: none)
 size_t nav_queue_words(int nx, int ny, int n_goals, int num_sms);
 void launch_nav_paths(const uint32_t *dist, int nx, int ny, int n_goals, const int3 *starts,
-                      int n, int max_len, int2 *paths, int32_t *lens, cudaStream_t st);
+                      int n, int max_len, int2 *paths, int32_t *lens, int num_sms,
+                      cudaStream_t st);
 
 }  // namespace ngs
 

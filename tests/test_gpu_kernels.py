@@ -95,6 +95,26 @@ def test_nav_paths_of_other_fields(R):
         assert lens[a] == len(cells) and np.array_equal(paths[a, :len(cells)], cells), a
 
 
+@pytest.mark.parametrize("n", [4256, 4257, 20_001])
+@pytest.mark.parametrize("plateaus", [False, True])
+def test_paths_of_many_agents(R, n, plateaus):
+    """Of 4256 agents (152 SMs) a CTA each, of more a thread: the paths that the agents
+    have in calls of a few hundred, on distance fields and on others, with starts outside
+    the map, on blocked cells and without such a goal among them."""
+    rng = np.random.default_rng(n)
+    ny, nx, max_len = 120, 170, 90
+    occ = torch.from_numpy((rng.random((1, ny, nx)) < 0.2).astype(np.uint8)).cuda()
+    dist = R.nav_fields(occ, [(5, 5), (100, 60), (169, 119)], 0, 0, 0)[1]
+    if plateaus:
+        dist = dist + torch.from_numpy(rng.integers(0, 2, (3, ny, nx)).astype(np.int32)).cuda()
+    starts = np.stack([rng.integers(-1, nx + 1, n), rng.integers(-1, ny + 1, n), rng.integers(-1, 4, n)], 1)
+    paths, lens = R.nav_paths(dist, starts, max_len)
+    assert int(lens.max()) == max_len and int(lens.min()) == 0
+    for k in range(0, n, n // 5):
+        p1, l1 = R.nav_paths(dist, starts[k:k + 300], max_len)
+        assert torch.equal(l1, lens[k:k + 300]) and torch.equal(p1, paths[k:k + 300]), k
+
+
 @pytest.mark.parametrize("cell,nx,ny,nz", [(0.05, 90, 85, 31), (0.004, 1000, 900, 3), (0.5, 9, 7, 2), (0.03, 1, 40, 40)])
 def test_slice_boxes_of_all_sizes(R, cell, nx, ny, nz):
     """Boxes from none or one cell to more than a warp takes at once (leaves of up to
