@@ -122,6 +122,7 @@ struct ngs_ctx {
     bool timing = false;
     std::vector<cudaEvent_t> ev;
     int ev_groups = 0;
+    bool far_depths = false;           // a graph's view of this scene reached kDepthNear
     int kernels_per_render = 0;
     uint32_t *h_counts = nullptr;      // page-locked: read_counts
 
@@ -906,6 +907,14 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
 ngs_status render_batched(ngs_ctx *c, int n_cams, cudaStream_t st) {
     Work &w = c->w;
     std::vector<SubBatch> sbs = plan(c, c->host_cams, kMaxCamsPerBatch);
+    // A graph holds one kind of depth sort for each sub-batch: in a scene where cameras come
+    // and go within reach of the far depths, all take the four passes from the first such
+    // view on. The results are the same; 320x240 views that came in turn took 191 us a call with
+    // a capture each time, 121 us so.
+    if (c->use_graph) {
+        for (const SubBatch &sb : sbs) c->far_depths = c->far_depths || !sb.near_depths;
+        for (SubBatch &sb : sbs) sb.near_depths = !c->far_depths;
+    }
     // graph key: layout of the cameras and every setting the launches bake in
     std::vector<int64_t> key;
     key.reserve(8 + 3 * n_cams);
@@ -914,7 +923,7 @@ ngs_status render_batched(ngs_ctx *c, int n_cams, cudaStream_t st) {
     key.push_back(cta_w_of(c)); key.push_back(cta_h_of(c));
     key.push_back(c->lod_blend ? 1 : 0);
     key.push_back(c->composite_order ? 1 : 0);
-    for (const SubBatch &sb : sbs) key.push_back(sb.near_depths ? 1 : 0);
+    key.push_back(c->far_depths ? 1 : 0);
     for (int i = 0; i < n_cams; ++i) {
         key.push_back(c->host_cams[i].width);
         key.push_back(c->host_cams[i].height);
@@ -1329,6 +1338,7 @@ NGS_API ngs_status ngs_load_scene(ngs_ctx *c, const ngs_gaussians *g, const ngs_
     for (int64_t i = 0; i < n; ++i) d.n_leaves += h->child_count[i] == 0 ? 1 : 0;
     d.attr_dtype = g->attr_dtype;
     c->loaded = true;
+    c->far_depths = false;
     ++c->scene_version;
     return NGS_OK;
 }

@@ -353,6 +353,37 @@ def test_depths_beyond_the_short_keys(mode):
     r.close()
 
 
+def test_views_that_reach_far_depths_and_others_share_a_graph():
+    """Views along the axis of a Gaussian 30 km away (four passes over the depth) and across
+    it (three would do), in turn: one capture each way at most, the pixels of the plain path."""
+    from paper_2603_15186_gb300 import Renderer
+    from scenegen import look_camera, make_uniform_box_scene
+    from scenegen.scene import build_hierarchy
+    near = make_uniform_box_scene(600, seed=12)
+    leaf = near.child_count == 0
+    scene = build_hierarchy(np.concatenate([near.pos[leaf], np.float32([[30_000, 2, 1.2]])]),
+                            np.concatenate([near.quat[leaf], np.float32([[1, 0, 0, 0]])]),
+                            np.concatenate([near.log_scale[leaf], np.full((1, 3), np.log(400.0), np.float32)]),
+                            np.concatenate([near.opacity[leaf], np.full(1, 0.8, np.float32)]),
+                            np.concatenate([near.sh[leaf], np.zeros((1, 16, 3), np.float32)]))
+    r = Renderer(cut_capacity=1 << 20, record_capacity=1 << 20, pair_capacity=1 << 22)
+    r.load_scene(scene)
+    cams = [look_camera((2.0, 2.0, 1.2), a, 160, 120, tau=0.0) for a in (np.pi / 2, 0.0)]
+    r.set_mode("plain")
+    want = [r.render([c])[0].clone() for c in cams]
+    r.set_mode("batched")
+    replayed = []
+    for k in (0, 0, 1, 0, 1, 0):
+        assert torch.equal(r.render([cams[k]])[0], want[k])
+        replayed.append(r.stats()["graph_replayed"])
+    assert replayed == [0, 1, 0, 1, 1, 1]
+    r.load_scene(near)
+    r.render([cams[1]])
+    r.render([cams[1]])
+    assert r.stats()["graph_replayed"] == 1
+    r.close()
+
+
 # pairs: less than a partition of the last tile pass; partitions with one value of the
 # tiles' low digit and with several; three passes over 76800 tiles
 @pytest.mark.parametrize("leaves,grow,width,height", [(40, 0.0, 640, 480), (3000, 1.0, 640, 480),
