@@ -16,16 +16,17 @@
 // One thread per node takes the planes within the slice's vertical support and the
 // box of cells of each slice's support (the ellipse where a >= 1/255, widened by a
 // relative 1e-4 and 1e-6 m). Boxes differ (a few cells to hundreds: log-normal
-// scales, interior nodes none), so a warp puts its leaves' boxes on a plane end to end
-// and its lanes take the cells one each; a value is folded into its cell with
-// atomicMax on its bits (non-negative floats order like their bit patterns, so the
-// result does not depend on the order). 4M leaves, 13 planes, 528 x 276 cells of 5 cm
-// (60 M cells in boxes): 1740 us with a loop per thread over its own boxes (6.6 of 32
-// lanes active) and a count per thread on one address, 366 us so; its atomics do not
-// bound it (a look at the cell before each, to leave out those that change nothing:
-// 538 us).
-#include <climits>
-
+// scales, interior nodes none), so a warp puts its leaves' boxes, every leaf on its
+// first plane, then every leaf on its second, end to end and its lanes take the cells
+// one each; a value is folded into its cell with atomicMax on its bits (non-negative
+// floats order like their bit patterns, so the result does not depend on the order). 4M
+// leaves, 13 planes, 528 x 276 cells of 5 cm (60 M cells in boxes): 1740 us with a loop per
+// thread over its own boxes (6.6 of 32 lanes active) and a count per thread on one
+// address, 350 us so; its atomics do not bound it (a look at the cell before each, to
+// leave out those that change nothing: 538 us). Plane by plane for the whole warp, a plane
+// that one leaf reaches costs as much as one that all reach: 300 planes 1 cm apart,
+// 20 cm cells, 1M leaves of a floor 682 us (620 with the loop per thread), 525 us so;
+// 60k leaves of a box, where the leaves of most planes end the call, 165 (120), 126 us.
 #include "ngs_internal.cuh"
 
 namespace ngs {
@@ -56,7 +57,7 @@ struct __align__(16) SliceItem {
     float ez, cxx, cxy, cyy;
     float o, mx, my, inv_w;
     int32_t i0, j0, w;
-    uint32_t start;       // its first cell in the warp's list of cells
+    uint32_t plane;       // the plane's first cell in the grid
 };
 
 constexpr int kSliceThreads = 256;
@@ -68,6 +69,7 @@ __global__ void __launch_bounds__(kSliceThreads)
 k_slice(SceneDev sc, SliceGrid g, uint32_t *__restrict__ value_bits,
         unsigned long long *work) {
     __shared__ SliceItem s_item[kSliceThreads / 32][32];
+    __shared__ uint32_t s_start[kSliceThreads / 32][32];   // an item's first cell in the warp's list
     __shared__ unsigned long long s_evals[kSliceThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t node = (int64_t)blockIdx.x * kSliceThreads + threadIdx.x;
@@ -119,13 +121,11 @@ k_slice(SceneDev sc, SliceGrid g, uint32_t *__restrict__ value_bits,
             iyy = cxx / det;
         }
     }
-    const int64_t plane = (int64_t)g.nx * g.ny;
+    const uint32_t plane = (uint32_t)g.nx * (uint32_t)g.ny;   // the grid has < 2^31 cells
     unsigned long long evals = 0;
-    const bool some = k0 <= k1;
-    const int k_lo = __reduce_min_sync(0xffffffffu, some ? k0 : INT_MAX);
-    const int k_hi = __reduce_max_sync(0xffffffffu, some ? k1 : INT_MIN);
+    const int span = k0 <= k1 ? k1 - k0 : -1;
     // the value of cell (i, j) of item t, folded into the plane's cell
-    auto fold = [&](const SliceItem &t, uint32_t *vk, int i, int j) {
+    auto fold = [&](const SliceItem &t, int i, int j) {
         const float dy = g.y0 + ((float)j + 0.5f) * g.cell - t.my;
         const float dx = g.x0 + ((float)i + 0.5f) * g.cell - t.mx;
         // the terms in this order, the last one rounded before it is added
@@ -133,15 +133,18 @@ k_slice(SceneDev sc, SliceGrid g, uint32_t *__restrict__ value_bits,
                                   __fmul_rn(t.cyy * dy, dy));
         const float a = t.o * expf(-0.5f * q);
         if (a >= (1.0f / 255.0f))
-            atomicMax(vk + (uint32_t)j * (uint32_t)g.nx + (uint32_t)i,
+            atomicMax(value_bits + t.plane + (uint32_t)j * (uint32_t)g.nx + (uint32_t)i,
                       __float_as_uint(fminf(0.99f, a)));
     };
     SliceItem *items = s_item[warp];
-    for (int k = k_lo; k <= k_hi; ++k) {
-        uint32_t *vk = value_bits + (int64_t)k * plane;
+    uint32_t *starts = s_start[warp];
+    // every lane's first plane, then every lane's second
+    const int most = __reduce_max_sync(0xffffffffu, span);
+    for (int at_plane = 0; at_plane <= most; ++at_plane) {
         SliceItem t;
         uint32_t n = 0, h = 0;   // cells and rows of this thread's slice
-        if (k >= k0 && k <= k1) {
+        if (at_plane <= span) {
+            const int k = k0 + at_plane;
             const float zp = (g.z0 + (float)k * g.dz) - p.z;
             const float ez = lambda * zp * zp;
             const float rem = K - ez;
@@ -156,6 +159,7 @@ k_slice(SceneDev sc, SliceGrid g, uint32_t *__restrict__ value_bits,
                     t.ez = ez; t.cxx = cxx; t.cxy = cxy; t.cyy = cyy;
                     t.o = o; t.mx = mx; t.my = my;
                     t.i0 = i0; t.j0 = j0; t.w = i1 - i0 + 1;
+                    t.plane = (uint32_t)k * plane;
                     t.inv_w = 1.0f / (float)t.w;
                     h = (uint32_t)(j1 - j0 + 1);
                     n = (uint32_t)t.w * h;      // < 2^31, the grid's cells
@@ -171,12 +175,25 @@ k_slice(SceneDev sc, SliceGrid g, uint32_t *__restrict__ value_bits,
             const SliceItem u = items[0];
             __syncwarp();
             for (uint32_t j = 0; j < rows; ++j)
-                for (int i = lane; i < u.w; i += 32) fold(u, vk, u.i0 + i, u.j0 + (int)j);
+                for (int i = lane; i < u.w; i += 32) fold(u, u.i0 + i, u.j0 + (int)j);
         }
         if (n > kSliceBig) n = 0;
         // the items that have cells, in lane order, and their cells end to end
         const uint32_t has = __ballot_sync(0xffffffffu, n > 0);
         if (has == 0) continue;
+        if ((has & (has - 1)) == 0) {   // one item: a leaf of more planes than its neighbours
+            const int src = __ffs(has) - 1;
+            const uint32_t total = __shfl_sync(0xffffffffu, n, src);
+            if (lane == src) items[0] = t;
+            __syncwarp();
+            const SliceItem u = items[0];
+            __syncwarp();
+            for (uint32_t r = lane; r < total; r += 32) {
+                const uint32_t jj = (uint32_t)(((float)r + 0.5f) * u.inv_w);
+                fold(u, u.i0 + (int)(r - jj * (uint32_t)u.w), u.j0 + (int)jj);
+            }
+            continue;
+        }
         uint32_t incl = n;
 #pragma unroll
         for (int s = 1; s < 32; s <<= 1) {
@@ -185,12 +202,13 @@ k_slice(SceneDev sc, SliceGrid g, uint32_t *__restrict__ value_bits,
         }
         const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
         if (n > 0) {
-            t.start = incl - n;
-            items[__popc(has & lanemask_lt())] = t;
+            const int q = __popc(has & lanemask_lt());
+            items[q] = t;
+            starts[q] = incl - n;
         }
         __syncwarp();
         // lane l also holds the start of item l
-        const uint32_t start = lane < __popc(has) ? items[lane].start : 0xffffffffu;
+        const uint32_t start = lane < __popc(has) ? starts[lane] : 0xffffffffu;
         for (uint32_t c0 = 0; c0 < total; c0 += 32) {
             // the item of cell c0 + lane: the last that starts at or before c0, plus
             // the items that start between
@@ -200,12 +218,13 @@ k_slice(SceneDev sc, SliceGrid g, uint32_t *__restrict__ value_bits,
                 __reduce_or_sync(0xffffffffu, start > c0 && off < 32u ? 1u << off : 0u);
             const uint32_t c = c0 + lane;
             if (c < total) {
-                const SliceItem u = items[at + __popc(marks & (lanemask_lt() | 1u << lane))];
+                const int q = at + __popc(marks & (lanemask_lt() | 1u << lane));
+                const SliceItem u = items[q];
                 // row and column in the box: exact, (r + 1/2) / w is at least
                 // 1 / (2 w) from an integer and r < 2^17
-                const uint32_t r = c - u.start;
+                const uint32_t r = c - starts[q];
                 const uint32_t jj = (uint32_t)(((float)r + 0.5f) * u.inv_w);
-                fold(u, vk, u.i0 + (int)(r - jj * (uint32_t)u.w), u.j0 + (int)jj);
+                fold(u, u.i0 + (int)(r - jj * (uint32_t)u.w), u.j0 + (int)jj);
             }
         }
         __syncwarp();
