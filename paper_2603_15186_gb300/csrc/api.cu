@@ -670,7 +670,7 @@ void enqueue_batched(ngs_ctx *c, const SubBatch &sb, int sb_index, cudaStream_t 
     launch_pair_offsets(w.rect, w.didx[dsel], w.counters + CNT_VIS, w.poff, w.counters,
                         w.pair_cap, w.counters + TK_SCAN, w.status, w.epoch, eo++, w.err,
                         w.chunk_first, w.rect_sorted, cams, thist, sb.tile_passes,
-                        grid_for(scan_status_words(recs), c->grid_scan), st);
+                        grid_for(offset_status_words(recs), c->grid_scan), st);
     mark(c, sb_index, MK_POFF, st);
     launch_duplicate(w.rect_sorted, w.didx[dsel], w.poff, w.chunk_first, w.counters + CNT_VIS,
                      w.counters + CNT_PAIRS, w.pair_cap, cams, w.pkey[0], w.pval[0], w.err,
@@ -839,7 +839,7 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
         eo += 4;
         const int dsel = sb.near_depths ? 1 : 0;   // three or four passes
         if (sb.near_depths) mark(c, ci, MK_DPASS0 + 3, st);
-        const int gscan = (int)std::max<int64_t>(1, scan_parts(n_vis));
+        const int gscan = (int)std::max<int64_t>(1, offset_parts(n_vis));
         uint32_t *thist = w.hist + kTileHist;
         launch_pair_offsets(w.rect, w.didx[dsel], w.counters + CNT_VIS, w.poff, w.counters,
                             w.pair_cap, w.counters + TK_SCAN, w.status, w.epoch, eo++, w.err,

@@ -288,7 +288,7 @@ k_scan(const uint32_t *__restrict__ in, const uint2 *__restrict__ rect,
     const int64_t n = n_dev ? (int64_t)*n_dev : n_host;
     const uint32_t epoch = *epoch_ptr + epoch_off;
     if (n == 0 && blockIdx.x == 0 && tid == 0 && total_out) *total_out = 0;
-    if (n <= kScanFew)
+    if (kGather && n <= kScanFew)
         scan_partitions<kGather, kScanItemsFew>(S, in, rect, idx, out, n, total_out, total_cap,
                                                 ticket, status, epoch, err, chunk_first,
                                                 chunk_cap, rect_out, cams, hist, passes);

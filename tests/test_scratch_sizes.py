@@ -16,8 +16,8 @@ def run_host(tmp_path, source):
 def test_status_words_hold_every_accepted_scan_and_sort(tmp_path):
     """Over capacities from one element to the default and scenes from one node block up:
     the status words that a standalone scan or sort within the limit uses, a render's
-    and a cut's, are all in the buffer. What the limit accepts is what it accepted when
-    every scan had partitions of 2048 elements."""
+    and a cut's, are all in the buffer, whatever the partitions that the header's constants
+    give them. What the limit accepts is one partition of 2048 elements a word."""
     n, refused, accepted, short = run_host(tmp_path, r"""
 #include <cstdio>
 #include <vector>
@@ -38,7 +38,7 @@ int main() {
       if (scan_accepted(m, b.limit) != ((m + 2047) / 2048 <= old)) return 1;
       if (!scan_accepted(m, b.limit)) { ++refused; continue; }
       ++accepted;
-      need((m + (m <= 1 << 20 ? 255 : 2047)) / (m <= 1 << 20 ? 256 : 2048));
+      need(scan_parts(m));
     }
     // sorts: 4096 keys a partition (64 bits), 256 words each
     const int64_t most = b.limit / 256 * 4096;
@@ -50,7 +50,7 @@ int main() {
     need((rec + 8191) / 8192 * 512);
     need((pairs + 8191) / 8192 * 256);
     need(blocks * 1024);
-    need((std::min<int64_t>(blocks * 1024, 1 << 20) + 255) / 256);
+    need(scan_parts(blocks * 1024));
   }
   std::printf("%ld %ld %ld %ld\n", n, refused, accepted, lacking);
   return 0;
