@@ -540,7 +540,8 @@ ngs_status cut_by_masks(ngs_ctx *c, const std::vector<CutCam> &hc, const int32_t
         for (int j = 0; j < sl.n_chunks; j += sl.n_masks)
             launch_cut_masks(frustum, group_begin != nullptr, plan.lanes, sc.box_lo, sc.box_hi, sc.n,
                              c->cut_cams, c->cut_groups + sl.unit0, c->cut_chunks + sl.chunk0 + j,
-                             std::min(sl.n_masks, sl.n_chunks - j), masks, words, c->cut_counts, w.err, st);
+                             std::min(sl.n_masks, sl.n_chunks - j), masks, words, c->cut_counts,
+                             w.err, st);
         const int64_t np = nblk * sl.n_units, sparts = scan_parts(np);
         launch_scan_u32(c->cut_counts, c->cut_poff, nullptr, np, c->cut_off32,
                         w.counters + TK_SCAN, w.status, w.epoch, 0, w.err,
@@ -719,13 +720,12 @@ void enqueue_batched(ngs_ctx *c, const SubBatch &sb, int sb_index, cudaStream_t 
     if (kept && !c->composite_order) k_copy_stats<<<1, 32, 0, st>>>(w.counters, kept);
 }
 
-int kernels_of(const SubBatch &sb, bool batched, bool order) {
+int kernels_of(const SubBatch &sb, bool batched) {
     // start, live partitions, fused cut + preprocess, partition scan and key
     // gather (which also counts the depth histograms); depth sort (3 or 4 passes);
     // pair offsets, duplication; tile sort (the last pass writing the tile
     // ranges) or, with a single tile, the ranges kernel; compositing; and in the
     // batched path the tile order, or else the stats copy
-    (void)order;
     return 5 + (sb.near_depths ? 3 : 4) + 2 + std::max(sb.tile_passes, 1) + 1 + (batched ? 1 : 0);
 }
 
@@ -889,7 +889,7 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
                          w.work64, nullptr, nullptr, on);
         mark(c, ci, MK_COMPOSITE, st);
         CK(cudaGetLastError());
-        c->kernels_per_render += kernels_of(sb, false, false);
+        c->kernels_per_render += kernels_of(sb, false);
         cut_tot += n_cut; vis_tot += n_vis; pair_tot += n_pairs;
         c->last_plan.push_back(sb);
         c->last_plan.back().c0 = ci;
@@ -935,7 +935,7 @@ ngs_status render_batched(ngs_ctx *c, int n_cams, cudaStream_t st) {
     if ((es = ensure_sb_events(c, (int)sbs.size())) != NGS_OK) return es;
     key.push_back(c->timing ? 1 : 0);
     c->kernels_per_render = 0;
-    for (const SubBatch &sb : sbs) c->kernels_per_render += kernels_of(sb, true, c->composite_order);
+    for (const SubBatch &sb : sbs) c->kernels_per_render += kernels_of(sb, true);
     CK(cudaMemcpyAsync(w.cams, c->host_cams.data(), sizeof(DevCamera) * n_cams,
                        cudaMemcpyHostToDevice, st));
     if (c->use_graph) {
@@ -1858,7 +1858,7 @@ NGS_API ngs_status ngs_sort_pairs(ngs_ctx *c, void *d_keys, uint32_t *d_vals, in
     a.vals[0] = d_vals; a.vals[1] = c->sort_tmp_vals;
     a.n_dev = nullptr; a.n_host = n; a.n_max = n;
     a.key_bytes = key_bytes; a.begin_bit = begin_bit; a.end_bit = end_bit;
-    a.digit_bits = 8;
+    a.digit_bits = 8; a.num_sms = c->num_sms;
     a.hist = c->w.hist; a.tickets = c->w.counters + TK_SORT0; a.status = c->w.status;
     a.epoch = c->w.epoch; a.epoch_off = 0; a.err = c->w.err;
     const int grid = (int)std::min<int64_t>(parts, key_bytes == 8 ? c->grid_sort64 : c->grid_sort32);

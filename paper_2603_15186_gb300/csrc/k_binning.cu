@@ -110,9 +110,11 @@ __device__ __forceinline__ void tile_digits_add(TileDigits &H, uint32_t k0, uint
     }
 }
 
-// A chain of at most this many partitions (they all run at once) is looked back over
-// by a warp, 32 partitions per round trip; on longer chains, where a look-back ends
-// after a window or two, one thread took 8% less time than a warp.
+// A chain of at most this many partitions is looked back over by a warp, 32 partitions
+// per round trip: five CTAs run on an SM (760 of 152), and the partitions that start
+// together look back over one another. On longer chains most look-backs end after a
+// window or two, and one thread took 8% less time than a warp. Either way partitions
+// come from a ticket, so what a look-back waits for is running or done.
 constexpr int kScanShortChain = 4096;
 // Rects of up to this many tile rows are counted by their own thread; a warp that has
 // a larger one deals all its rows to its lanes. 260k records of a 720p view on

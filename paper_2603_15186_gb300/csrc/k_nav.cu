@@ -515,7 +515,8 @@ void launch_nav_paths(const uint32_t *dist, int nx, int ny, int n_goals, const i
         k_nav_paths_each<<<(n + 127) / 128, 128, 0, st>>>(dist, nx, ny, n_goals, starts, n, max_len,
                                                           paths, lens);
     else if (n > 0)
-        k_nav_paths<<<n, kNavPathThreads, 0, st>>>(dist, nx, ny, n_goals, starts, n, max_len, paths, lens);
+        k_nav_paths<<<n, kNavPathThreads, 0, st>>>(dist, nx, ny, n_goals, starts, n, max_len, paths,
+                                                   lens);
 }
 
 }  // namespace ngs

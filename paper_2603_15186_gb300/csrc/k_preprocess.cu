@@ -40,6 +40,8 @@ constexpr int kPreThreads = 256;
 // 945, 5721 + 889, 5914 + 914 us on 256 mixed views of a 4M-leaf floor; 87 + 22, 56 + 14,
 // 52 + 12 us on eight 333x187 views of a 1M-leaf floor; 44 + 21, 40 + 14, 40 + 11 us on one
 // 720p view of the former, whose partition scan takes 6, 10, 19 us.
+// Each context, and each lane of a server, keeps 24 bytes of tables for every partition of
+// 1024 cameras: 252 MB for 5.25 M nodes with 2 (126 MB with 4).
 constexpr int kPreItems = 2;
 constexpr int kPrePart = kPreThreads * kPreItems;     // nodes per partition
 
@@ -997,9 +999,10 @@ k_part_scan(const uint32_t *__restrict__ vis_count, int n_cams, int64_t nblk,
 // of its visible Gaussians (skipping holes) and writes their record indices at
 // the partition's dense position. On the
 // way it counts the digit histograms of the depth sort's passes (four of 8 bits, or, with
-// kNear, three of 9 bits on keys less their base) into hist[passes][digits] (zeroed beforehand; the last CTA scans them): positive float depths share
-// their high digits, so a warp whose keys agree on a digit adds its count once
-// instead of contending on one shared-memory counter.
+// kNear, three of 9 bits on keys less their base) into hist[passes][digits] (zeroed
+// beforehand; the last CTA scans them): positive float depths share their high digits,
+// so a warp whose keys agree on a digit adds its count once instead of contending on one
+// shared-memory counter.
 template <bool kNear>
 __global__ void __launch_bounds__(256)
 k_part_gather(const uint32_t *__restrict__ part_list, int n_cams, int64_t nblk,

@@ -314,7 +314,7 @@ static void launch_sort_t(const SortArgs &a, int grid, const LaunchOn &st) {
     if (!a.hist_ready) {
         cudaMemsetAsync(a.hist, 0, sizeof(uint32_t) * kRadix * passes, st.st);
         const int ugrid = (int)std::max<int64_t>(
-            1, std::min<int64_t>((a.n_max + kSortThreads * kUp - 1) / (kSortThreads * kUp), 8 * 152));
+            1, std::min<int64_t>(parts_of(a.n_max, kSortThreads * kUp), 8 * a.num_sms));
         k_upsweep<K><<<ugrid, kSortThreads, 0, st.st>>>((const K *)a.keys[0], a.n_dev, a.n_host,
                                                      a.begin_bit, a.end_bit, a.hist,
                                                      a.tickets + kMaxPasses, a.err);

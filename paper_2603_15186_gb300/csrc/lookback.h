@@ -30,7 +30,9 @@ inline int64_t parts_of(int64_t n, int64_t part) { return (n + part - 1) / part;
 
 // partitions, and status words, of a scan of n elements, and of n records' pair offsets
 inline int64_t scan_parts(int64_t n) { return parts_of(n, kScanPart); }
-inline int64_t offset_parts(int64_t n) { return n <= kScanFew ? parts_of(n, kScanPartFew) : scan_parts(n); }
+inline int64_t offset_parts(int64_t n) {
+    return n <= kScanFew ? parts_of(n, kScanPartFew) : scan_parts(n);
+}
 // the most that the pair offsets of up to n records have
 inline int64_t offset_status_words(int64_t n) {
     return std::max(offset_parts(n), offset_parts(std::min(n, kScanFew)));

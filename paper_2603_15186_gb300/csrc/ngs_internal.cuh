@@ -334,8 +334,8 @@ __device__ __forceinline__ void digit_scan_by_last(uint32_t *hist, int passes, u
 }
 
 // look_back by a whole warp (all lanes call it with the same arguments and get the
-// same result), 32 predecessors per round trip: for a short chain whose partitions
-// all run at once, where a look-back walks most of the chain.
+// same result), 32 predecessors per round trip: for a short chain, where a look-back
+// walks over most of the partitions that started with its own.
 __device__ __forceinline__ bool look_back_warp(const uint64_t *status, int64_t part,
                                                uint32_t epoch, uint32_t *excl, int *err) {
     const int lane = threadIdx.x & 31;
@@ -523,6 +523,7 @@ struct SortArgs {
     int key_bytes;
     int begin_bit, end_bit;
     int digit_bits;           // 8, or 9 (32-bit keys with hist_ready, no ranges)
+    int num_sms;              // without hist_ready: the upsweep's grid
     bool hist_ready;          // hist already holds the digit counts' exclusive prefixes
     uint32_t *hist;           // [passes][256 or 512]
     // last pass: skip_last_keys writes the values only (the sorted keys are

@@ -141,7 +141,7 @@ extern "C" NGS_API ngs_status ngs_sort_pairs_static(void *d_keys, uint32_t *d_va
     a.vals[0] = d_vals; a.vals[1] = (uint32_t *)(base + kOffVals);
     a.n_dev = nullptr; a.n_host = n; a.n_max = n;
     a.key_bytes = key_bytes; a.begin_bit = begin_bit; a.end_bit = end_bit;
-    a.digit_bits = 8;
+    a.digit_bits = 8; a.num_sms = sms;
     a.hist = (uint32_t *)(base + kOffHist);   // cleared by the launcher
     a.tickets = tickets; a.status = status;
     a.epoch = epoch; a.epoch_off = 0; a.err = err;
