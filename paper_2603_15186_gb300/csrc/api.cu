@@ -315,6 +315,14 @@ void sort_hook(void *user, int step) {
     mark(h->c, h->group, h->first_mark + step, h->st);
 }
 
+// Most cameras of a sub-batch. They share the record slots, and each may see its whole
+// cut: an antichain of the tree, at most as many nodes as the tree has leaves.
+int most_cams(const ngs_ctx *c) {
+    const int64_t per_cam = c->scene.n_leaves > 0 ? c->scene.n_leaves : c->scene.n;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(
+        c->cfg.record_capacity / std::max<int64_t>(per_cam, 1), kMaxCamsPerBatch));
+}
+
 ngs_status ensure_work(ngs_ctx *c) {
     if (c->work_ready) return NGS_OK;
     Work &w = c->w;
@@ -336,8 +344,7 @@ ngs_status ensure_work(ngs_ctx *c) {
     A(dalloc(&w.cut_ids, (size_t)w.cut_cap));
     A(dalloc(&w.cut_off, kMaxCamsPerBatch + 1));
     A(dalloc(&w.vis_count, kMaxCamsPerBatch));
-    w.part_cap = std::max<int64_t>(1, (c->scene.n + cutpre_partition_nodes() - 1) /
-                                          cutpre_partition_nodes() * kMaxCamsPerBatch);
+    w.part_cap = std::max<int64_t>(1, parts_of(c->scene.n, cutpre_partition_nodes()) * most_cams(c));
     A(dalloc(&w.part_list, (size_t)w.part_cap));
     A(dalloc(&w.group_list, (size_t)w.part_cap));
     A(dalloc(&w.part_info, (size_t)w.part_cap));
@@ -577,18 +584,13 @@ void set_depth_bits(SortArgs &a, bool near) {
     a.digit_bits = near ? 9 : 8;
 }
 
-// Splits cameras into sub-batches: at most kMaxCamsPerBatch cameras, at most
-// max_tiles tiles (one camera alone may exceed it), cut and record bounds
-// (a camera's cut is an antichain of the tree, so it holds at most as many
-// nodes as the tree has leaves) and an estimate of the pairs.
-std::vector<SubBatch> plan(ngs_ctx *c, std::vector<DevCamera> &cams, int max_cams_per_batch) {
+// Splits cameras into sub-batches: at most most_cams cameras (the record slots and the
+// partition tables are sized for them), at most max_tiles tiles (one camera alone may
+// exceed it) and an estimate of the pairs.
+std::vector<SubBatch> plan(ngs_ctx *c, std::vector<DevCamera> &cams) {
     std::vector<SubBatch> out;
-    const int64_t per_cam = c->scene.n_leaves > 0 ? c->scene.n_leaves : c->scene.n;
     const int64_t max_tiles = c->cfg.max_tiles_per_batch;
-    // the visible Gaussians of a sub-batch (at most per_cam per camera) share
-    // the record slots
-    const int64_t cams_by_cut =
-        std::max<int64_t>(1, c->w.rec_cap / std::max<int64_t>(per_cam, 1));
+    const int max_cams = most_cams(c);
     int i = 0;
     const int N = (int)cams.size();
     while (i < N) {
@@ -600,8 +602,8 @@ std::vector<SubBatch> plan(ngs_ctx *c, std::vector<DevCamera> &cams, int max_cam
             const int64_t t = (int64_t)d.tiles_x * d.tiles_y;
             const double p = c->pairs_per_pixel * (double)d.width * d.height;
             const int cnt = sb.c1 - sb.c0;
-            if (cnt > 0 && (tiles + t > max_tiles || cnt + 1 > max_cams_per_batch ||
-                            cnt + 1 > cams_by_cut || pairs + p > (double)c->w.pair_cap))
+            if (cnt > 0 && (tiles + t > max_tiles || cnt + 1 > max_cams ||
+                            pairs + p > (double)c->w.pair_cap))
                 break;
             cams[sb.c1].tile_base = (uint32_t)tiles;
             sb.near_depths = sb.near_depths && near_depths(c, d);
@@ -906,7 +908,7 @@ ngs_status render_plain(ngs_ctx *c, int n_cams, cudaStream_t st) {
 
 ngs_status render_batched(ngs_ctx *c, int n_cams, cudaStream_t st) {
     Work &w = c->w;
-    std::vector<SubBatch> sbs = plan(c, c->host_cams, kMaxCamsPerBatch);
+    std::vector<SubBatch> sbs = plan(c, c->host_cams);
     // A graph holds one kind of depth sort for each sub-batch: in a scene where cameras come
     // and go within reach of the far depths, all take the four passes from the first such
     // view on. The results are the same; 320x240 views that came in turn took 191 us a call with

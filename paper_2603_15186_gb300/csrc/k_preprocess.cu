@@ -40,8 +40,8 @@ constexpr int kPreThreads = 256;
 // 945, 5721 + 889, 5914 + 914 us on 256 mixed views of a 4M-leaf floor; 87 + 22, 56 + 14,
 // 52 + 12 us on eight 333x187 views of a 1M-leaf floor; 44 + 21, 40 + 14, 40 + 11 us on one
 // 720p view of the former, whose partition scan takes 6, 10, 19 us.
-// Each context, and each lane of a server, keeps 24 bytes of tables for every partition of
-// 1024 cameras: 252 MB for 5.25 M nodes with 2 (126 MB with 4).
+// A context (each lane of a server) keeps 24 bytes of tables for every partition and camera
+// of a sub-batch: 3.9 MB for 5.25 M nodes and 2^26 records (16 cameras).
 constexpr int kPreItems = 2;
 constexpr int kPrePart = kPreThreads * kPreItems;     // nodes per partition
 

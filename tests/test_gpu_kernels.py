@@ -353,6 +353,23 @@ def test_depths_beyond_the_short_keys(mode):
     r.close()
 
 
+@pytest.mark.parametrize("per", [1, 3, 40])
+def test_sub_batches_of_as_many_cameras_as_the_records_hold(small_floor, floor_views, per):
+    """Record slots for so many cameras' whole cuts, which the partition tables are sized
+    for too: the views come in sub-batches of at most that many, with the pixels of each alone."""
+    from paper_2603_15186_gb300 import Renderer
+    leaves = int((small_floor.child_count == 0).sum())
+    r = Renderer(cut_capacity=1 << 20, record_capacity=per * leaves, pair_capacity=1 << 26)
+    r.load_scene(small_floor)
+    cams = floor_views[:50]
+    images = [x.clone() for x in r.render(cams)]
+    assert r.stats()["sub_batches"] >= -(-50 // per)   # the pairs' estimate may split them further
+    r.set_mode("plain")
+    for k in range(0, 50, 7):
+        assert torch.equal(r.render([cams[k]])[0], images[k]), k
+    r.close()
+
+
 def test_views_that_reach_far_depths_and_others_share_a_graph():
     """Views along the axis of a Gaussian 30 km away (four passes over the depth) and across
     it (three would do), in turn: one capture each way at most, the pixels of the plain path."""
