@@ -184,16 +184,16 @@ def measured_peaks():
 
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum, mean
 # over the launches of one render of this workload at 32x32 tiles in 16x16
-# compositing blocks, batch 128; for "onesweep" over all 18 radix passes) from
+# compositing blocks, batch 128; for "onesweep" over all 15 radix passes) from
 # the one-pass ncu capture summarised in profiles/traffic_batch256_floor4m_f16.md.
 # Each figure is tied to the sources of the kernel it was taken on (sha256 of
 # the files, concatenated, first 16 hex digits) and reads null once they change.
 MEASURED_TRAFFIC = {
-    "onesweep": (1_257_100_000, ("k_sort.cu", "ngs_internal.cuh"), "4db60b1584962499"),
-    "composite": (712_500_000, ("k_composite.cu", "ngs_internal.cuh"), "76ceb844a89ff03c"),
-    "cut_preprocess": (3_596_900_000, ("k_preprocess.cu", "ngs_internal.cuh"), "6d567f9e49be4b20"),
-    "duplicate": (2_100_600_000, ("k_binning.cu", "ngs_internal.cuh"), "b3d4843c4c7845b0"),
-    "pair_offsets": (1_220_500_000, ("k_binning.cu", "ngs_internal.cuh"), "b3d4843c4c7845b0"),
+    "onesweep": (1_361_500_000, ("k_sort.cu", "ngs_internal.cuh"), "2676ccac13f9d01d"),
+    "composite": (711_700_000, ("k_composite.cu", "ngs_internal.cuh"), "649ac6f4780c4db6"),
+    "cut_preprocess": (3_238_000_000, ("k_preprocess.cu", "ngs_internal.cuh"), "0d19f7d849f3e6ed"),
+    "duplicate": (2_094_700_000, ("k_binning.cu", "ngs_internal.cuh"), "45512d2116a8f759"),
+    "pair_offsets": (1_225_800_000, ("k_binning.cu", "ngs_internal.cuh"), "45512d2116a8f759"),
 }
 
 
